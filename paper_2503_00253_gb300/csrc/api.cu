@@ -17,6 +17,35 @@ using namespace infoesrf;
 namespace infoesrf {
 static std::atomic<long long> g_launches{0};
 void note_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+
+AuxStream* aux_stream() {
+  constexpr int kMaxDev = 64;
+  static thread_local AuxStream aux[kMaxDev];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  AuxStream& a = aux[dev];
+  if (!a.s) {
+    cudaStream_t s = nullptr;
+    cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
+    bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
+    for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&e[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+      cudaGetLastError();
+      for (int i = 0; i < 3; ++i)
+        if (e[i]) cudaEventDestroy(e[i]);
+      if (s) cudaStreamDestroy(s);
+      return nullptr;
+    }
+    a.s = s;
+    a.mid = e[0];
+    a.jq = e[1];
+    a.jb = e[2];
+  }
+  return &a;
+}
 }  // namespace infoesrf
 
 namespace {
@@ -257,21 +286,21 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
     pr.Clo = cv.take<__nv_bfloat16>((size_t)pr.tile_cap * kTileM * kTileK * 2);
     pr.Wp = cv.take<float>((size_t)dp * N * 4);
     pr.rinvp = cv.take<float>((size_t)dp * 4);
-    pr.Pdir = cv.take<__nv_bfloat16>((size_t)J * dp * 2);
+    pr.Pdir = cv.take<__nv_bfloat16>((size_t)2 * J * dp * 2);
     pr.Yv = cv.take<float>((size_t)J * dp * 4);
     pr.Xv = cv.take<float>((size_t)J * dp * 4);
     pr.Rv = cv.take<float>((size_t)J * dp * 4);
     pr.pty = cv.take<float>((size_t)pr.nrt * J * 4);
-    pr.dots = cv.take<double>((size_t)nsub * J * tile_dot_values((int)kk) * 8);
-    pr.dsum = cv.take<double>((size_t)J * tile_dot_values((int)kk) * 8);
+    pr.dots = cv.take<float>((size_t)nsub * J * tile_dot_values((int)kk) * 4);
+    pr.phiT = cv.take<float>((size_t)2 * kk * dp * 4);
     pr.sysd = cv.take<double>((size_t)J * 8 * 8);
     pr.lcoef = cv.take<float>((size_t)J * 2 * kMaxK * 4);
     pr.sigmaf = cv.take<float>((size_t)J * 4);
     pr.active = cv.take<int32_t>((size_t)J * 4);
-    pr.unit_active = cv.take<int32_t>((size_t)((J + kTileUnit - 1) / kTileUnit) * 4);
-    pr.unit_list = cv.take<int32_t>((size_t)((J + kTileUnit - 1) / kTileUnit) * 4);
+    pr.alphaf = cv.take<float>((size_t)J * 4);
+    pr.betaf = cv.take<float>((size_t)J * 4);
     pr.nactive = cv.take<int32_t>(4 * 4);
-    pr.alist = cv.take<int32_t>((size_t)J * 4);
+    pr.alist = cv.take<int32_t>((size_t)3 * J * 4);
     // operand planes of the tensor-core state update (tile_state.cu)
     pr.st_NV = (int32_t)((N + 15) / 16 * 16);
     pr.st_W = cv.take<__nv_bfloat16>((size_t)3 * dp * kStK * 2);
@@ -413,44 +442,6 @@ int status_to_code(int32_t bits) {
   if (bits & kStatBreakdown) return INFO_ESRF_ERR_BREAKDOWN;
   if (bits & kStatNotConverged) return INFO_ESRF_NOT_CONVERGED;
   return INFO_ESRF_OK;
-}
-
-// Side stream and events, per host thread and device, for the work that
-// overlaps the main sequence: the quadrature and the state-obs band run while
-// the Ritz pairs are computed.  Created on first use and kept for the life of
-// the thread (like a library handle).
-struct AuxStream {
-  cudaStream_t s = nullptr;
-  cudaEvent_t mid = nullptr, jq = nullptr, jb = nullptr;
-};
-
-AuxStream* aux_stream() {
-  constexpr int kMaxDev = 64;
-  static thread_local AuxStream aux[kMaxDev];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  AuxStream& a = aux[dev];
-  if (!a.s) {
-    cudaStream_t s = nullptr;
-    cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
-    bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
-    for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&e[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) {
-      cudaGetLastError();
-      for (int i = 0; i < 3; ++i)
-        if (e[i]) cudaEventDestroy(e[i]);
-      if (s) cudaStreamDestroy(s);
-      return nullptr;
-    }
-    a.s = s;
-    a.mid = e[0];
-    a.jq = e[1];
-    a.jb = e[2];
-  }
-  return &a;
 }
 
 int run_batch(const info_esrf_problem* probs, int32_t count, const info_esrf_options* opt_in, void* ws,

@@ -51,16 +51,17 @@ struct TileMmArgs {
   const int32_t* colblk;        // [tiles] column block of each stored block
   const __nv_bfloat16* P;       // [J][d_pad] directions
   const float* sigma;           // [J] shifts (NULL: zero)
-  const int32_t* active;        // [ceil(J / 16)] nonzero: the unit of 16 systems has an unconverged one (or NULL: all)
+  const int32_t* count;         // device: the first *count rows of P are multiplied (NULL: all J)
+  const int32_t* list;          // shift of row i: sigma[list[i]] (NULL: sigma[i])
   float* Y;                     // [J][d_pad] sigma p + C p
   float* pty;                   // partial p^T y per row tile (or NULL): [nrt][J], or [J][nrt] if pty_by_system
   int32_t* status;              // status bits (kStatTimeout), or NULL
   int64_t d_pad;
   int32_t J, nrt, nchunks, pty_by_system;
-  int32_t units;                // number of nonzero flags in `active` (ignored when it is NULL)
-  int32_t* ulist;               // [ceil(J / 16)] scratch: the ordered list of those units
+  int32_t J_run;                // host bound of *count (ignored when count is NULL)
+  int32_t upc;                  // units of 16 rows of P per CTA (set by the launcher)
 };
-constexpr int kTileUnit = 16;   // systems per unit of the tile matvec (one 16-row TMA box of P)
+constexpr int kTileUnit = 16;   // systems per unit of the tile matvec
 int launch_tile_mm(TileMmArgs a, const void* chi, const void* clo, int64_t ntiles, cudaStream_t st);
 constexpr int kStK = 128;           // member slots of the tensor-core state update (N <= 128)
 constexpr int kTileDotRows = 512;   // rows per partial dot product of the BF16 PCG
@@ -103,9 +104,9 @@ int run_tile_pcg_capture(const ProblemDev& p, const ProblemDev* dp, const TileCa
 // u = S r for the listed learned systems, with partial sums of u^T u
 // (tile_learn.cu); stages of the BF16 PCG loop.
 void launch_tile_learn_u(const ProblemDev& p, const ProblemDev* dp, const int32_t* list, int64_t count, int nsub,
-                         cudaStream_t st);
+                         int it, cudaStream_t st);
 void launch_tile_capture_record(const ProblemDev& p, const ProblemDev* dp, const TileCapture& cap, int it,
-                                cudaStream_t st);
+                                const int32_t* list, int64_t count, cudaStream_t st);
 void launch_tile_capture_finish(const ProblemDev& p, const ProblemDev* dp, const TileCapture& cap, float* Z,
                                 float* feat, cudaStream_t st);
 
@@ -208,21 +209,22 @@ struct ProblemDev {
   float* Wp;                    // [d_pad][N] W in tile order (0 at padding)
   float* rinvp;                 // [d_pad] R^-1/2 in tile order (0 at padding)
   // BF16 PCG state: systems j = sid (mean first, then q * N + i), J = nsys
-  __nv_bfloat16* Pdir;          // [J][d_pad] search directions (bf16, as used)
-  float* Yv;                    // [J][d_pad] sigma p + C p
+  __nv_bfloat16* Pdir;          // [2][J][d_pad] search directions by position (bf16, as used), iterations in turn
+  __host__ __device__ __nv_bfloat16* Pcur(int it) const { return Pdir + (it & 1) * (int64_t)nsys * d_pad; }
+  float* Yv;                    // [J][d_pad] sigma p + C p by position
   float* Xv;                    // [J][d_pad] iterates
   float* Rv;                    // [J][d_pad] residuals
-  float* pty;                   // [J][nrt] p^T y per row tile
-  double* dots;                 // [J][2 kR + 1][nsub] partial r^T r, Phi^T r, (C Phi)^T r per row block
-  double* dsum;                 // [J][2 kR + 1] their sums
+  float* pty;                   // [J][nrt] p^T y per row tile, by position
+  float* dots;                  // [J][nsub][2 kR + 2] partial r^T r, Phi^T r, (C Phi)^T r, u^T u per row block, by position
+  float* phiT;                  // [2 kR][d_pad] Phi and C Phi transposed
   double* sysd;                 // [J][8] per-system scalars (see tile_pcg.cu)
-  float* lcoef;                 // [J][2 kR] LMP coefficients of the current direction update
+  float* lcoef;                 // [J][2 kMaxK] LMP coefficients c, -t of the current direction update, by position
+  float* alphaf;                // [J] alpha by position
+  float* betaf;                 // [J] beta by position
   float* sigmaf;                // [J] shift per system (FP32)
   int32_t* active;              // [J] 1 while the system runs
-  int32_t* unit_active;         // [ceil(J / 16)] 1 while a unit of 16 systems has a running system
-  int32_t* unit_list;           // [ceil(J / 16)] the tile matvec's ordered list of those units
-  int32_t* nactive;             // [2] running systems; copy of status[0] for the host
-  int32_t* alist;               // [J] the running systems (unordered), rebuilt every iteration
+  int32_t* nactive;             // [4] running systems (iterations in turn, three slots); copy of status[0]
+  int32_t* alist;               // [2][J] the running systems (unordered), iterations in turn; [J] their old positions
   // learned correction on the BF16 path, for observations on every point of a
   // periodic 2-D lattice (the stencil S over lattice offsets, see tile_learn.cu)
   int32_t* lat_info;            // [16] device: ok, Lx, Ly, x0, y0, sx, sy, retries, learned systems
@@ -301,6 +303,17 @@ void launch_obs_matvec(const ProblemDev& pr, const ProblemDev* dpr, int32_t nvec
                        const double* sigma, double* Y, cudaStream_t st);
 void launch_lmp_apply(const ProblemDev& pr, const ProblemDev* dpr, int32_t nvec, const double* Rv,
                       const double* sigma, double* Z, cudaStream_t st);
+
+// Side stream and events, per host thread and device, for the work that
+// overlaps the main sequence (the quadrature and the state-obs band under the
+// Ritz stage; the BF16 path's read of the running count).  Created on first
+// use and kept for the life of the thread (like a library handle); NULL when
+// that fails.
+struct AuxStream {
+  cudaStream_t s = nullptr;
+  cudaEvent_t mid = nullptr, jq = nullptr, jb = nullptr;
+};
+AuxStream* aux_stream();
 
 // Host-side count of kernel launches issued by this library.
 void note_launches(int n);

@@ -173,8 +173,9 @@ __global__ void k_lat_nbr(const ProblemDev* tab) {
 // row-block partial sums of u^T u (dot value 2 k + 1).  CTA = (block of kRows
 // rows, group of kSys systems), the block's stencil table staged once.
 __global__ void __launch_bounds__(kVecThreads) k_tpcg_learn_u(const ProblemDev* dpr, const int32_t* list,
-                                                             int64_t count) {
+                                                             int it) {
   const ProblemDev& pr = *dpr;
+  const int64_t count = list ? pr.nactive[it % 3] : pr.nsys;
   const int64_t sb = blockIdx.x, g0 = (int64_t)blockIdx.y * kSys;
   const int64_t J = pr.nsys, dp = pr.d_pad;
   const int k = pr.kR, NVD = tile_dot_values(k);
@@ -219,24 +220,31 @@ __global__ void __launch_bounds__(kVecThreads) k_tpcg_learn_u(const ProblemDev* 
   }
 #pragma unroll
   for (int o = kRowLanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (j >= 0 && r0 == 0) pr.dots[(j * NVD + 2 * k + 1) * (int64_t)gridDim.x + sb] = (double)acc;
+  if (j >= 0 && r0 == 0) pr.dots[((g0 + s) * gridDim.x + sb) * NVD + 2 * k + 1] = acc;
 }
 
 // Capture: the directions p (as the matvec used them, BF16) and images
 // y = sigma p + C p of the selected systems at iteration it, in lattice order;
-// zero for a system that no longer runs.
-__global__ void k_tcap_record(const ProblemDev* dpr, const int32_t* sel, int nsel, int it, int K, float* V,
-                              float* Y) {
+// zero for a system that no longer runs.  The directions and images are kept by
+// position in the list of running systems, which every CTA searches.
+__global__ void k_tcap_record(const ProblemDev* dpr, const int32_t* sel, int nsel, int it, int K,
+                              const int32_t* list, float* V, float* Y) {
   const ProblemDev& pr = *dpr;
   const int s = blockIdx.y;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nsel || i >= pr.d) return;
   const int64_t j = pr.mean_sys + sel[s];
+  __shared__ int pos;
+  if (threadIdx.x == 0) pos = -1;
+  __syncthreads();
+  for (int64_t e = threadIdx.x; e < pr.nactive[it % 3]; e += blockDim.x)
+    if (list[e] == j) pos = (int)e;   // at most once
+  __syncthreads();
+  if (i >= pr.d) return;
   const int64_t row = (int64_t)s * K + (it - 1);
   float v = 0.f, y = 0.f;
-  if (j < pr.nsys && pr.active[j]) {
-    const int64_t a = j * pr.d_pad + pr.lat_tpos[i];
-    v = __bfloat162float(pr.Pdir[a]);
+  if (pos >= 0) {
+    const int64_t a = pos * pr.d_pad + pr.lat_tpos[i];
+    v = __bfloat162float(pr.Pcur(it)[a]);
     y = pr.Yv[a];
   }
   V[row * pr.d + i] = v;
@@ -342,7 +350,7 @@ void launch_tile_lattice(const ProblemTable& tab, const ProblemDev* dtab, cudaSt
 }
 
 void launch_tile_learn_u(const ProblemDev& p, const ProblemDev* dp, const int32_t* list, int64_t count, int nsub,
-                         cudaStream_t st) {
+                         int it, cudaStream_t st) {
   if (count < 1) return;
   static thread_local int raised = -1;
   int dev = 0;
@@ -353,14 +361,15 @@ void launch_tile_learn_u(const ProblemDev& p, const ProblemDev* dp, const int32_
     raised = dev;
   }
   const dim3 grid((unsigned)nsub, (unsigned)((count + kSys - 1) / kSys));
-  k_tpcg_learn_u<<<grid, kVecThreads, smem, st>>>(dp, list, count);
+  k_tpcg_learn_u<<<grid, kVecThreads, smem, st>>>(dp, list, it);
   note_launches(1);
 }
 
 void launch_tile_capture_record(const ProblemDev& p, const ProblemDev* dp, const TileCapture& cap, int it,
-                                cudaStream_t st) {
+                                const int32_t* list, int64_t count, cudaStream_t st) {
+  (void)count;
   const dim3 grid((unsigned)((p.d + 255) / 256), (unsigned)cap.nsel);
-  k_tcap_record<<<grid, 256, 0, st>>>(dp, cap.sel, cap.nsel, it, cap.K, cap.V, cap.Y);
+  k_tcap_record<<<grid, 256, 0, st>>>(dp, cap.sel, cap.nsel, it, cap.K, list, cap.V, cap.Y);
   note_launches(1);
 }
 

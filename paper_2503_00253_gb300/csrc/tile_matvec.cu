@@ -11,15 +11,16 @@
 // stored as two BF16 planes hi = bf16(C), lo = bf16(C - hi), row-major
 // [tile][128][64].  The directions are BF16, system-major [J][d_pad].
 //
-// Kernel.  Systems are grouped in units of 16 (one 16-row TMA box of P); a
-// launch covers the units that hold an unconverged system, split evenly over
-// `nchunks` CTAs per row tile (at most BN / 16 units each), so that converged
-// systems cost no tensor-core work.  One CTA of 4 warps per (row tile, chunk):
-// warp 0 lane 0 streams the blocks of the row tile through an S-stage ring of
-// shared memory with 2-D TMA loads (128-byte swizzle): the hi and lo planes of
-// the C block (the A operand, 128 x 64, K-major) and, per run of consecutive
-// units, one slab of their directions (together the B operand, 16 u x 64,
-// K-major; one tensor map per box height 16 .. 256 rows).  Warp 1
+// Kernel.  The running systems' directions are consecutive rows of P (the PCG
+// keeps them by position), so a launch covers ceil(count / 16) units of 16
+// rows, split evenly over `nchunks` CTAs per row tile (at most BN / 16 units
+// each): converged systems cost no tensor-core work.  One CTA of 4 warps per
+// (row tile, chunk): warp 0 lane 0 streams the blocks of the row tile through
+// an S-stage ring of shared memory with 2-D TMA loads (128-byte swizzle): the
+// hi and lo planes of the C block (the A operand, 128 x 64, K-major) and one
+// slab of directions (the B operand, 16 u x 64, K-major).  The row tile's
+// column-block list is staged in shared memory first: read from global memory
+// inside the loop, its latency stood in front of every stage's loads.  Warp 1
 // lane 0 issues tcgen05.mma kind::f16 (BF16 x BF16, FP32 accumulate, N = 16 u)
 // into a 128 x 16 u FP32 accumulator in tensor memory: four K = 16 steps for
 // hi, four for lo, then a commit that frees the stage.  After the last block
@@ -47,51 +48,22 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-constexpr int kMaxUnits = 16;                        // units per CTA at most (256 systems)
+constexpr int kMaxList = 1024;                       // column blocks of a row tile staged in shared memory
 
 // At most BN systems (BN / 16 units) per CTA, S pipeline stages.
 template <int BN, int S>
 struct TileMmShape {
   static constexpr int kUnits = BN / kTileUnit;
   static constexpr int kStage = 2 * kABytes + BN * kTileK * 2;
-  static constexpr int kCtrl = 256;   // mbarriers, TMEM slot, flags, the CTA's units and loads
-  static_assert(kUnits <= kMaxUnits, "units per CTA");
-  static_assert(8 * (2 * S + 1) + 4 + 16 + 8 * kUnits <= kCtrl, "control block");
-  static constexpr size_t kSmem = 1024 + (size_t)S * kStage + kCtrl + 4 * BN * sizeof(float);
+  static constexpr int kCtrl = 128;   // mbarriers, TMEM slot, flags
+  static_assert(8 * (2 * S + 1) + 4 + 12 <= kCtrl, "control block");
+  static constexpr size_t kSmem = 1024 + (size_t)S * kStage + kCtrl + kMaxList * 4 + 4 * BN * sizeof(float);
 };
-
-// Tensor maps of P with boxes of 64 columns and 16 (i + 1) rows, i = 0 .. 15.
-struct PMaps {
-  CUtensorMap m[kMaxUnits];
-};
-
-// Ordered list of the units whose flag is set (one CTA of 1024 threads).
-__global__ void __launch_bounds__(1024) k_tile_units(const int32_t* flags, int nunits, int32_t* ulist) {
-  __shared__ int wsum[32];
-  __shared__ int base;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) base = 0;
-  __syncthreads();
-  for (int u0 = 0; u0 < nunits; u0 += 1024) {
-    const int u = u0 + (int)threadIdx.x;
-    const bool act = u < nunits && flags[u] != 0;
-    const unsigned m = __ballot_sync(0xffffffffu, act);
-    if (lane == 0) wsum[warp] = __popc(m);
-    __syncthreads();
-    int off = base;
-    for (int w = 0; w < warp; ++w) off += wsum[w];
-    if (act) ulist[off + __popc(m & ((1u << lane) - 1u))] = u;
-    __syncthreads();
-    if (threadIdx.x == 0)
-      for (int w = 0; w < 32; ++w) base += wsum[w];
-    __syncthreads();
-  }
-}
 
 template <int BN, int S>
 __global__ void __launch_bounds__(128, 1)
     k_tile_mm(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
-              const __grid_constant__ PMaps maps_p, const TileMmArgs args) {
+              const __grid_constant__ CUtensorMap map_p, const TileMmArgs args) {
   using Shape = TileMmShape<BN, S>;
   constexpr int kStage = Shape::kStage;
   extern __shared__ unsigned char smem_raw[];
@@ -102,38 +74,25 @@ __global__ void __launch_bounds__(128, 1)
   uint64_t* empty = full + S;
   uint64_t* accf = empty + S;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(accf + 1);
-  int* flags = reinterpret_cast<int*>(tslot + 1);   // [0] abort, [1] loads issued, [2] stages consumed, [3] runs
-  int* units = flags + 4;                            // the CTA's units, in order
-  int* runs = units + Shape::kUnits;                 // runs of consecutive units: first rank | length << 8
-  float* red = reinterpret_cast<float*>(ctrl + Shape::kCtrl);
+  int* flags = reinterpret_cast<int*>(tslot + 1);   // [0] abort, [1] loads issued, [2] stages consumed
+  int* cols = reinterpret_cast<int*>(ctrl + Shape::kCtrl);   // the row tile's column blocks (the first kMaxList)
+  float* red = reinterpret_cast<float*>(cols + kMaxList);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // an overflowed block pattern is not read (uniform across the grid)
   if (args.status && (*reinterpret_cast<volatile int32_t*>(args.status) & kStatTileOverflow)) return;
   const int chunk = (int)(blockIdx.x % (unsigned)args.nchunks);
   const int rt = (int)(blockIdx.x / (unsigned)args.nchunks);
-  // this CTA's units: ranks [chunk T / nchunks, (chunk + 1) T / nchunks) of the T listed units
-  // (at most kUnits: nchunks >= T / kUnits)
-  const int T = args.units;
-  const int lo = (int)((int64_t)chunk * T / args.nchunks);
-  const int nu = min((int)((int64_t)(chunk + 1) * T / args.nchunks) - lo, Shape::kUnits);
-  if (nu <= 0) return;   // uniform across the CTA, before any barrier or TMEM use
-  if (threadIdx.x < nu) units[threadIdx.x] = args.ulist ? args.ulist[lo + threadIdx.x] : lo + (int)threadIdx.x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int nr = 0;
-    for (int i = 0; i < nu;) {
-      int len = 1;
-      while (i + len < nu && units[i + len] == units[i] + len) ++len;
-      runs[nr++] = i | (len << 8);
-      i += len;
-    }
-    flags[3] = nr;
-  }
+  // this CTA's rows of P: [c0, c0 + ncol), ncol a multiple of 16
+  const int T = args.count ? *args.count : args.J;
+  const int c0 = chunk * args.upc * kTileUnit;
+  if (c0 >= T) return;   // uniform across the CTA, before any barrier or TMEM use
+  const int nu = min(args.upc, (T - c0 + kTileUnit - 1) / kTileUnit);
   const int ncol = nu * kTileUnit;
-  const uint32_t stage_bytes = 2 * kABytes + nu * kUnitBytes;
+  const uint32_t stage_bytes = 2 * kABytes + args.upc * kUnitBytes;
   const int t0 = args.rowptr[rt];
   const int nk = args.rowptr[rt + 1] - t0;
+  for (int e = threadIdx.x; e < min(nk, kMaxList); e += 128) cols[e] = args.colblk[t0 + e];
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -147,13 +106,13 @@ __global__ void __launch_bounds__(128, 1)
     fence_mbar_init();
     tma_prefetch_map(&map_hi);
     tma_prefetch_map(&map_lo);
+    tma_prefetch_map(&map_p);
   }
   if (warp == 2) tmem_alloc(tslot, BN);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  const int nruns = flags[3];
 
   if (warp == 0 && lane == 0) {
     // producer: C block planes and each unit's slab of the directions for the block's columns
@@ -167,14 +126,11 @@ __global__ void __launch_bounds__(128, 1)
       if (*reinterpret_cast<volatile int*>(&flags[0])) break;
       unsigned char* st = smem + s * kStage;
       const int tile = t0 + kb;
-      const int xcol = args.colblk[tile] * kTileK;
+      const int xcol = (kb < kMaxList ? cols[kb] : args.colblk[tile]) * kTileK;
       mbar_arrive_expect_tx(&full[s], stage_bytes);
       tma_load_2d(st, &map_hi, &full[s], 0, tile * kTileM);
       tma_load_2d(st + kABytes, &map_lo, &full[s], 0, tile * kTileM);
-      for (int r = 0; r < nruns; ++r) {
-        const int i = runs[r] & 255, len = runs[r] >> 8;
-        tma_load_2d(st + 2 * kABytes + i * kUnitBytes, &maps_p.m[len - 1], &full[s], xcol, units[i] * kTileUnit);
-      }
+      tma_load_2d(st + 2 * kABytes, &map_p, &full[s], xcol, c0);
     }
     flags[1] = kb;
   } else if (warp == 1 && lane == 0) {
@@ -213,14 +169,14 @@ __global__ void __launch_bounds__(128, 1)
     for (int i = 0; i < nu; ++i) {   // one unit = 16 accumulator columns
       float v[16];
       tmem_ld16(tbase + (uint32_t)(i * kTileUnit), v);
-      const int jb = units[i] * kTileUnit;
+      const int jb = c0 + i * kTileUnit;
 #pragma unroll
       for (int c = 0; c < kTileUnit; ++c) {
         const int j = jb + c;
         float dot = 0.f;
-        if (j < args.J) {
+        if (j < T) {
           const float p = __bfloat162float(args.P[(int64_t)j * args.d_pad + a]);
-          const float y = args.sigma ? fmaf(args.sigma[j], p, v[c]) : v[c];
+          const float y = args.sigma ? fmaf(args.sigma[args.list ? args.list[j] : j], p, v[c]) : v[c];
           args.Y[(int64_t)j * args.d_pad + a] = y;
           dot = p * y;
         }
@@ -231,8 +187,8 @@ __global__ void __launch_bounds__(128, 1)
     __syncthreads();
     if (args.pty)
       for (int t = threadIdx.x; t < ncol; t += blockDim.x) {
-        const int j = units[t / kTileUnit] * kTileUnit + t % kTileUnit;
-        if (j < args.J) {
+        const int j = c0 + t;
+        if (j < T) {
           const float v = (red[t] + red[BN + t]) + (red[2 * BN + t] + red[3 * BN + t]);
           if (args.pty_by_system) args.pty[(int64_t)j * args.nrt + rt] = v;
           else args.pty[(int64_t)rt * args.J + j] = v;
@@ -249,17 +205,15 @@ __global__ void __launch_bounds__(128, 1)
 }
 
 template <int BN, int S>
-int launch_tile_mm_t(TileMmArgs a, const void* chi, const void* clo, int64_t ntiles, cudaStream_t st) {
+int launch_tile_mm_t(TileMmArgs a, int units, const void* chi, const void* clo, int64_t ntiles, cudaStream_t st) {
   using Shape = TileMmShape<BN, S>;
-  a.nchunks = (a.units + Shape::kUnits - 1) / Shape::kUnits;
-  CUtensorMap mh, ml;
-  PMaps mp;
+  a.nchunks = (units + Shape::kUnits - 1) / Shape::kUnits;
+  a.upc = (units + a.nchunks - 1) / a.nchunks;
+  CUtensorMap mh, ml, mp;
   if (!encode_bf16(&mh, chi, kTileK, (uint64_t)ntiles * kTileM, kTileK, kTileM) ||
-      !encode_bf16(&ml, clo, kTileK, (uint64_t)ntiles * kTileM, kTileK, kTileM))
+      !encode_bf16(&ml, clo, kTileK, (uint64_t)ntiles * kTileM, kTileK, kTileM) ||
+      !encode_bf16(&mp, a.P, (uint64_t)a.d_pad, (uint64_t)a.J, (uint64_t)a.d_pad, (uint32_t)(kTileUnit * a.upc)))
     return INFO_ESRF_ERR_CUDA;
-  for (int i = 0; i < Shape::kUnits; ++i)
-    if (!encode_bf16(&mp.m[i], a.P, (uint64_t)a.d_pad, (uint64_t)a.J, (uint64_t)a.d_pad, (uint32_t)(kTileUnit * (i + 1))))
-      return INFO_ESRF_ERR_CUDA;
   static thread_local int raised_dev = -1;
   int dev = 0;
   cudaGetDevice(&dev);
@@ -278,24 +232,19 @@ int launch_tile_mm_t(TileMmArgs a, const void* chi, const void* clo, int64_t nti
 }  // namespace
 
 int launch_tile_mm(TileMmArgs a, const void* chi, const void* clo, int64_t ntiles, cudaStream_t st) {
-  const int32_t nunits = (a.J + kTileUnit - 1) / kTileUnit;
   if (a.nrt < 1 || a.J < 1 || a.d_pad % kTileM || (int64_t)a.nrt * kTileM != a.d_pad ||
-      ntiles * kTileM >= (int64_t(1) << 31) || (a.active && (!a.ulist || a.units < 0 || a.units > nunits)))
+      ntiles * kTileM >= (int64_t(1) << 31) || (a.count && (a.J_run < 0 || a.J_run > a.J)))
     return INFO_ESRF_ERR_INVALID_ARG;
-  if (a.active) {
-    if (a.units == 0) return INFO_ESRF_OK;
-    k_tile_units<<<1, 1024, 0, st>>>(a.active, nunits, a.ulist);
-    note_launches(1);
-  } else {
-    a.units = nunits;
-    a.ulist = nullptr;
-  }
-  // up to 8 units (128 systems): a 128-column accumulator and 4 stages; else
-  // up to 16 units per CTA, 3 stages.  (Two 256-column accumulators per CTA,
-  // so that a C block load serves 512 systems, leave room for two stages only
-  // and measured slower: 1225 against 1273 TFLOP/s on the tilemm workload.)
-  if (a.units <= 8) return launch_tile_mm_t<128, 4>(a, chi, clo, ntiles, st);
-  return launch_tile_mm_t<256, 3>(a, chi, clo, ntiles, st);
+  const int units = ((a.count ? a.J_run : a.J) + kTileUnit - 1) / kTileUnit;
+  if (units == 0) return INFO_ESRF_OK;
+  // up to 4 units (64 systems): 5 stages of 40 KB; up to 8 units: a 128-column
+  // accumulator and 4 stages; else up to 16 units per CTA, 3 stages.  (Two
+  // 256-column accumulators per CTA, so that a C block load serves 512
+  // systems, leave room for two stages only and measured slower: 1225 against
+  // 1273 TFLOP/s on the tilemm workload.)
+  if (units <= 4) return launch_tile_mm_t<64, 5>(a, units, chi, clo, ntiles, st);
+  if (units <= 8) return launch_tile_mm_t<128, 4>(a, units, chi, clo, ntiles, st);
+  return launch_tile_mm_t<256, 3>(a, units, chi, clo, ntiles, st);
 }
 
 }  // namespace infoesrf
@@ -314,7 +263,6 @@ extern "C" int info_esrf_bf16_tile_matvec(int32_t n_row_tiles, const int32_t* ro
   a.colblk = colblk_dev;
   a.P = reinterpret_cast<const __nv_bfloat16*>(P_dev);
   a.sigma = sigma_dev;
-  a.active = nullptr;
   a.Y = Y_dev;
   a.pty = pty_dev;
   a.status = status_dev;

@@ -25,26 +25,28 @@
 // r = b - C_q x up to the accuracy of the product (C kept as hi + lo BF16
 // planes, about 16 significant bits; products exact, FP32 accumulation).
 // Rounding p only perturbs the conjugacy of the directions, not the system
-// that is solved.  Converged systems stop updating; a 256-system chunk whose
-// systems have all stopped is skipped by the matvec.  The host reads the
-// count of running systems after every iteration (one stream synchronization
-// per iteration).
+// that is solved.  Converged systems leave the lists of running systems, and with them
+// the matvec.
 #include <cuda_bf16.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "info_esrf.h"
 #include "internal.h"
+#include "tile_mma.cuh"
 
 namespace infoesrf {
 
 namespace {
 
-constexpr int kSys = 16;           // systems per CTA in the vector kernels
-constexpr int kDotRows = kTileDotRows;   // rows per CTA (and per partial dot product)
-constexpr int kVecThreads = 256;   // 16 row lanes per system, four rows per lane and step
+constexpr int kDotRows = kTileDotRows;   // rows per CTA of the update (and per partial dot product)
+constexpr int kVecWarps = 4;       // row chunks per CTA of the direction kernel, one per warp
+constexpr int kVecThreads = 32 * kVecWarps;
+constexpr int kMaxGroup = 32;      // systems per CTA of the direction kernel at most
 // per-system FP64 scalars in sysd[j][8]
-enum { kRho = 0, kAlpha = 1, kBeta = 2, kBn2 = 3, kRr = 4, kFirst = 5 };
+enum { kRho = 0, kBn2 = 1, kRr = 2, kFirst = 3 };
 
 __device__ __forceinline__ double sys_sigma(const ProblemDev& pr, int64_t j) {
   if (j < pr.mean_sys) return 1.0;
@@ -52,7 +54,7 @@ __device__ __forceinline__ double sys_sigma(const ProblemDev& pr, int64_t j) {
   return pr.s[q] + 1.0;
 }
 
-// x = 0, r = b, p = 0 and the per-system state (mode 0), or (mode 1) the
+// x = 0, r = b and the per-system state (mode 0), or (mode 1) the
 // per-system state of the systems marked for a retry without the learned
 // term, whose vectors k_tpcg_retry_vectors has reset.
 __global__ void k_tpcg_init(const ProblemDev* dpr, int mode, int allow_learn) {
@@ -62,8 +64,6 @@ __global__ void k_tpcg_init(const ProblemDev* dpr, int mode, int allow_learn) {
   if (i < J && (mode == 0 || pr.learn_on[i] == 2)) {
     double* sd = pr.sysd + i * 8;
     sd[kRho] = 0.0;
-    sd[kAlpha] = 0.0;
-    sd[kBeta] = 0.0;
     sd[kBn2] = 0.0;
     sd[kRr] = 0.0;
     sd[kFirst] = 1.0;
@@ -81,6 +81,8 @@ __global__ void k_tpcg_init(const ProblemDev* dpr, int mode, int allow_learn) {
       pr.learn_on[i] = on;
     }
   }
+  if (i == 0)
+    for (int c = 0; c < 4; ++c) pr.nactive[c] = 0;
   if (mode != 0 || i >= J * pr.d_pad) return;
   const int64_t j = i / pr.d_pad, a = i % pr.d_pad;
   float b = 0.f;
@@ -91,10 +93,9 @@ __global__ void k_tpcg_init(const ProblemDev* dpr, int mode, int allow_learn) {
   }
   pr.Xv[i] = 0.f;
   pr.Rv[i] = b;
-  pr.Pdir[i] = __float2bfloat16_rn(0.f);
 }
 
-// x = 0, r = b, p = 0 for the systems marked for a retry (learn_on == 2).
+// x = 0, r = b for the systems marked for a retry (learn_on == 2).
 __global__ void k_tpcg_retry_vectors(const ProblemDev* dpr) {
   const ProblemDev& pr = *dpr;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -109,7 +110,6 @@ __global__ void k_tpcg_retry_vectors(const ProblemDev* dpr) {
   }
   pr.Xv[i] = 0.f;
   pr.Rv[i] = b;
-  pr.Pdir[i] = __float2bfloat16_rn(0.f);
 }
 
 // A learned system that failed: stop it and mark it for the retry.
@@ -119,466 +119,559 @@ __device__ __forceinline__ void mark_retry(const ProblemDev& pr, int64_t j) {
   atomicAdd(&pr.lat_info[7], 1);
 }
 
-// alpha_j = rho_j / p_j^T y_j (one warp per system: lanes over the row-tile
-// partials, a fixed shuffle tree); resets the unit flags and the running counts.
-__global__ void k_tpcg_alpha(const ProblemDev* dpr, int it, int nunits, int reset_only) {
-  const ProblemDev& pr = *dpr;
-  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gt < nunits) pr.unit_active[gt] = 0;
-  if (gt == 0) {
-    pr.nactive[0] = 0;
-    pr.nactive[2] = 0;
-  }
-  const int lane = threadIdx.x & 31;
-  const int64_t j = gt >> 5;
-  if (j >= pr.nsys || reset_only) return;
-  double* sd = pr.sysd + j * 8;
-  if (!pr.active[j]) {
-    if (lane == 0) sd[kAlpha] = 0.0;
-    return;
-  }
+// Systems are addressed in two ways.  X, R and the FP64 scalars belong to the
+// system j.  What one iteration hands to the next kernel (the directions P,
+// their images Y, the partial sums and the coefficients) is kept by position
+// in the iteration's list of running systems: list[pos] = j, and the next
+// list's src[pos] = position in the list before.  So the matvec runs over
+// consecutive rows of P (one TMA box per stage, no idle columns), and a kernel
+// finds what it needs one load after the list.  The lists are appended with
+// atomics: their order differs from run to run, which no result depends on
+// (every column of the product and every sum belongs to one system).
+//
+// Counts rotate over three slots: iteration `it` runs cnt[it % 3] systems,
+// appends the survivors to cnt[(it + 1) % 3] and clears cnt[(it + 2) % 3].
+__device__ __forceinline__ int64_t list_count(const ProblemDev& pr, const int32_t* list, int it) {
+  return list ? pr.nactive[it % 3] : pr.nsys;
+}
+
+// alpha = rho_j / p^T y of the system at position pos by one warp (lanes over
+// the row-tile partials, a fixed shuffle tree; every lane returns it).
+// record: this warp also keeps the iteration count and handles a breakdown
+// (p^T y <= 0 or not finite), which stops the system with alpha = 0.
+__device__ __forceinline__ double warp_alpha(const ProblemDev& pr, int64_t j, int64_t pos, int it, bool record,
+                                             int lane) {
   double pap = 0.0;
-  const float* src = pr.pty + j * pr.nrt;
+  const float* src = pr.pty + pos * pr.nrt;
+  const double rho = pr.sysd[j * 8 + kRho];
   for (int64_t t = lane; t < pr.nrt; t += 32) pap += (double)src[t];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) pap += __shfl_xor_sync(0xffffffffu, pap, o);
-  if (lane != 0) return;
-  if (pap > 0.0 && isfinite(pap)) {
-    sd[kAlpha] = sd[kRho] / pap;
-    pr.iters[j] = it;
-  } else {
-    sd[kAlpha] = 0.0;
-    if (pr.learn_on && pr.learn_on[j] == 1) {
+  const bool ok = pap > 0.0 && isfinite(pap);
+  const double al = ok ? rho / pap : 0.0;
+  if (record && lane == 0) {
+    if (ok) {
+      pr.iters[j] = it;
+    } else if (pr.learn_on && pr.learn_on[j] == 1) {
       mark_retry(pr, j);
     } else {
       pr.active[j] = 0;
       atomicOr(&pr.status[0], kStatBreakdown);
     }
   }
+  return al;
 }
 
-// Step 3 (update = 1) or the dot products of r alone (update = 0): CTA =
-// (block of kDotRows rows, group of kSys systems); Phi and C Phi of the rows
-// are staged in shared memory once and reused by every system of the group.
-// Systems: list[blockIdx.y * kSys + s] for positions below count (list = NULL:
-// systems blockIdx.y * kSys + s).
-__device__ __forceinline__ int64_t listed_system(const int32_t* list, int64_t count, int64_t pos, int64_t J) {
-  if (pos >= count) return J;   // past the end: no system
-  return list ? list[pos] : pos;
-}
-
-// Column stride (floats) of the staged [Phi | C Phi]: the block's rows plus
-// 4, so that a column is read along the rows with 16-byte loads (four
-// consecutive rows per thread, consecutive threads on consecutive rows: no
-// bank conflict) and the transposing writes of the staging spread over the
-// banks.
-constexpr int kPhCol = kDotRows + 4;
-__host__ __device__ __forceinline__ size_t phi_stage_bytes(int k) { return (size_t)2 * k * kPhCol * sizeof(float); }
-
-// Stages rows abase .. abase + kDotRows - 1 of [Phi | C Phi] transposed into
-// shared memory: pht[m * kPhCol + row] (m < k: Phi, k <= m < 2k: C Phi).
-// Phi and C Phi are contiguous [d][k] blocks, so each is read with 16-byte
-// loads that are all independent (a block of rows starts at a multiple of 4
-// floats); rows at or past d are zero.
-__device__ __forceinline__ void stage_phi(const ProblemDev& pr, int64_t abase, int k, float* pht) {
-  const int64_t a1 = abase + kDotRows < pr.d ? abase + kDotRows : pr.d;
-  const int nrows = a1 > abase ? (int)(a1 - abase) : 0;
-  const int tot = nrows * k, ntail = kDotRows - nrows;
-  for (int e = threadIdx.x; e < 2 * k * ntail; e += blockDim.x) {
-    const int m = e / ntail, row = nrows + e % ntail;
-    pht[m * kPhCol + row] = 0.f;
-  }
-#pragma unroll
-  for (int which = 0; which < 2; ++which) {
-    const float* src = reinterpret_cast<const float*>(which == 0 ? pr.Phi : pr.CPhi) + abase * k;
-    const float4* src4 = reinterpret_cast<const float4*>(src);
-    float* dst = pht + which * k * kPhCol;
-#pragma unroll 4
-    for (int q = threadIdx.x; q < tot / 4; q += blockDim.x) {
-      const float4 v = src4[q];
-      const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int e = 4 * q + i, row = e / k, m = e - row * k;
-        dst[m * kPhCol + row] = vv[i];
-      }
-    }
-    for (int e = (tot & ~3) + threadIdx.x; e < tot; e += blockDim.x) {
-      const int row = e / k, m = e - row * k;
-      dst[m * kPhCol + row] = src[e];
-    }
-  }
-}
-
-// CTA layout of steps 3 and 5: thread t serves system t / kRowLanes of the
-// group and rows t % kRowLanes, t % kRowLanes + kRowLanes, ... of the block,
-// so the kSys systems advance side by side and each thread runs a long loop
-// of independent rows.
-constexpr int kRowLanes = kVecThreads / kSys;   // 16
-
-// Step 3 (update = 1) or the dot products of r alone (update = 0).
-// NV32: 32-value chunks of the dot vector (r^T r, f, g): 1 for k <= 14 (the
-// float4 loop then covers 28 columns of [Phi | C Phi]), else 2 (k <= 24).
-template <int NV32>
-__global__ void __launch_bounds__(kVecThreads) k_tpcg_update(const ProblemDev* dpr, int update,
-                                                             const int32_t* list, int64_t count) {
+// Step 2 for problems of many row tiles: one warp per position.  With few row
+// tiles (kFusedAlpha) the update kernel forms alpha itself.
+__global__ void k_tpcg_alpha(const ProblemDev* dpr, int it, const int32_t* list) {
   const ProblemDev& pr = *dpr;
-  const int64_t sb = blockIdx.x;
-  const int64_t g0 = (int64_t)blockIdx.y * kSys;
-  const int k = pr.kR, NV = 2 * k + 1, NVD = tile_dot_values(k);
-  const int64_t J = pr.nsys, dp = pr.d_pad;
-  extern __shared__ float4 phs_dyn4[];   // [2 k][kPhCol / 4]
-  float* phs = reinterpret_cast<float*>(phs_dyn4);
-  __shared__ float part[kSys][2][32 * NV32];   // per system: the two half-lanes' reduce-scatter results
-  __shared__ int64_t sys[kSys];
+  const int64_t pos = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (pos >= list_count(pr, list, it)) return;
+  const double al = warp_alpha(pr, list[pos], pos, it, true, lane);
+  if (lane == 0) pr.alphaf[pos] = (float)al;
+}
+// Row tiles up to which the update kernel sums p^T y itself: every one of its
+// CTAs repeats the sum for its systems, nrt / 32 FP64 additions a lane.  At 32
+// row tiles a separate launch cost 4.3 us of a 110 us iteration; at 512 the
+// repeats would read 30 MB of partials per iteration.
+constexpr int kFusedAlpha = 128;
+
+// [Phi | C Phi] transposed, phiT[m][a] (m < k: Phi, then C Phi; zero at the
+// padding rows): the vector kernels read a column at four consecutive rows
+// with one coalesced 16-byte load.  Built once per analysis.
+__global__ void k_tpcg_phit(const ProblemDev* dpr) {
+  const ProblemDev& pr = *dpr;
+  const int k = pr.kR;
+  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= pr.d_pad) return;
+  const float* P = reinterpret_cast<const float*>(pr.Phi);
+  const float* A = reinterpret_cast<const float*>(pr.CPhi);
+  const bool in = a < pr.d;
+  for (int m = 0; m < k; ++m) {
+    pr.phiT[(int64_t)m * pr.d_pad + a] = in ? P[a * k + m] : 0.f;
+    pr.phiT[(int64_t)(k + m) * pr.d_pad + a] = in ? A[a * k + m] : 0.f;
+  }
+}
+
+__device__ __forceinline__ float4 bf16x4(uint2 w) {
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                     __uint_as_float(w.y & 0xffff0000u));
+}
+
+// Step 3 (update = 1 or 2: x += alpha p, r -= alpha y first; 2 forms alpha
+// here) and the partial dot products r^T r, Phi^T r, (C Phi)^T r over the
+// CTA's kDotRows rows, dots[j][block][NVD].
+//
+// Sixteen lanes serve the rows of a system, four consecutive rows per lane and
+// step; a thread carries SPT systems side by side, so one 16-byte read of a
+// staged column serves 4 SPT FMAs.  The columns come as 2 k bulk copies of the
+// transposed [Phi | C Phi] on one mbarrier, under which the first vectors
+// load; the next step's vectors load under the current step's FMAs.  HBM-bound
+// at large sizes (22 bytes a row and system), latency-bound at small ones.
+// (A transposing stage by all threads and one system per thread took 13.2 us a
+// launch at 4096 rows x 66 systems on average and 67 us at 65,536 x 145.)
+// The order of every sum is that of one thread per (system, lane) with rows
+// ascending, whatever SPT.
+constexpr int kRowLanes = 16;
+constexpr int kUpdThreads = 128;
+constexpr int kUpdSlots = kUpdThreads / kRowLanes;   // 8
+
+struct VecStep {
+  float4 r, y, x;
+  uint2 p;
+};
+
+template <int NV32, int SPT>
+__global__ void __launch_bounds__(kUpdThreads) k_tpcg_update(const ProblemDev* dpr, int update, const int32_t* list,
+                                                             int it) {
+  constexpr int kSys = kUpdSlots * SPT;
+  extern __shared__ float4 phs_dyn4[];   // [2 k][kDotRows / 4]
+  __shared__ alignas(8) uint64_t bar;
+  __shared__ int32_t sys[kSys];
   __shared__ float als[kSys];
+  const ProblemDev& pr = *dpr;
+  const int k = pr.kR, NVD = tile_dot_values(k);
+  const int64_t dp = pr.d_pad;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t count = list_count(pr, list, it);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) pr.nactive[(it + 2) % 3] = 0;
+  const int64_t g0 = (int64_t)blockIdx.y * kSys;
+  if (g0 >= count) return;
+  const int64_t abase = (int64_t)blockIdx.x * kDotRows;
+  const int nrow = (int)(dp - abase < kDotRows ? dp - abase : kDotRows);   // a multiple of 128
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    fence_mbar_init();
+    if (k > 0) mbar_arrive_expect_tx(&bar, (uint32_t)(2 * k * nrow * 4));
+    for (int m = 0; m < 2 * k; ++m)
+      bulk_load(phs_dyn4 + m * (kDotRows / 4), pr.phiT + (int64_t)m * dp + abase, (uint32_t)(nrow * 4), &bar);
+  }
   if (threadIdx.x < kSys) {
-    const int64_t j = listed_system(list, count, g0 + threadIdx.x, J);
-    const bool run = j < J && pr.active[j];
-    sys[threadIdx.x] = run ? j : -1;
-    als[threadIdx.x] = run ? (float)pr.sysd[j * 8 + kAlpha] : 0.f;
+    const int64_t pos = g0 + threadIdx.x;
+    const int64_t j = pos < count ? (list ? list[pos] : pos) : -1;
+    als[threadIdx.x] = j >= 0 && update == 1 ? pr.alphaf[pos] : 0.f;
+    sys[threadIdx.x] = j >= 0 && (list || pr.active[j]) ? (int32_t)j : -1;
   }
   __syncthreads();
-  bool any = false;
-  for (int s = 0; s < kSys; ++s) any |= sys[s] >= 0;
-  if (!any) return;
-  const int64_t abase = sb * kDotRows;
-  stage_phi(pr, abase, k, phs);
-  __syncthreads();
-  const int s = threadIdx.x / kRowLanes, r0 = threadIdx.x % kRowLanes;
-  const int64_t j = sys[s];
-  float acc[32 * NV32];
+  if (update == 2) {
+    for (int s = warp; s < kSys; s += kUpdThreads / 32) {
+      const int j = sys[s];
+      if (j < 0) continue;
+      const double al = warp_alpha(pr, j, g0 + s, it, blockIdx.x == 0, lane);
+      if (lane == 0) als[s] = (float)al;
+    }
+    __syncthreads();
+  }
+  const int slot = threadIdx.x / kRowLanes, r0 = threadIdx.x % kRowLanes;
+  int64_t base[SPT], pbase[SPT];   // first element of each of the thread's systems (X, R) and positions (Y, P)
+  float al[SPT];
 #pragma unroll
-  for (int v = 0; v < 32 * NV32; ++v) acc[v] = 0.f;
-  if (j >= 0) {
-    const float al = als[s];
-    // four consecutive rows per step: 16-byte loads of r, y, x and 8 bytes of p
-    // (d_pad and the row block are multiples of 4, so a group never straddles dp)
-    for (int r4 = 4 * r0; r4 < kDotRows; r4 += 4 * kRowLanes) {
-      const int64_t a = abase + r4;
-      if (a >= dp) break;
-      const int64_t e = j * dp + a;
-      float4 rv = *reinterpret_cast<const float4*>(pr.Rv + e);
+  for (int u = 0; u < SPT; ++u) {
+    const int s = slot * SPT + u;
+    base[u] = sys[s] < 0 ? -1 : (int64_t)sys[s] * dp + abase;
+    pbase[u] = (g0 + s) * dp + abase;
+    al[u] = als[s];
+  }
+  float acc[SPT][32 * NV32];
+#pragma unroll
+  for (int u = 0; u < SPT; ++u)
+#pragma unroll
+    for (int v = 0; v < 32 * NV32; ++v) acc[u][v] = 0.f;
+  VecStep cur[SPT], nxt[SPT];
+  auto load = [&](VecStep (&w)[SPT], int r4) {
+#pragma unroll
+    for (int u = 0; u < SPT; ++u) {
+      w[u].r = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (base[u] < 0 || r4 >= nrow) continue;
+      w[u].r = *reinterpret_cast<const float4*>(pr.Rv + base[u] + r4);
       if (update) {
-        const uint2 pw = *reinterpret_cast<const uint2*>(pr.Pdir + e);
-        const __nv_bfloat162* pp = reinterpret_cast<const __nv_bfloat162*>(&pw);
-        const float2 p01 = __bfloat1622float2(pp[0]), p23 = __bfloat1622float2(pp[1]);
-        float4 xv = *reinterpret_cast<const float4*>(pr.Xv + e);
-        const float4 yv = *reinterpret_cast<const float4*>(pr.Yv + e);
-        xv.x = fmaf(al, p01.x, xv.x);
-        xv.y = fmaf(al, p01.y, xv.y);
-        xv.z = fmaf(al, p23.x, xv.z);
-        xv.w = fmaf(al, p23.y, xv.w);
-        rv.x = fmaf(-al, yv.x, rv.x);
-        rv.y = fmaf(-al, yv.y, rv.y);
-        rv.z = fmaf(-al, yv.z, rv.z);
-        rv.w = fmaf(-al, yv.w, rv.w);
-        *reinterpret_cast<float4*>(pr.Xv + e) = xv;
-        *reinterpret_cast<float4*>(pr.Rv + e) = rv;
+        w[u].y = *reinterpret_cast<const float4*>(pr.Yv + pbase[u] + r4);
+        w[u].x = *reinterpret_cast<const float4*>(pr.Xv + base[u] + r4);
+        w[u].p = *reinterpret_cast<const uint2*>(pr.Pcur(it) + pbase[u] + r4);
       }
-      acc[0] = fmaf(rv.x, rv.x, acc[0]);
-      acc[0] = fmaf(rv.y, rv.y, acc[0]);
-      acc[0] = fmaf(rv.z, rv.z, acc[0]);
-      acc[0] = fmaf(rv.w, rv.w, acc[0]);
-      // column m of [Phi | C Phi] at the four rows: one 16-byte load
-      const float4* col4 = phs_dyn4 + r4 / 4;
+    }
+  };
+  load(cur, 4 * r0);
+  if (k > 0 && !mbar_wait(&bar, 0)) {
+    atomicOr(&pr.status[0], kStatTimeout);
+    return;
+  }
+#pragma unroll 1
+  for (int r4 = 4 * r0; r4 < nrow; r4 += 4 * kRowLanes) {
+    load(nxt, r4 + 4 * kRowLanes);
 #pragma unroll
-      for (int m = 0; m < 32 * NV32 - 1; ++m) {
-        if (m < 2 * k) {
-          const float4 f = col4[m * (kPhCol / 4)];
-          float t = acc[1 + m];
-          t = fmaf(f.x, rv.x, t);
-          t = fmaf(f.y, rv.y, t);
-          t = fmaf(f.z, rv.z, t);
-          acc[1 + m] = fmaf(f.w, rv.w, t);
+    for (int u = 0; u < SPT; ++u) {
+      if (update && base[u] >= 0) {
+        const float4 p = bf16x4(cur[u].p);
+        cur[u].x.x = fmaf(al[u], p.x, cur[u].x.x);
+        cur[u].x.y = fmaf(al[u], p.y, cur[u].x.y);
+        cur[u].x.z = fmaf(al[u], p.z, cur[u].x.z);
+        cur[u].x.w = fmaf(al[u], p.w, cur[u].x.w);
+        cur[u].r.x = fmaf(-al[u], cur[u].y.x, cur[u].r.x);
+        cur[u].r.y = fmaf(-al[u], cur[u].y.y, cur[u].r.y);
+        cur[u].r.z = fmaf(-al[u], cur[u].y.z, cur[u].r.z);
+        cur[u].r.w = fmaf(-al[u], cur[u].y.w, cur[u].r.w);
+        *reinterpret_cast<float4*>(pr.Xv + base[u] + r4) = cur[u].x;
+        *reinterpret_cast<float4*>(pr.Rv + base[u] + r4) = cur[u].r;
+      }
+      acc[u][0] = fmaf(cur[u].r.x, cur[u].r.x, acc[u][0]);
+      acc[u][0] = fmaf(cur[u].r.y, cur[u].r.y, acc[u][0]);
+      acc[u][0] = fmaf(cur[u].r.z, cur[u].r.z, acc[u][0]);
+      acc[u][0] = fmaf(cur[u].r.w, cur[u].r.w, acc[u][0]);
+    }
+    const float4* col4 = phs_dyn4 + r4 / 4;
+#pragma unroll
+    for (int m = 0; m < 32 * NV32 - 1; ++m) {
+      if (m < 2 * k) {
+        const float4 f = col4[m * (kDotRows / 4)];
+#pragma unroll
+        for (int u = 0; u < SPT; ++u) {
+          float t = acc[u][1 + m];
+          t = fmaf(f.x, cur[u].r.x, t);
+          t = fmaf(f.y, cur[u].r.y, t);
+          t = fmaf(f.z, cur[u].r.z, t);
+          acc[u][1 + m] = fmaf(f.w, cur[u].r.w, t);
         }
       }
     }
+#pragma unroll
+    for (int u = 0; u < SPT; ++u) cur[u] = nxt[u];
   }
   // reduce over the 16 row lanes of each system (a half-warp): a reduce-scatter
-  // with offsets 8, 4, 2, 1 leaves lane l of the half with values 2 l and 2 l + 1
-  // of each 32-value chunk (fixed order of additions)
-  const int hl = r0;   // lane within the half-warp
+  // with offsets 8, 4, 2, 1 leaves two values of each 32-value chunk per lane
+  const int nsub = gridDim.x;
+  const int vlane = 16 * ((r0 >> 3) & 1) + 8 * ((r0 >> 2) & 1) + 4 * ((r0 >> 1) & 1) + 2 * (r0 & 1);
 #pragma unroll
-  for (int c = 0; c < NV32; ++c) {
-    float* v = acc + 32 * c;
+  for (int u = 0; u < SPT; ++u) {
 #pragma unroll
-    for (int off = 8, width = 16; off >= 1; off >>= 1, width >>= 1) {
-      const bool up = (hl & off) != 0;
+    for (int c = 0; c < NV32; ++c) {
+      float* v = acc[u] + 32 * c;
 #pragma unroll
-      for (int i = 0; i < width; ++i) {
-        const float send = up ? v[i] : v[i + width];
-        const float keep = up ? v[i + width] : v[i];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+      for (int off = 8, width = 16; off >= 1; off >>= 1, width >>= 1) {
+        const bool up = (r0 & off) != 0;
+#pragma unroll
+        for (int i = 0; i < width; ++i) {
+          const float send = up ? v[i] : v[i + width];
+          const float keep = up ? v[i + width] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+      }
+      float* out = pr.dots + ((g0 + slot * SPT + u) * nsub + blockIdx.x) * NVD;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int vi = 32 * c + vlane + i;
+        if (base[u] >= 0 && vi <= 2 * k) out[vi] = v[i];
       }
     }
-    // after the rounds lane hl holds the sums of values 2 hl', 2 hl' + 1 with hl' the
-    // bit-reversal-free index: value index = 16 b3 + 8 b2 + 4 b1 + 2 b0 + i, i in {0, 1}
-    const int vbase = 32 * c + 16 * ((hl >> 3) & 1) + 8 * ((hl >> 2) & 1) + 4 * ((hl >> 1) & 1) + 2 * (hl & 1);
-    part[s][0][vbase] = v[0];
-    part[s][0][vbase + 1] = v[1];
+  }
+}
+
+// Step 4: one CTA per position.  The row-chunk partials are summed in FP64
+// (warp w takes the chunks w, w + 8, ..., lane v the value v; then the warps in
+// order: the same order every call), warp 0 then runs the k x k algebra of the
+// preconditioner with one lane per Ritz vector and the k^2 products spread over
+// the CTA.  (One thread per system ran k^2 dependent FP64 steps: 42 us a
+// launch, a quarter to a third of an iteration on small problems.)
+constexpr int kScalThreads = 256;
+__global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev* dpr, int nsub, int last,
+                                                               const int32_t* list, int32_t* next, int32_t* src,
+                                                               int it) {
+  const ProblemDev& pr = *dpr;
+  const int64_t pos = blockIdx.x;
+  const int64_t j = pos < list_count(pr, list, it) ? (list ? list[pos] : pos) : -1;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x == 0 && tid == 0) pr.nactive[3] = pr.status[0];   // timeouts and overflow are set by earlier kernels
+  if (j < 0 || !pr.active[j]) return;
+  const int k = pr.kR, NVD = tile_dot_values(k);
+  __shared__ double part[kScalThreads / 32][2 * kMaxK + 2];
+  __shared__ double v[2 * kMaxK + 2];   // r^T r, f = Phi^T r, g = (C Phi)^T r, u^T u
+  __shared__ double t_s[kMaxK], ti_s[kMaxK];
+  __shared__ double gt_s[kMaxK][kMaxK + 1];
+  __shared__ int go;
+  for (int e = lane; e < NVD; e += 32) {
+    double sum = 0.0;
+    const float* d = pr.dots + pos * nsub * NVD + e;
+    for (int cb = warp; cb < nsub; cb += kScalThreads / 32) sum += (double)d[(int64_t)cb * NVD];
+    part[warp][e] = sum;
+  }
+  const double sigma = sys_sigma(pr, j);
+  if (tid < k) ti_s[tid] = 1.0 / (pr.theta[tid] + sigma);
+  __syncthreads();
+  if (tid < NVD) {
+    double sum = 0.0;
+#pragma unroll
+    for (int w = 0; w < kScalThreads / 32; ++w) sum += part[w][tid];
+    v[tid] = sum;
+    if (tid >= 1 && tid <= k) t_s[tid - 1] = sum * ti_s[tid - 1];
   }
   __syncthreads();
-  const int64_t nsub = gridDim.x;
-  for (int e = threadIdx.x; e < kSys * NV; e += blockDim.x) {
-    const int ss = e / NV, v = e % NV;
-    if (sys[ss] >= 0) pr.dots[(sys[ss] * NVD + v) * nsub + sb] = (double)part[ss][0][v];
-  }
-}
-
-// Sums of the row-block partials: one CTA per listed system, one warp per
-// value (r^T r, f, g), lanes over the row blocks (contiguous), then a fixed
-// shuffle tree: the same order every call.
-__global__ void __launch_bounds__(256) k_tpcg_reduce(const ProblemDev* dpr, int nsub, const int32_t* list,
-                                                     int64_t count) {
-  const ProblemDev& pr = *dpr;
-  const int64_t j = listed_system(list, count, blockIdx.x, pr.nsys);
-  if (j >= pr.nsys || !pr.active[j]) return;
-  const int NV = tile_dot_values(pr.kR);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int v = warp; v < NV; v += blockDim.x >> 5) {
-    const double* src = pr.dots + (j * NV + v) * (int64_t)nsub;
-    double t = 0.0;
-    for (int sb = lane; sb < nsub; sb += 32) t += src[sb];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) pr.dsum[j * NV + v] = t;
-  }
-}
-
-// Step 4: one thread per system.
-__global__ void k_tpcg_scalars(const ProblemDev* dpr, int nsub, int last) {
-  const ProblemDev& pr = *dpr;
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j == 0) pr.nactive[1] = pr.status[0];   // timeouts and overflow are set by earlier kernels
-  if (j >= pr.nsys || !pr.active[j]) return;
-  const int k = pr.kR, NVD = tile_dot_values(k);
-  const double* v = pr.dsum + j * NVD;   // r^T r, f = Phi^T r, g = (C Phi)^T r, u^T u
-  (void)nsub;
   double* sd = pr.sysd + j * 8;
   const double rr = v[0];
   const bool first = sd[kFirst] != 0.0;
-  if (first) sd[kBn2] = rr;
-  sd[kRr] = rr;
-  const double bn2 = sd[kBn2];
-  pr.relres[j] = bn2 > 0.0 ? sqrt(rr / bn2) : 0.0;
   const bool lrn = pr.learn_on && pr.learn_on[j] == 1;
-  bool act = true;
-  if (pr.fixed_iters <= 0 && !(rr > pr.tol * pr.tol * bn2)) act = false;
-  if (!isfinite(rr) && lrn) {
-    mark_retry(pr, j);
-    return;
-  }
-  if (!(rr > 0.0) || !isfinite(rr)) act = false;
-  if (last && act) {
-    // iteration cap reached with the system still running
-    if (lrn && pr.fixed_iters <= 0) {
+  if (tid == 0) {
+    go = 0;
+    const double bn2 = first ? rr : sd[kBn2];
+    if (first) sd[kBn2] = rr;
+    sd[kRr] = rr;
+    pr.relres[j] = bn2 > 0.0 ? sqrt(rr / bn2) : 0.0;
+    bool act = true;
+    if (pr.fixed_iters <= 0 && !(rr > pr.tol * pr.tol * bn2)) act = false;
+    if (!isfinite(rr) && lrn) {
       mark_retry(pr, j);
-      return;
-    }
-    if (pr.fixed_iters <= 0) atomicOr(&pr.status[0], kStatNotConverged);
-    act = false;
-  }
-  if (!act) {
-    pr.active[j] = 0;
-    return;
-  }
-  const double sigma = sys_sigma(pr, j);
-  const double beta_lmp = sigma + pr.scal[1];
-  double rho = rr;
-  float* lc = pr.lcoef + j * 2 * kMaxK;
-  if (k > 0) {
-    double t[kMaxK], t2[kMaxK];
-    for (int m = 0; m < k; ++m) t[m] = v[1 + m] / (pr.theta[m] + sigma);
-    double gt = 0.0, fc = 0.0;
-    for (int m = 0; m < k; ++m) {
-      double acc = v[1 + k + m] + sigma * v[1 + m];
-      for (int i2 = 0; i2 < k; ++i2) {
-        const int ge = m * k + i2, gtr = i2 * k + m;
-        const double G = pr.gram[2 * k * k + ge] + sigma * (pr.gram[k * k + ge] + pr.gram[k * k + gtr]) +
-                         sigma * sigma * pr.gram[ge];
-        acc -= G * t[i2];
+    } else {
+      if (!(rr > 0.0) || !isfinite(rr)) act = false;
+      if (last && act) {
+        // iteration cap reached with the system still running
+        if (lrn && pr.fixed_iters <= 0) {
+          mark_retry(pr, j);
+        } else {
+          if (pr.fixed_iters <= 0) atomicOr(&pr.status[0], kStatNotConverged);
+          pr.active[j] = 0;
+        }
+        act = false;
+      } else if (!act) {
+        pr.active[j] = 0;
       }
-      t2[m] = acc;
+      go = act ? 1 : 0;
     }
-    for (int m = 0; m < k; ++m) {
-      const double c = (beta_lmp - sigma) * t[m] - t2[m] / (pr.theta[m] + sigma);
-      gt += v[1 + k + m] * t[m];
-      fc += v[1 + m] * c;
-      lc[m] = (float)t[m];
-      lc[kMaxK + m] = (float)c;
-    }
-    rho = rr - gt + fc;
   }
+  // G_q t, one product per thread: G_q = A^T A + sigma (A^T Phi + Phi^T A) + sigma^2 Phi^T Phi
+  for (int e = tid; e < k * k; e += kScalThreads) {
+    const int m = e / k, i2 = e - m * k;
+    const double G = pr.gram[2 * k * k + e] + sigma * (pr.gram[k * k + e] + pr.gram[k * k + i2 * k + m]) +
+                     sigma * sigma * pr.gram[e];
+    gt_s[m][i2] = G * t_s[i2];
+  }
+  __syncthreads();
+  if (!go || warp != 0) return;
+  float* lc = pr.lcoef + pos * 2 * kMaxK;
+  double gt = 0.0, fc = 0.0;
+  if (lane < k) {
+    const double f = v[1 + lane], g = v[1 + k + lane], t = t_s[lane];
+    double s0 = 0.0, s1 = 0.0;   // two chains
+    int i2 = 0;
+    for (; i2 + 1 < k; i2 += 2) {
+      s0 += gt_s[lane][i2];
+      s1 += gt_s[lane][i2 + 1];
+    }
+    if (i2 < k) s0 += gt_s[lane][i2];
+    const double t2 = (g + sigma * f) - (s0 + s1);
+    const double cc = pr.scal[1] * t - t2 * ti_s[lane];   // (beta_lmp - sigma) t - T^-1 t2
+    gt = g * t;
+    fc = f * cc;
+    lc[lane] = (float)cc;   // Phi columns take c, C Phi columns -t
+    lc[k + lane] = -(float)t;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    gt += __shfl_xor_sync(0xffffffffu, gt, o);
+    fc += __shfl_xor_sync(0xffffffffu, fc, o);
+  }
+  if (lane != 0) return;
+  double rho = k > 0 ? rr - gt + fc : rr;
   if (lrn) {   // rho = r^T (a P^-1 + S S) r = a r^T P^-1 r + u^T u
     const int64_t q = j < pr.mean_sys ? pr.Q : (j - pr.mean_sys) / pr.N;
     rho = (double)pr.learn_coef[q * kLearnOut] * rho + v[2 * k + 1];
   }
-  sd[kBeta] = first ? 0.0 : rho / sd[kRho];
+  pr.betaf[pos] = first ? 0.f : (float)(rho / sd[kRho]);
   sd[kRho] = rho;
   sd[kFirst] = 0.0;
-  if (atomicExch(&pr.unit_active[j / kTileUnit], 1) == 0) atomicAdd(&pr.nactive[2], 1);
-  pr.alist[atomicAdd(&pr.nactive[0], 1)] = (int32_t)j;
+  const int at = atomicAdd(&pr.nactive[(it + 1) % 3], 1);
+  next[at] = (int32_t)j;
+  src[at] = (int32_t)pos;
 }
 
-// Step 5: p = bf16(r - (C Phi) t + Phi c + beta p) for the running systems;
-// same CTA layout as step 3, the coefficients of all its systems staged once.
-// learned != 0: the dynamic buffer also holds the block's stencil table, and
-// a learned system takes z = a (r - (C Phi) t + Phi c) + S u.
-__global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev* dpr, int learned) {
+// Step 5: p = bf16(r - (C Phi) t + Phi c + beta p) for the running systems, from
+// the old position's direction to the new one's (two buffers).  A warp owns 64
+// rows (two consecutive ones per lane) and holds [Phi | C Phi] of its rows in
+// registers while it runs over the CTA's systems, four at a time so that their
+// loads overlap: 4 k FMAs a lane and system with the coefficients as
+// broadcasts, no staging.  (Staging a transposed copy of 512 rows per CTA in
+// shared memory, read per system: 14.4 us a launch at 4096 rows, 52 us at 65,536.)
+// K: columns of Phi held.
+// learned != 0: a learned system takes z = a (r - (C Phi) t + Phi c) + S u.
+template <int K, int RPL>
+__global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev* dpr, const int32_t* list,
+                                                                const int32_t* src, int group, int learned, int it) {
+  constexpr int kBatch = 4;
   const ProblemDev& pr = *dpr;
-  const int64_t sb = blockIdx.x;
-  const int64_t g0 = (int64_t)blockIdx.y * kSys;
   const int k = pr.kR;
-  const int64_t J = pr.nsys, dp = pr.d_pad;
-  const int64_t count = pr.nactive[0];   // the list the scalars kernel just built
-  extern __shared__ float4 phs_dyn4[];   // [2 k][kPhCol / 4]
-  float* phs = reinterpret_cast<float*>(phs_dyn4);
-  __shared__ float4 tc4[kSys][2 * kMaxK / 4];   // per system: c (Phi coefficients), then -t (C Phi)
-  __shared__ int64_t sys[kSys];
-  __shared__ float bes[kSys];
-  __shared__ int lon[kSys];
-  __shared__ float las[kSys], ltap[kSys][kLatBins];
-  if (threadIdx.x < kSys) {
-    const int64_t j = listed_system(pr.alist, count, g0 + threadIdx.x, J);
-    const bool run = j < J && pr.active[j];
-    sys[threadIdx.x] = run ? j : -1;
-    bes[threadIdx.x] = run ? (float)pr.sysd[j * 8 + kBeta] : 0.f;
-    const bool on = learned && run && pr.learn_on[j] == 1;
-    lon[threadIdx.x] = on ? 1 : 0;
-    las[threadIdx.x] = 1.f;
-    if (on) {
+  const int64_t dp = pr.d_pad;
+  const int64_t count = pr.nactive[(it + 1) % 3];   // the list the scalars kernel just built
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t g0 = (int64_t)blockIdx.y * group;
+  if (g0 >= count) return;
+  __shared__ float4 tc4[kMaxGroup][2 * K / 4];   // per system: c (Phi coefficients), then -t (C Phi)
+  __shared__ int32_t sys[kMaxGroup], from[kMaxGroup];
+  __shared__ float bes[kMaxGroup];
+  __shared__ float las[kMaxGroup], ltap[kMaxGroup][kLatBins];   // learned systems: a (0: not learned) and taps
+  if (threadIdx.x < kMaxGroup) {
+    const int64_t pos = g0 + threadIdx.x;
+    const bool on = (int)threadIdx.x < group && pos < count;
+    const int j = on ? list[pos] : -1, f = on ? src[pos] : 0;
+    sys[threadIdx.x] = j;
+    from[threadIdx.x] = f;
+    bes[threadIdx.x] = on ? pr.betaf[f] : 0.f;
+    float la = 0.f;
+    if (learned && on && pr.learn_on[j] == 1) {
       const int64_t q = j < pr.mean_sys ? pr.Q : (j - pr.mean_sys) / pr.N;
-      las[threadIdx.x] = pr.learn_coef[q * kLearnOut];
+      la = pr.learn_coef[q * kLearnOut];
       for (int b = 0; b < kLatBins; ++b) ltap[threadIdx.x][b] = pr.learn_coef[q * kLearnOut + 1 + b];
     }
+    las[threadIdx.x] = la;
   }
   __syncthreads();
-  bool any = false, anyl = false;
-  for (int s = 0; s < kSys; ++s) {
-    any |= sys[s] >= 0;
-    anyl |= lon[s] != 0;
-  }
-  if (!any) return;
-  const int64_t abase = sb * kDotRows;
-  stage_phi(pr, abase, k, phs);
-  int32_t* nbr_s = reinterpret_cast<int32_t*>(phs + 2 * k * kPhCol);   // [kDotRows][kLatPts]
-  if (anyl) {
-    const int64_t nrow = dp - abase < kDotRows ? dp - abase : kDotRows;
-    for (int64_t e = threadIdx.x; e < nrow * kLatPts; e += blockDim.x) nbr_s[e] = pr.lat_nbr[abase * kLatPts + e];
-  }
   float* tcf = reinterpret_cast<float*>(tc4);
-  for (int e = threadIdx.x; e < kSys * 2 * kMaxK; e += blockDim.x) {
-    const int s = e / (2 * kMaxK), m = e % (2 * kMaxK);
+  for (int e = threadIdx.x; e < group * 2 * K; e += kVecThreads) {
+    const int s = e / (2 * K), m = e % (2 * K);
     float v = 0.f;
     if (sys[s] >= 0) {
-      // aligned with the staged columns: Phi columns take c, C Phi columns take -t
-      if (m < k) v = pr.lcoef[sys[s] * 2 * kMaxK + kMaxK + m];
-      else if (m < 2 * k) v = -pr.lcoef[sys[s] * 2 * kMaxK + (m - k)];
+      const float* lc = pr.lcoef + (int64_t)from[s] * 2 * kMaxK;
+      if (m < K) v = m < k ? lc[m] : 0.f;
+      else v = m - K < k ? lc[k + m - K] : 0.f;
     }
     tcf[e] = v;
   }
+  const __nv_bfloat16* Pold = pr.Pcur(it);
+  __nv_bfloat16* Pnew = pr.Pcur(it + 1);
+  const int64_t chunk = (int64_t)blockIdx.x * kVecWarps + warp;
+  const bool mine = chunk < dp / (32 * RPL);
+  const int64_t a = chunk * 32 * RPL + lane * RPL;
+  float c[2 * K][RPL];   // loaded while the coefficients are on their way to shared memory
+#pragma unroll
+  for (int m = 0; m < 2 * K; ++m) {
+    const int mm = m < K ? m : k + (m - K);
+    const bool in = mine && (m < K ? m < k : m - K < k);
+#pragma unroll
+    for (int i = 0; i < RPL; ++i) c[m][i] = 0.f;
+    if (in) {
+      const float* src = pr.phiT + (int64_t)mm * dp + a;
+      if constexpr (RPL == 4) {
+        const float4 t = __ldg(reinterpret_cast<const float4*>(src));
+        c[m][0] = t.x; c[m][1] = t.y; c[m][2] = t.z; c[m][3] = t.w;
+      } else {
+        const float2 t = __ldg(reinterpret_cast<const float2*>(src));
+        c[m][0] = t.x; c[m][1] = t.y;
+      }
+    }
+  }
   __syncthreads();
-  const int s = threadIdx.x / kRowLanes, r0 = threadIdx.x % kRowLanes;
-  const int64_t j = sys[s];
-  if (j < 0) return;
-  const float be = bes[s];
-  const bool sl = lon[s] != 0;
-  const float la = las[s];
-  float w[kLatPts];
+  if (!mine) return;
+#pragma unroll 1
+  for (int s0 = 0; s0 < group; s0 += kBatch) {
+    float z[kBatch][RPL];
+    uint32_t pw[kBatch][RPL / 2];
 #pragma unroll
-  for (int n = 0; n < kLatPts; ++n) w[n] = sl ? ltap[s][lat_bin(n)] : 0.f;
-  const float* u = pr.learn_u + j * dp;
-  for (int r4 = 4 * r0; r4 < kDotRows; r4 += 4 * kRowLanes) {   // four rows per step
-    const int64_t a = abase + r4;
-    if (a >= dp) break;
-    const int64_t e = j * dp + a;
-    const float4 rv = *reinterpret_cast<const float4*>(pr.Rv + e);
-    const uint2 pw = *reinterpret_cast<const uint2*>(pr.Pdir + e);
-    const __nv_bfloat162* pp = reinterpret_cast<const __nv_bfloat162*>(&pw);
-    const float2 p01 = __bfloat1622float2(pp[0]), p23 = __bfloat1622float2(pp[1]);
-    float z[4] = {rv.x, rv.y, rv.z, rv.w};
-    const float pv[4] = {p01.x, p01.y, p23.x, p23.y};
-    // column m of [Phi | C Phi] at the four rows: one 16-byte load
-    const float4* col4 = phs_dyn4 + r4 / 4;
+    for (int b = 0; b < kBatch; ++b) {
+      const int j = sys[s0 + b];
+      if (j < 0) continue;
+      const int64_t e = (int64_t)j * dp + a;
+      if constexpr (RPL == 4) {
+        const float4 r = *reinterpret_cast<const float4*>(pr.Rv + e);
+        z[b][0] = r.x; z[b][1] = r.y; z[b][2] = r.z; z[b][3] = r.w;
+        const uint2 w = *reinterpret_cast<const uint2*>(Pold + from[s0 + b] * dp + a);
+        pw[b][0] = w.x;
+        pw[b][RPL / 2 - 1] = w.y;
+      } else {
+        const float2 r = *reinterpret_cast<const float2*>(pr.Rv + e);
+        z[b][0] = r.x; z[b][1] = r.y;
+        pw[b][0] = *reinterpret_cast<const uint32_t*>(Pold + from[s0 + b] * dp + a);
+      }
+    }
 #pragma unroll
-    for (int q = 0; q < 2 * kMaxK / 4; ++q) {
-      if (4 * q < 2 * k) {
+    for (int b = 0; b < kBatch; ++b) {
+      const int s = s0 + b, j = sys[s];
+      if (j < 0) continue;
+#pragma unroll
+      for (int q = 0; q < 2 * K / 4; ++q) {
         const float4 c4 = tc4[s][q];   // four coefficients (a broadcast load)
         const float cq[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (4 * q + i >= 2 * k) break;   // only 2 k columns are staged
-          const float4 f = col4[(4 * q + i) * (kPhCol / 4)];
-          z[0] = fmaf(f.x, cq[i], z[0]);
-          z[1] = fmaf(f.y, cq[i], z[1]);
-          z[2] = fmaf(f.z, cq[i], z[2]);
-          z[3] = fmaf(f.w, cq[i], z[3]);
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int i = 0; i < RPL; ++i) z[b][i] = fmaf(c[4 * q + u][i], cq[u], z[b][i]);
+      }
+      const float be = bes[s], la = las[s];
+      __nv_bfloat162 out[RPL / 2];
+#pragma unroll
+      for (int i = 0; i < RPL; ++i) {
+        if (la > 0.f) {   // z = a P^-1 r + S u
+          const int32_t* nb = pr.lat_nbr + (a + i) * kLatPts;
+          const float* u = pr.learn_u + (int64_t)j * dp;
+          float su = 0.f;
+#pragma unroll
+          for (int n = 0; n < kLatPts; ++n) su = fmaf(ltap[s][lat_bin(n)], __ldg(u + nb[n]), su);
+          z[b][i] = fmaf(la, z[b][i], su);
         }
+        const uint32_t w = pw[b][i / 2];
+        const float p = __uint_as_float((i & 1) ? (w & 0xffff0000u) : (w << 16));
+        // beta = 0 (a first direction): the old position holds nothing of this system
+        z[b][i] = a + i < pr.d ? (be != 0.f ? fmaf(be, p, z[b][i]) : z[b][i]) : 0.f;
       }
-    }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (sl) {   // z = a P^-1 r + S u
-        const int32_t* nb = nbr_s + (r4 + i) * kLatPts;
-        float su = 0.f;
-#pragma unroll
-        for (int n = 0; n < kLatPts; ++n) su = fmaf(w[n], __ldg(u + nb[n]), su);
-        z[i] = fmaf(la, z[i], su);
-      }
-      z[i] = (a + i < pr.d) ? fmaf(be, pv[i], z[i]) : 0.f;
+      for (int i = 0; i < RPL / 2; ++i) out[i] = __floats2bfloat162_rn(z[b][2 * i], z[b][2 * i + 1]);
+      __nv_bfloat16* dst = Pnew + (g0 + s) * dp + a;
+      if constexpr (RPL == 4) *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(out);
+      else *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(out);
     }
-    __nv_bfloat162 out[2] = {__floats2bfloat162_rn(z[0], z[1]), __floats2bfloat162_rn(z[2], z[3])};
-    *reinterpret_cast<uint2*>(pr.Pdir + e) = *reinterpret_cast<const uint2*>(out);
   }
+}
+
+// Systems per CTA of the direction kernel (a multiple of its batch of four):
+// enough that a CTA's load of [Phi | C Phi] (80 bytes a row) is small beside
+// its systems' vectors (8 bytes a row each), few enough that small problems
+// still give every SM about 12 warps.
+int dir_group(int64_t nchunk, int64_t count, int sms) {
+  const int64_t g = (nchunk * count + 12 * sms - 1) / (12 * (int64_t)sms);
+  return (int)std::min<int64_t>(std::max<int64_t>((g + 3) / 4 * 4, 4), kMaxGroup);
 }
 
 }  // namespace
 
 // Runs the PCG of one BF16 problem (host copy p, device copy dp) to
-// convergence or the iteration cap.  Synchronizes the stream once per
-// iteration to read the number of running systems.  cap != NULL: records the
-// Krylov samples of its systems at iterations 1..cap->K and stops after K
-// iterations, without the learned term.
+// convergence or the iteration cap.  The kernels take the number of running
+// systems from the device; the host needs it only to size the launches and to
+// stop, so it reads it one iteration late: iteration `it` is launched with the
+// count after iteration it - 2, while iteration it - 1 runs (the count never
+// grows), and the call that finds nothing running costs one iteration of
+// empty launches.  cap != NULL: records the Krylov samples of its systems at
+// iterations 1..cap->K and stops after K iterations, without the learned term.
 static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t st, double* mm_ms, int* mm_count,
                          const TileCapture* cap) {
   const int64_t J = p.nsys;
   if (J < 1) return 0;
-  cudaEvent_t ev[2] = {nullptr, nullptr};
-  if (mm_ms && (cudaEventCreate(&ev[0]) != cudaSuccess || cudaEventCreate(&ev[1]) != cudaSuccess)) {
-    cudaGetLastError();
-    if (ev[0]) cudaEventDestroy(ev[0]);
-    return INFO_ESRF_ERR_CUDA;
-  }
-  bool timed = false;   // an event pair of the previous iteration awaits reading
-  auto read_time = [&]() {
-    if (!timed) return;
-    float ms = 0.f;
-    if (cudaEventElapsedTime(&ms, ev[0], ev[1]) == cudaSuccess) {
-      *mm_ms += ms;
-      ++*mm_count;
-    }
-    timed = false;
-  };
+  AuxStream* aux = aux_stream();
+  if (!aux) return INFO_ESRF_ERR_CUDA;
+  const cudaEvent_t counted[2] = {aux->mid, aux->jq};   // the scalars of iterations in turn are done
+  cudaEvent_t ev[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // matvec begin and end, iterations in turn
   struct Destroy {
-    cudaEvent_t* e;
+    cudaEvent_t (*e)[2];
     ~Destroy() {
-      if (e[0]) cudaEventDestroy(e[0]);
-      if (e[1]) cudaEventDestroy(e[1]);
+      for (int i = 0; i < 4; ++i)
+        if (e[i / 2][i % 2]) cudaEventDestroy(e[i / 2][i % 2]);
     }
   } destroy{ev};
-  const int nunits = (int)((J + kTileUnit - 1) / kTileUnit);
+  for (int i = 0; mm_ms && i < 4; ++i)
+    if (cudaEventCreate(&ev[i / 2][i % 2]) != cudaSuccess) {
+      cudaGetLastError();
+      return INFO_ESRF_ERR_CUDA;
+    }
+  const bool wide = p.kR > 12;   // 24 columns of Phi in registers
   const int nsub = (int)((p.d_pad + kDotRows - 1) / kDotRows);
+  const int64_t dchunks = p.d_pad / 64;
   const dim3 gsys((unsigned)((J + 127) / 128));
   const dim3 gall((unsigned)((J * p.d_pad + 255) / 256));
-  const dim3 gvec((unsigned)nsub, (unsigned)((J + kSys - 1) / kSys));
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return INFO_ESRF_ERR_CUDA;
   TileMmArgs ta{};
   ta.rowptr = p.rowptr;
   ta.colblk = p.colblk;
-  ta.P = p.Pdir;
   ta.sigma = p.sigmaf;
-  ta.active = p.unit_active;
-  ta.ulist = p.unit_list;
   ta.Y = p.Yv;
   ta.pty = p.pty;
   ta.status = p.status;
@@ -590,68 +683,111 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
   if (cap) maxit = cap->K;
   // the learned term is possible when the problem has a model and its tables
   bool learned = !cap && p.learned_model && p.learn_on && p.lat_info;
-  const size_t vsm = phi_stage_bytes(p.kR);
-  size_t dsm = vsm;   // + the stencil table while learned systems run (set below)
-  const bool wide = 2 * p.kR > 28;   // k > 14: 64-value dot vectors (the 32-value loop covers 28 columns)
+  const bool fused_alpha = p.nrt <= kFusedAlpha;
+  const size_t usm = (size_t)2 * p.kR * kDotRows * sizeof(float);
   static thread_local int raised = -1;
-  int dev = 0;
-  cudaGetDevice(&dev);
   if (raised != dev) {
-    const int mx = (int)phi_stage_bytes(kMaxK);
-    const int mxd = mx + kDotRows * kLatPts * (int)sizeof(int32_t);
-    if (cudaFuncSetAttribute(k_tpcg_update<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) != cudaSuccess ||
-        cudaFuncSetAttribute(k_tpcg_update<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) != cudaSuccess ||
-        cudaFuncSetAttribute(k_tpcg_direction, cudaFuncAttributeMaxDynamicSharedMemorySize, mxd) != cudaSuccess)
+    const int mx = 2 * kMaxK * kDotRows * (int)sizeof(float);
+    if (cudaFuncSetAttribute(k_tpcg_update<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) != cudaSuccess ||
+        cudaFuncSetAttribute(k_tpcg_update<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) != cudaSuccess ||
+        cudaFuncSetAttribute(k_tpcg_update<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) != cudaSuccess)
       return INFO_ESRF_ERR_CUDA;
     raised = dev;
   }
-  int32_t host[3] = {0, 0, 0};   // running systems, status bits, active units
-  auto update = [&](dim3 grid, int upd, const int32_t* list, int64_t count) {
-    if (wide) k_tpcg_update<2><<<grid, kVecThreads, vsm, st>>>(dp, upd, list, count);
-    else k_tpcg_update<1><<<grid, kVecThreads, vsm, st>>>(dp, upd, list, count);
+  // The lists of running systems and of their positions before, in turn.
+  int32_t* lists[2] = {p.alist, p.alist + J};
+  int32_t* srcs = p.alist + 2 * J;
+  // mode 0: the dot products of r alone; 1, 2: the update (2 forms alpha in it)
+  auto update = [&](int mode, const int32_t* list, int64_t count, int it) {
+    // two systems per thread (half the reads of [Phi | C Phi]) once that still
+    // gives every SM two CTAs; 64 dot values (k > 15) leave registers for one
+    const int spt = p.kR <= 15 && nsub * count >= 32 * (int64_t)sms ? 2 : 1;
+    const dim3 grid((unsigned)nsub, (unsigned)((count + kUpdSlots * spt - 1) / (kUpdSlots * spt)));
+    if (p.kR > 15) k_tpcg_update<2, 1><<<grid, kUpdThreads, usm, st>>>(dp, mode, list, it);
+    else if (spt == 2) k_tpcg_update<1, 2><<<grid, kUpdThreads, usm, st>>>(dp, mode, list, it);
+    else k_tpcg_update<1, 1><<<grid, kUpdThreads, usm, st>>>(dp, mode, list, it);
   };
-  const dim3 galpha((unsigned)(((32 * J > nunits ? 32 * J : nunits) + 255) / 256));
-  // the first direction of every running system: r = b, z = M r, p = z
+  auto direction = [&](const int32_t* list, int64_t count, int it) {
+    const int group = dir_group(dchunks, count, sms);
+    const dim3 grid((unsigned)((dchunks + kVecWarps - 1) / kVecWarps), (unsigned)((count + group - 1) / group));
+    if (wide) k_tpcg_direction<24, 2><<<grid, kVecThreads, 0, st>>>(dp, list, srcs, group, learned ? 1 : 0, it);
+    else k_tpcg_direction<12, 2><<<grid, kVecThreads, 0, st>>>(dp, list, srcs, group, learned ? 1 : 0, it);
+  };
+  // iteration 0, the first direction of every running system: r = b, z = M r, p = z
   auto start = [&]() {
-    update(gvec, 0, nullptr, J);
-    if (learned) launch_tile_learn_u(p, dp, nullptr, J, nsub, st);
-    k_tpcg_reduce<<<(unsigned)J, 256, 0, st>>>(dp, nsub, nullptr, J);
-    k_tpcg_alpha<<<galpha, 256, 0, st>>>(dp, 0, nunits, 1);   // resets the unit flags and the counts
-    k_tpcg_scalars<<<gsys, 128, 0, st>>>(dp, nsub, maxit <= 0 ? 1 : 0);
-    k_tpcg_direction<<<gvec, kVecThreads, dsm, st>>>(dp, learned ? 1 : 0);
-    note_launches(5);
+    update(0, nullptr, J, 0);
+    if (learned) launch_tile_learn_u(p, dp, nullptr, J, nsub, 0, st);
+    k_tpcg_scalars<<<(unsigned)J, kScalThreads, 0, st>>>(dp, nsub, maxit <= 0 ? 1 : 0, nullptr, lists[1], srcs, 0);
+    cudaEventRecord(counted[0], st);
+    direction(lists[1], J, 0);
+    note_launches(3);
+  };
+  // counts[it + 1] (and the status word) after iteration it, read on the side
+  // stream so that the main stream keeps running
+  int32_t host[4] = {0, 0, 0, 0};
+  auto read_counts = [&](int it) -> int {
+    if (cudaStreamWaitEvent(aux->s, counted[it & 1], 0) != cudaSuccess ||
+        cudaMemcpyAsync(host, p.nactive, sizeof(host), cudaMemcpyDeviceToHost, aux->s) != cudaSuccess ||
+        cudaStreamSynchronize(aux->s) != cudaSuccess)
+      return INFO_ESRF_ERR_CUDA;
+    return 0;
   };
   auto iterate = [&]() -> int {
-    for (int it = 1; it <= maxit; ++it) {
-      // running systems (and the status word) after the previous iteration
-      if (cudaMemcpyAsync(host, p.nactive, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-          cudaStreamSynchronize(st) != cudaSuccess)
-        return INFO_ESRF_ERR_CUDA;
-      read_time();   // the previous launch has completed (stream synchronized)
-      if (host[0] == 0) break;
-      if (host[1] & (kStatTimeout | kStatTileOverflow)) break;
-      const int64_t nrun = host[0];
-      ta.units = host[2];
-      const dim3 glist((unsigned)nsub, (unsigned)((nrun + kSys - 1) / kSys));
-      if (mm_ms) cudaEventRecord(ev[0], st);
-      if (launch_tile_mm(ta, p.Chi, p.Clo, p.tile_cap, st) != 0) return INFO_ESRF_ERR_CUDA;
-      if (mm_ms) {
-        cudaEventRecord(ev[1], st);
-        timed = true;
+    int64_t bound = J;   // systems that iteration it may run
+    int timed = -1;      // the iteration whose matvec events await reading
+    auto read_time = [&]() -> int {
+      if (timed < 0) return 0;
+      float ms = 0.f;
+      if (cudaEventSynchronize(ev[timed & 1][1]) != cudaSuccess) return INFO_ESRF_ERR_CUDA;
+      if (cudaEventElapsedTime(&ms, ev[timed & 1][0], ev[timed & 1][1]) == cudaSuccess) {
+        *mm_ms += ms;
+        ++*mm_count;
       }
-      if (cap) launch_tile_capture_record(p, dp, *cap, it, st);
-      k_tpcg_alpha<<<galpha, 256, 0, st>>>(dp, it, nunits, 0);
-      update(glist, 1, p.alist, nrun);
-      if (learned) launch_tile_learn_u(p, dp, p.alist, nrun, nsub, st);
-      k_tpcg_reduce<<<(unsigned)nrun, 256, 0, st>>>(dp, nsub, p.alist, nrun);
-      k_tpcg_scalars<<<gsys, 128, 0, st>>>(dp, nsub, it == maxit ? 1 : 0);
-      k_tpcg_direction<<<glist, kVecThreads, dsm, st>>>(dp, learned ? 1 : 0);
-      note_launches(5);
+      timed = -1;
+      return 0;
+    };
+    for (int it = 1; it <= maxit; ++it) {
+      if (it >= 2) {
+        if (read_counts(it - 2) || (mm_ms && read_time())) return INFO_ESRF_ERR_CUDA;
+        if (host[3] & (kStatTimeout | kStatTileOverflow)) return 0;
+        bound = host[(it - 1) % 3];   // running in iteration it - 1
+        if (bound == 0) return 0;     // it ran nothing, and its matvec is not counted
+        if (mm_ms) timed = it - 1;
+      }
+      const int32_t* list = lists[it & 1];
+      int32_t* next = lists[(it + 1) & 1];
+      ta.P = p.Pcur(it);
+      ta.count = p.nactive + it % 3;
+      ta.list = list;
+      ta.J_run = (int32_t)bound;
+      if (mm_ms) cudaEventRecord(ev[it & 1][0], st);
+      if (launch_tile_mm(ta, p.Chi, p.Clo, p.tile_cap, st) != 0) return INFO_ESRF_ERR_CUDA;
+      if (mm_ms) cudaEventRecord(ev[it & 1][1], st);
+      if (cap) launch_tile_capture_record(p, dp, *cap, it, list, bound, st);
+      if (!fused_alpha) {
+        k_tpcg_alpha<<<(unsigned)((32 * bound + 255) / 256), 256, 0, st>>>(dp, it, list);
+        note_launches(1);
+      }
+      update(fused_alpha ? 2 : 1, list, bound, it);
+      if (learned) launch_tile_learn_u(p, dp, list, bound, nsub, it, st);
+      k_tpcg_scalars<<<(unsigned)bound, kScalThreads, 0, st>>>(dp, nsub, it == maxit ? 1 : 0, list, next, srcs, it);
+      cudaEventRecord(counted[it & 1], st);
+      direction(next, bound, it);
+      note_launches(3);
+    }
+    if (mm_ms && maxit >= 1) {   // the cap was reached: the last two matvecs, if they ran anything
+      if (read_time()) return INFO_ESRF_ERR_CUDA;
+      if (read_counts(maxit - 1)) return INFO_ESRF_ERR_CUDA;
+      if (host[maxit % 3] > 0) {
+        timed = maxit;
+        if (read_time()) return INFO_ESRF_ERR_CUDA;
+      }
     }
     return 0;
   };
   k_tpcg_init<<<gall, 256, 0, st>>>(dp, 0, learned ? 1 : 0);
-  note_launches(1);
+  k_tpcg_phit<<<(unsigned)((p.d_pad + 255) / 256), 256, 0, st>>>(dp);
+  note_launches(2);
   if (learned) {   // systems that use the term (none: the plain loop)
     int32_t nl = 0;
     if (cudaMemcpyAsync(&nl, p.lat_info + 8, sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -659,7 +795,6 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
       return INFO_ESRF_ERR_CUDA;
     learned = nl > 0;
   }
-  if (learned) dsm = vsm + (size_t)kDotRows * kLatPts * sizeof(int32_t);
   start();
   int rc = iterate();
   if (rc) return rc;
@@ -669,7 +804,6 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
     if (cudaMemcpyAsync(&retries, p.lat_info + 7, sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
       return INFO_ESRF_ERR_CUDA;
-    read_time();
     if (retries > 0) {
       k_tpcg_retry_vectors<<<gall, 256, 0, st>>>(dp);
       k_tpcg_init<<<gsys, 128, 0, st>>>(dp, 1, 0);
@@ -678,10 +812,6 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
       rc = iterate();
       if (rc) return rc;
     }
-  }
-  if (timed) {
-    if (cudaEventSynchronize(ev[1]) != cudaSuccess) return INFO_ESRF_ERR_CUDA;
-    read_time();
   }
   return cudaGetLastError() == cudaSuccess ? 0 : INFO_ESRF_ERR_CUDA;
 }

@@ -757,7 +757,6 @@ void launch_tile_ritz_matvec(const ProblemTable& tab, const ProblemDev* dtab, in
     a.colblk = p.colblk;
     a.P = p.Pdir;
     a.sigma = nullptr;
-    a.active = nullptr;
     a.Y = p.Yv;
     a.pty = nullptr;
     a.status = p.status;
