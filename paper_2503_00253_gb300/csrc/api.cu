@@ -238,8 +238,12 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
   pr.xo_val = cv.take<void>((size_t)pr.max_xo * n * esz);
   pr.xo_col = cv.take<int32_t>((size_t)pr.max_xo * n * 4);
   pr.xo_nnz = cv.take<int32_t>(n * 4);
-  pr.Om = cv.take<void>((size_t)d * l * esz);
-  pr.Yb = cv.take<void>((size_t)d * l * esz);
+  const size_t basis = align_up((size_t)d * l * esz);   // Om, then Yb
+  char* om = cv.take<char>(2 * basis);
+  pr.Om = om;
+  pr.Yb = om ? om + basis : nullptr;
+  const size_t phit = (size_t)2 * k * (o.precision == 2 ? pr.d_pad : d) * esz;
+  pr.phiT = phit <= 2 * basis ? om : cv.take<void>(phit);
   pr.Gm = cv.take<double>((size_t)l * l * 8);
   pr.Rm = cv.take<double>((size_t)l * l * 8);
   pr.ev = cv.take<double>((size_t)l * 8);
@@ -286,13 +290,12 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
     pr.Clo = cv.take<__nv_bfloat16>((size_t)pr.tile_cap * kTileM * kTileK * 2);
     pr.Wp = cv.take<float>((size_t)dp * N * 4);
     pr.rinvp = cv.take<float>((size_t)dp * 4);
-    pr.Pdir = cv.take<__nv_bfloat16>((size_t)2 * J * dp * 2);
+    pr.Pdir = cv.take<__nv_bfloat16>((size_t)J * dp * 2);
     pr.Yv = cv.take<float>((size_t)J * dp * 4);
     pr.Xv = cv.take<float>((size_t)J * dp * 4);
     pr.Rv = cv.take<float>((size_t)J * dp * 4);
     pr.pty = cv.take<float>((size_t)pr.nrt * J * 4);
     pr.dots = cv.take<float>((size_t)nsub * J * tile_dot_values((int)kk) * 4);
-    pr.phiT = cv.take<float>((size_t)2 * kk * dp * 4);
     pr.sysd = cv.take<double>((size_t)J * 8 * 8);
     pr.lcoef = cv.take<float>((size_t)J * 2 * kMaxK * 4);
     pr.sigmaf = cv.take<float>((size_t)J * 4);
@@ -304,6 +307,7 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
     // operand planes of the tensor-core state update (tile_state.cu)
     pr.st_NV = (int32_t)((N + 15) / 16 * 16);
     pr.st_W = cv.take<__nv_bfloat16>((size_t)3 * dp * kStK * 2);
+    pr.Pdir1 = J <= 3 * kStK ? pr.st_W : cv.take<__nv_bfloat16>((size_t)J * dp * 2);   // the finish fills st_W anew
     pr.st_V = cv.take<__nv_bfloat16>((size_t)2 * pr.st_NV * dp * 2);
     pr.st_vm = cv.take<float>((size_t)dp * 4);
     pr.st_xyz = cv.take<int4>((size_t)dp * 16);
@@ -318,9 +322,14 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
   }
 }
 
+// Workspace up to which info_esrf_analysis_noalloc serves a call.  The optional
+// quads of C are left out of a reported size that they alone would push past
+// it, and out of any workspace that they don't fit.
+constexpr size_t kNoallocBytes = size_t(32) << 20;
+
 // Builds the host table for a batch; with ws == nullptr only sizes it.
 int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_options& o, void* ws,
-                ProblemTable& tab, size_t* bytes_out, ProblemDev** dtab_out, int32_t** counter_out,
+                size_t ws_bytes, ProblemTable& tab, size_t* bytes_out, ProblemDev** dtab_out, int32_t** counter_out,
                 void** scratch_out, size_t* scratch_bytes_out, int num_sms) {
   if (count < 1) return INFO_ESRF_ERR_INVALID_ARG;
   if (count > kMaxProblems) return INFO_ESRF_ERR_UNSUPPORTED;
@@ -424,6 +433,25 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
     if (mscg_plan(tab, num_sms, o.cluster_size, &tab.ms) != 0) return INFO_ESRF_ERR_UNSUPPORTED;
     tab.ms_scratch = tab.ms.scratch_bytes ? cv.take<void>(tab.ms.scratch_bytes) : nullptr;
   }
+  // the quads of C, last
+  const size_t base = cv.off;
+  size_t quads = 0;
+  int64_t qcap[kMaxProblems];
+  for (int i = 0; i < count; ++i) {
+    const int64_t nb = (tab.p[i].d + 3) / 4;
+    qcap[i] = pcg_quad_cap(tab.p[i], count, o.solver, o.cluster_size);
+    if (qcap[i]) quads += align_up(qcap[i] * nb * 16) + align_up(qcap[i] * nb * 4) + align_up(nb * 4);
+  }
+  if (ws ? base + quads <= ws_bytes : (base > kNoallocBytes || base + quads <= kNoallocBytes))
+    for (int i = 0; i < count; ++i) {
+      ProblemDev& pr = tab.p[i];
+      const int64_t nb = (pr.d + 3) / 4;
+      if (!qcap[i]) continue;
+      pr.qcap = qcap[i];
+      pr.qval = cv.take<float>(pr.qcap * nb * 16);
+      pr.qcol = cv.take<int32_t>(pr.qcap * nb * 4);
+      pr.qn = cv.take<int32_t>(nb * 4);
+    }
   *bytes_out = cv.off;
   if (dtab_out) *dtab_out = dtab;
   if (counter_out) *counter_out = counter;
@@ -457,7 +485,7 @@ int run_batch(const info_esrf_problem* probs, int32_t count, const info_esrf_opt
   int32_t* counter = nullptr;
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
-  rc = build_table(probs, count, o, ws, tab, &need, &dtab, &counter, &scratch, &scratch_bytes, sms);
+  rc = build_table(probs, count, o, ws, ws_bytes, tab, &need, &dtab, &counter, &scratch, &scratch_bytes, sms);
   if (rc) return rc;
   if (need > ws_bytes) return INFO_ESRF_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
@@ -543,12 +571,14 @@ int run_batch(const info_esrf_problem* probs, int32_t count, const info_esrf_opt
       cudaStreamWaitEvent(aux->s, aux->mid, 0);
       launch_quadrature(tab, dtab, aux->s);
       launch_learn_coef(tab, dtab, aux->s);
+      launch_pcg_quads(tab, dtab, aux->s);
       cudaEventRecord(aux->jq, aux->s);
       launch_band_state(tab, dtab, aux->s);
       cudaEventRecord(aux->jb, aux->s);
     } else {
       launch_quadrature(tab, dtab, st);
       launch_learn_coef(tab, dtab, st);
+      launch_pcg_quads(tab, dtab, st);
       launch_band_state(tab, dtab, st);
     }
     mark(1);
@@ -721,7 +751,7 @@ size_t info_esrf_batched_workspace_size(const info_esrf_problem* probs, int32_t 
   if (check_options(opt, &o)) return 0;
   static thread_local ProblemTable tab;
   size_t need = 0;
-  if (build_table(probs, count, o, nullptr, tab, &need, nullptr, nullptr, nullptr, nullptr, num_sms_current()))
+  if (build_table(probs, count, o, nullptr, 0, tab, &need, nullptr, nullptr, nullptr, nullptr, num_sms_current()))
     return 0;
   return need;
 }
@@ -870,7 +900,7 @@ static int prepare_one(const info_esrf_grid* grid, int64_t N, const double* X_de
   static thread_local ProblemTable tab;
   size_t need = 0;
   ProblemDev* dtab = nullptr;
-  rc = build_table(&P, 1, o, ws, tab, &need, &dtab, nullptr, nullptr, nullptr, num_sms_current());
+  rc = build_table(&P, 1, o, ws, ws_bytes, tab, &need, &dtab, nullptr, nullptr, nullptr, num_sms_current());
   if (rc) return rc;
   if (need > ws_bytes) return INFO_ESRF_ERR_WORKSPACE;
   *dpr = dtab;
@@ -1070,7 +1100,7 @@ int info_esrf_prepared_band_capacity(const info_esrf_grid* grid, int64_t N, int6
   info_esrf_problem P = one_problem(grid, N, &dx, d, &di, nullptr, &dx, Q, 1.0, nullptr, &dx);
   static thread_local ProblemTable tab;
   size_t need = 0;
-  rc = build_table(&P, 1, o, nullptr, tab, &need, nullptr, nullptr, nullptr, nullptr, 160);
+  rc = build_table(&P, 1, o, nullptr, 0, tab, &need, nullptr, nullptr, nullptr, nullptr, 160);
   if (rc) return rc;
   if (max_oo) *max_oo = tab.p[0].max_oo;
   if (max_xo) *max_xo = tab.p[0].max_xo;

@@ -150,7 +150,7 @@ struct ProblemDev {
   double* rinv;         // [d] R^-1/2
   double* bmean;        // [d] R^-1/2 (y - H mu)
   double* scal;         // [8] 0 gershgorin bound, 1 min diag C, 2 ell, 3 nonzeros of C (BF16 path), 4 sum of diag C
-  int32_t* status;      // [4]
+  int32_t* status;      // [4] 0 status bits, 1 solver path, 2 nonzero: a quad of C beyond its capacity
   double* s;            // [Q] quadrature nodes
   double* p;            // [Q] quadrature weights
   void* oo_val;         // [max_oo][d] T: C(a, b) (ELL, transposed)
@@ -168,7 +168,14 @@ struct ProblemDev {
   void* Phi;            // [d][kR] T Ritz vectors
   void* CPhi;           // [d][kR] T C Phi
   double* theta;        // [kR] Ritz values of C
+  void* phiT;           // [2 kR][d] T Phi and C Phi transposed (BF16 path: rows of d_pad), in the memory of
+                        // Om and Yb where it fits: made after the eigensolver is done with them
   double* gram;         // [3][kR][kR]: Phi^T Phi, A^T Phi, A^T A with A = C Phi
+  // C by quads of rows for the general kernel's FP32 matvec, or NULL (see k_pcg_quads)
+  float* qval;                  // [qcap][ceil(d / 4)][4]
+  int32_t* qcol;                // [qcap][ceil(d / 4)]
+  int32_t* qn;                  // [ceil(d / 4)]
+  int64_t qcap;
   // learned correction a_q P_q^-1 + S_q^T S_q (optional)
   const float* learned_model;   // network parameters, NULL: none
   double learned_max_shift;     // > 0: learned term only for sigma <= this
@@ -209,14 +216,14 @@ struct ProblemDev {
   float* Wp;                    // [d_pad][N] W in tile order (0 at padding)
   float* rinvp;                 // [d_pad] R^-1/2 in tile order (0 at padding)
   // BF16 PCG state: systems j = sid (mean first, then q * N + i), J = nsys
-  __nv_bfloat16* Pdir;          // [2][J][d_pad] search directions by position (bf16, as used), iterations in turn
-  __host__ __device__ __nv_bfloat16* Pcur(int it) const { return Pdir + (it & 1) * (int64_t)nsys * d_pad; }
+  __nv_bfloat16* Pdir;          // [J][d_pad] search directions by position (bf16, as used), even iterations
+  __nv_bfloat16* Pdir1;         // [J][d_pad] of odd iterations; in the memory of st_W where it fits
+  __host__ __device__ __nv_bfloat16* Pcur(int it) const { return (it & 1) ? Pdir1 : Pdir; }
   float* Yv;                    // [J][d_pad] sigma p + C p by position
   float* Xv;                    // [J][d_pad] iterates
   float* Rv;                    // [J][d_pad] residuals
   float* pty;                   // [J][nrt] p^T y per row tile, by position
   float* dots;                  // [J][nsub][2 kR + 2] partial r^T r, Phi^T r, (C Phi)^T r, u^T u per row block, by position
-  float* phiT;                  // [2 kR][d_pad] Phi and C Phi transposed
   double* sysd;                 // [J][8] per-system scalars (see tile_pcg.cu)
   float* lcoef;                 // [J][2 kMaxK] LMP coefficients c, -t of the current direction update, by position
   float* alphaf;                // [J] alpha by position
@@ -340,6 +347,9 @@ int launch_mscg(const ProblemTable& tab, const ProblemDev* dtab, const MsPlan& p
 // its fall-back flag.
 constexpr int kCounterInts = 256;
 static_assert(1 + 2 * kMaxProblems <= kCounterInts, "PCG counter area");
+
+int64_t pcg_quad_cap(const ProblemDev& p, int count, int32_t solver, int32_t cluster_size);
+void launch_pcg_quads(const ProblemTable& tab, const ProblemDev* dtab, cudaStream_t st);
 
 // PCG vector scratch per CTA when vectors do not fit in shared memory.
 size_t pcg_scratch_bytes(const ProblemTable& tab, int num_sms);

@@ -8,8 +8,8 @@
 // All systems share the band of C, formed once per analysis, so the matvec
 // is a banded sparse-times-dense product over a group of JT systems that
 // share one shift.  Each CTA owns one group at a time: its PCG vectors sit
-// in shared memory (or in a private global slice when d is large), so a
-// group iterates to convergence without any grid-wide synchronization.
+// in shared memory as far as they fit (in a private global slice otherwise),
+// so a group iterates to convergence without any grid-wide synchronization.
 // Groups come from an atomic queue, so CTAs that finish early take more.
 //
 // Preconditioner: the limited-memory preconditioner of App. E,
@@ -17,64 +17,73 @@
 // applied with f = Phi^T r, g = A^T r (A = C Phi) and the k x k matrix
 // G_q = (C_q Phi)^T (C_q Phi):  t = T^-1 f,  t2 = g + sigma f - G_q t,
 // c = (beta - sigma) t - T^-1 t2,  z = r - A t + Phi c,  r^T z = r^T r - g.t + f.c.
-// So f, g and r^T r come out of the same block reduction as the residual
-// norm, and one PCG iteration needs two block reductions.
+// So f, g and r^T r come out of one pass over the residual.
 //
-// Scalars (rho, alpha, beta, norms, the k x k preconditioner algebra) are FP64
-// and handled by one thread per system; dot products of FP32 vectors are
-// accumulated as float-float pairs.
+// Scalars (rho, alpha, beta, norms, the k x k preconditioner algebra) are FP64,
+// one warp per system; dot products of FP32 vectors are accumulated as
+// float-float pairs.
 #include <math.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "internal.h"
 
 namespace infoesrf {
 
-template <typename T, int JT>
-struct Row {
-  T v[JT];
+// Layout of a group's vectors: [row][JT], a row's JT systems side by side.  A
+// work item is VL consecutive systems of a row (16 bytes of FP32, one FP64
+// value); item i = row G + g with G = JT / VL, so consecutive items are
+// consecutive in memory and a thread that strides by a multiple of G always
+// serves the same systems g VL .. g VL + VL - 1.
+//
+// FP64: one value per item, because the FP64 pipe (about two lanes per clock
+// and SM) is the bound and only needs every warp to carry some of the work.
+// FP32: four, so that an entry of C serves four systems per 16-byte read of p.
+constexpr int kPcgThreads = 512;
+constexpr int kPcgWarps = kPcgThreads / 32;
+template <typename T> struct PcgVec;
+template <> struct PcgVec<float> { static constexpr int VL = 4, JT = 8; };
+template <> struct PcgVec<double> { static constexpr int VL = 1, JT = 2; };
+
+template <typename T>
+struct Item {
+  T v[PcgVec<T>::VL];
 };
-
-template <typename T, int JT>
-__device__ __forceinline__ Row<T, JT> ld_row(const T* base, int64_t a) {
-  static_assert((sizeof(T) * JT) % 16 == 0, "row must be a multiple of 16 bytes");
-  Row<T, JT> r;
-  const uint4* src = reinterpret_cast<const uint4*>(base + a * JT);
-  uint4* dst = reinterpret_cast<uint4*>(r.v);
-#pragma unroll
-  for (int i = 0; i < (int)(sizeof(T) * JT / 16); ++i) dst[i] = src[i];
-  return r;
+__device__ __forceinline__ Item<float> ld_item(const float* p) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  return Item<float>{{t.x, t.y, t.z, t.w}};
 }
-
-template <typename T, int JT>
-__device__ __forceinline__ void st_row(T* base, int64_t a, const Row<T, JT>& r) {
-  uint4* dst = reinterpret_cast<uint4*>(base + a * JT);
-  const uint4* src = reinterpret_cast<const uint4*>(r.v);
-#pragma unroll
-  for (int i = 0; i < (int)(sizeof(T) * JT / 16); ++i) dst[i] = src[i];
+__device__ __forceinline__ Item<double> ld_item(const double* p) { return Item<double>{{*p}}; }
+__device__ __forceinline__ void st_item(float* p, const Item<float>& a) {
+  *reinterpret_cast<float4*>(p) = make_float4(a.v[0], a.v[1], a.v[2], a.v[3]);
 }
+__device__ __forceinline__ void st_item(double* p, const Item<double>& a) { *p = a.v[0]; }
 
 struct GroupInfo {
   int prob;
   int lanes;     // active systems in this group
   int i0;        // first member (perturbation groups)
   int q;         // quadrature index, -1 for the mean system
-  int lg;        // group index inside the problem
 };
 
 __device__ __forceinline__ GroupInfo decode_group(const ProblemDev* tab, int count, int gg) {
   GroupInfo gi;
-  int p = 0;
-  while (p + 1 < count && tab[p + 1].group_base <= gg) ++p;
-  const ProblemDev& pr = tab[p];
-  gi.prob = p;
-  gi.lg = gg - pr.group_base;
-  if (gi.lg < pr.mean_sys) {         // the mean system comes first (hardest shift)
+  int lo = 0, hi = count - 1;   // the last problem whose group_base is at most gg
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (tab[mid].group_base <= gg) lo = mid;
+    else hi = mid - 1;
+  }
+  const ProblemDev& pr = tab[lo];
+  gi.prob = lo;
+  const int lg = gg - pr.group_base;
+  if (lg < pr.mean_sys) {         // the mean system comes first (hardest shift)
     gi.q = -1;
     gi.i0 = 0;
     gi.lanes = 1;
   } else {
-    const int pg = gi.lg - pr.mean_sys;
+    const int pg = lg - pr.mean_sys;
     gi.q = pg / pr.groups_per_q;
     gi.i0 = (pg % pr.groups_per_q) * pr.JT;
     const int left = (int)pr.N - gi.i0;
@@ -83,74 +92,117 @@ __device__ __forceinline__ GroupInfo decode_group(const ProblemDev* tab, int cou
   return gi;
 }
 
-template <typename T, int JT, int KMAX>
+template <typename T, int KMAX>
 struct PcgShared {
-  double rho[JT], bn2[JT], rr[JT];
+  static constexpr int JT = PcgVec<T>::JT;
+  alignas(16) T coef[2 * KMAX][JT];        // direction: c for the Phi columns, -t for the C Phi columns
+  T red[4 * kPcgWarps][JT];                // projections: [set][4 nq columns]
   double Gq[KMAX * KMAX + 1];
-  double thq[KMAX + 1];
+  double ith[KMAX + 1];                    // 1 / (theta + sigma)
+  double rho[JT], bn2[JT], rr[JT];
   T alpha[JT], beta[JT];
-  T tco[JT][KMAX + 1], cco[JT][KMAX + 1];
-  int active[JT];
-  int iters[JT];
-  int any_active;
-  int group;
+  float wpf[JT][kPcgWarps][2];
+  double wpd[JT][kPcgWarps];
+  double ts[JT][KMAX + 1];
+  int active[JT], iters[JT];
+  int any_active, group;
   double sigma, beta_lmp;
 };
 
-// Warp-level partial of a DotAcc into shared memory (lane 0 writes).
-template <typename T>
-__device__ __forceinline__ void warp_partial(const DotAcc<T>& acc, float* ff, double* dd, int lane) {
+// Sums acc over the lanes of a warp that serve the same systems (lane mod G)
+// and writes the warp's partial of each system.
+template <typename T, int KMAX>
+__device__ __forceinline__ void warp_partials(PcgShared<T, KMAX>& sh, const DotAcc<T> (&acc)[PcgVec<T>::VL], int warp,
+                                              int lane) {
+  constexpr int VL = PcgVec<T>::VL, G = PcgVec<T>::JT / VL;
+#pragma unroll
+  for (int v = 0; v < VL; ++v) {
+    if constexpr (sizeof(T) == 4) {
+      float hi = acc[v].hi, lo = acc[v].lo;
+#pragma unroll
+      for (int o = 16; o >= G; o >>= 1) {
+        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
+        const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        ff_merge(hi, lo, h2, l2);
+      }
+      if (lane < G) {
+        sh.wpf[lane * VL + v][warp][0] = hi;
+        sh.wpf[lane * VL + v][warp][1] = lo;
+      }
+    } else {
+      double s = acc[v].value();
+#pragma unroll
+      for (int o = 16; o >= G; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane < G) sh.wpd[lane * VL + v][warp] = s;
+    }
+  }
+}
+
+// Sum of the warps' partials of system j, by one warp.  Every lane returns lane
+// 0's value: the callers branch on it, and all lanes must take the same way
+// (the low parts of a float-float butterfly may differ between lanes).
+template <typename T, int KMAX>
+__device__ __forceinline__ double combine_partials(const PcgShared<T, KMAX>& sh, int j, int lane) {
+  static_assert(kPcgWarps <= 32, "one lane per warp partial");
+  double s;
   if constexpr (sizeof(T) == 4) {
-    float hi = acc.hi, lo = acc.lo;
+    float hi = lane < kPcgWarps ? sh.wpf[j][lane][0] : 0.f, lo = lane < kPcgWarps ? sh.wpf[j][lane][1] : 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
       const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
       ff_merge(hi, lo, h2, l2);
     }
-    if (lane == 0) { ff[0] = hi; ff[1] = lo; }
+    s = (double)hi + (double)lo;
   } else {
-    const double s = warp_sum(acc.value());
-    if (lane == 0) dd[0] = s;
+    s = lane < kPcgWarps ? sh.wpd[j][lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   }
+  return __shfl_sync(0xffffffffu, s, 0);
 }
 
-// Sum of the NW warp partials written by warp_partial (called by one thread).
-template <typename T, int NW>
-__device__ __forceinline__ double combine_partials(const float (*ff)[2], const double* dd) {
-  if constexpr (sizeof(T) == 4) {
-    float hi = 0.f, lo = 0.f;
-    for (int w = 0; w < NW; ++w) ff_merge(hi, lo, ff[w][0], ff[w][1]);
-    return (double)hi + (double)lo;
-  } else {
-    double s = 0.0;
-    for (int w = 0; w < NW; ++w) s += dd[w];
-    return s;
-  }
+// Where a group's vectors live, by the problem's size: level 0 all four in
+// shared memory, 1 the direction p (which the matvec gathers) there and the
+// others in the CTA's global slice, 2 all in the slice.
+struct PcgLayout {
+  int level;
+  size_t pvec, vec;   // elements of p (rows padded by a quarter in FP32) and of the others
+};
+
+// Row of p in its buffer: FP32 rows of 32 bytes get one empty row after every
+// four, so that rows four apart (the e-th columns of neighbouring row quads)
+// start in different banks.
+template <typename T>
+__host__ __device__ __forceinline__ int64_t p_row(int64_t a) {
+  return sizeof(T) == 4 ? a + (a >> 2) : a;
 }
 
-// CTAs per SM the kernel is compiled for: kPcgFp32CtasPerSm for the FP32 path
-// with a small Ritz rank (the register budget a thread then gets lets that
-// many 256-thread CTAs share an SM), one otherwise.  The grid is sized by the
-// measured occupancy at launch, and the vector scratch by this count.
-constexpr int kPcgFp32CtasPerSm = 2;
+constexpr size_t kPcgSmem = 200 * 1024;   // dynamic shared memory of a CTA (one CTA per SM)
+constexpr int kPcgChunk = 1024;           // rows of r staged at a time for the projections (levels 1 and 2)
+
+template <typename T>
+__host__ __device__ __forceinline__ PcgLayout pcg_layout(int64_t d) {
+  constexpr int JT = PcgVec<T>::JT;
+  PcgLayout l;
+  l.vec = (size_t)d * JT;
+  l.pvec = (size_t)p_row<T>(d + 3) * JT;
+  const size_t chunk = (size_t)kPcgChunk * JT * sizeof(T);
+  if ((l.pvec + 3 * l.vec) * sizeof(T) <= kPcgSmem) l.level = 0;
+  else if (l.pvec * sizeof(T) + chunk <= kPcgSmem) l.level = 1;
+  else l.level = 2;
+  return l;
+}
+
 template <typename T, int KMAX>
-constexpr int pcg_ctas_per_sm() { return (sizeof(T) == 4 && KMAX <= 12) ? kPcgFp32CtasPerSm : 1; }
-
-template <typename T, int JT, int KMAX>
-__global__ void __launch_bounds__(kThreads, pcg_ctas_per_sm<T, KMAX>())
+__global__ void __launch_bounds__(kPcgThreads, 1)
 k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* gscratch,
-      int64_t scratch_stride, int use_smem, uint64_t band_mask, const int32_t* band_fb) {
+      int64_t scratch_stride, uint64_t band_mask, const int32_t* band_fb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int NW = kThreads / 32;
-  constexpr int NVCAP = KMAX <= 12 ? 32 : 64;    // rr, f[k], g[k]
-  __shared__ PcgShared<T, JT, KMAX> sh;
-  __shared__ T red[JT][NVCAP][NW];
-  __shared__ double redd[JT][NVCAP];
-  __shared__ float wpf[JT][NW][2];
-  __shared__ double wpd[JT][NW];
-
+  constexpr int JT = PcgVec<T>::JT, VL = PcgVec<T>::VL, G = JT / VL;
+  __shared__ PcgShared<T, KMAX> sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = tid % G;   // which systems of a row this thread serves, in every item loop
   // Problems in band_mask were given to the band kernel first; this kernel
   // solves them only where it fell back (band_fb[p] != 0).
   auto band_solved = [&](int p) { return ((band_mask >> p) & 1ull) && band_fb[p] == 0; };
@@ -173,18 +225,22 @@ k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* g
       __syncthreads();
       continue;
     }
-    const int64_t d = pr.d, N = pr.N;
+    const int d = (int)pr.d;
+    const int64_t N = pr.N;
     const int k = pr.kR < KMAX ? pr.kR : KMAX;
-
-    T* base = use_smem ? reinterpret_cast<T*>(smem_raw) : gscratch + (int64_t)blockIdx.x * scratch_stride;
-    T* vr = base;
-    T* vp = base + d * JT;
-    T* vy = base + 2 * d * JT;
-    T* vx = base + 3 * d * JT;
-    const T* val = reinterpret_cast<const T*>(pr.oo_val);
-    const T* Phi = reinterpret_cast<const T*>(pr.Phi);
-    const T* CPhi = reinterpret_cast<const T*>(pr.CPhi);
-    const T* W = reinterpret_cast<const T*>(pr.W);
+    const PcgLayout lay = pcg_layout<T>(d);
+    T* sm = reinterpret_cast<T*>(smem_raw);
+    T* slice = gscratch + (int64_t)blockIdx.x * scratch_stride;
+    T* vp = lay.level <= 1 ? sm : slice + 3 * lay.vec;
+    T* vr = lay.level == 0 ? sm + lay.pvec : slice;
+    T* vy = vr + lay.vec;
+    T* vx = vy + lay.vec;
+    T* rbuf = lay.level == 0 ? vr : (lay.level == 1 ? sm + lay.pvec : sm);   // rows of r under projection
+    const int crows = lay.level == 0 ? d : kPcgChunk;
+    const T* __restrict__ val = reinterpret_cast<const T*>(pr.oo_val);
+    const int32_t* __restrict__ col = pr.oo_col;
+    const T* __restrict__ PhiT = reinterpret_cast<const T*>(pr.phiT);   // [2 k][d]
+    const T* __restrict__ W = reinterpret_cast<const T*>(pr.W);
 
     // ---- group setup: shift, LMP constants, G_q ----
     if (tid == 0) {
@@ -195,7 +251,7 @@ k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* g
     __syncthreads();
     const double sigma = sh.sigma;
     const T sigma_t = to_t<T>(sigma);
-    for (int e = tid; e < k * k; e += blockDim.x) {
+    for (int e = tid; e < k * k; e += kPcgThreads) {
       const int i = e / k, j = e % k;
       const int kk = pr.kR;   // gram matrices are stored with the problem's k
       const int ge = i * kk + j, gt = j * kk + i;
@@ -203,214 +259,348 @@ k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* g
       sh.Gq[e] = pr.gram[2 * kk * kk + ge] + sigma * (pr.gram[kk * kk + ge] + pr.gram[kk * kk + gt]) +
                  sigma * sigma * pr.gram[ge];
     }
-    for (int m = tid; m < k; m += blockDim.x) sh.thq[m] = pr.theta[m] + sigma;
+    for (int m = tid; m < k; m += kPcgThreads) sh.ith[m] = 1.0 / (pr.theta[m] + sigma);
     if (tid < JT) {
       sh.active[tid] = tid < gi.lanes;
       sh.iters[tid] = 0;
       sh.beta[tid] = T(0);
       sh.rr[tid] = 0.0;
+      sh.alpha[tid] = T(0);
     }
 
     // ---- x = 0, r = b, p = 0 ----
-    for (int64_t a = tid; a < d; a += blockDim.x) {
-      Row<T, JT> rb, zero;
-      const T ri = to_t<T>(pr.rinv[a]);
-#pragma unroll
-      for (int j = 0; j < JT; ++j) {
-        zero.v[j] = T(0);
-        T b = T(0);
-        if (j < gi.lanes) {
-          if (gi.q < 0) b = to_t<T>(pr.bmean[a]);
-          else b = W[a * N + gi.i0 + j] * ri;
-        }
-        rb.v[j] = b;
+    for (int e = tid; e < d * JT; e += kPcgThreads) {
+      const int a = e / JT, j = e % JT;
+      T b = T(0);
+      if (j < gi.lanes) {
+        if (gi.q < 0) b = to_t<T>(pr.bmean[a]);
+        else b = W[a * N + gi.i0 + j] * to_t<T>(pr.rinv[a]);
       }
-      st_row<T, JT>(vr, a, rb);
-      st_row<T, JT>(vp, a, zero);
-      st_row<T, JT>(vx, a, zero);
+      vr[e] = b;
+      vx[e] = T(0);
+      vp[p_row<T>(a) * JT + j] = T(0);
     }
     __syncthreads();
 
     bool first = true;
     const int maxit = pr.fixed_iters > 0 ? pr.fixed_iters : pr.max_iter;
-    const int pk = pr.kR;   // row stride of Phi / CPhi
+    const int nq = (2 * k + 3) / 4;              // column quads of [Phi | C Phi]
+    const int sets = nq > 0 ? kPcgWarps / nq : 1;   // warps per quad
+    const int quad = nq > 0 ? warp % nq : 0, set = nq > 0 ? warp / nq : 0;
 
-    // rr, f = Phi^T r, g = A^T r -> preconditioner scalars
-    auto reduce_residual = [&]() {
-#pragma unroll 1
-      for (int j = 0; j < JT; ++j) {
-        T v[NVCAP];
+    // The update x += alpha p, r -= alpha y (not on the first call), then
+    // r^T r, f = Phi^T r and g = A^T r, in one pass: rows of r go through
+    // shared memory, where warp (quad, set) projects them on its four columns
+    // with 4 JT register accumulators, lanes over rows (coalesced columns).
+    // Then the scalars, one warp per system.
+    auto residual_pass = [&]() {
+      DotAcc<T> rr[VL];
+      T acc[4][JT];
 #pragma unroll
-        for (int i = 0; i < NVCAP; ++i) v[i] = T(0);
-        DotAcc<T> rr;
-        for (int64_t a = tid; a < d; a += blockDim.x) {
-          const T r = vr[a * JT + j];
-          rr.add_prod(r, r);
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int m = 0; m < KMAX; ++m) {
-            if (m < k) {
-              v[1 + m] += Phi[a * pk + m] * r;
-              v[1 + KMAX + m] += CPhi[a * pk + m] * r;
+        for (int j = 0; j < JT; ++j) acc[i][j] = T(0);
+      T al[VL];
+#pragma unroll
+      for (int v = 0; v < VL; ++v) al[v] = sh.alpha[g * VL + v];
+      for (int c0 = 0; c0 < d; c0 += crows) {
+        const int nr = d - c0 < crows ? d - c0 : crows;
+        // kU items at once: their loads are all in flight before the first use
+        // (levels 1 and 2 stream the vectors from L2)
+        constexpr int kU = 2;
+        for (int it0 = tid; it0 < nr * G; it0 += kU * kPcgThreads) {
+          Item<T> r[kU], y[kU], x[kU], p[kU];
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const int it = it0 + u * kPcgThreads;
+            if (it >= nr * G) continue;
+            const int64_t o = ((int64_t)c0 * G + it) * VL;
+            r[u] = ld_item(vr + o);
+            if (first) continue;
+            y[u] = ld_item(vy + o);
+            x[u] = ld_item(vx + o);
+            p[u] = ld_item(vp + p_row<T>(c0 + it / G) * JT + g * VL);
+          }
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const int it = it0 + u * kPcgThreads;
+            if (it >= nr * G) continue;
+            const int64_t o = ((int64_t)c0 * G + it) * VL;
+            if (!first) {
+#pragma unroll
+              for (int v = 0; v < VL; ++v) {
+                x[u].v[v] += al[v] * p[u].v[v];
+                r[u].v[v] -= al[v] * y[u].v[v];
+              }
+              st_item(vx + o, x[u]);
+              st_item(vr + o, r[u]);
+            }
+            if (lay.level != 0) st_item(rbuf + (int64_t)it * VL, r[u]);
+#pragma unroll
+            for (int v = 0; v < VL; ++v) rr[v].add_prod(r[u].v[v], r[u].v[v]);
+          }
+        }
+        if (nq == 0) continue;
+        __syncthreads();
+        if (set < sets) {
+          const int m0 = 4 * quad;
+#pragma unroll 2
+          for (int a = lane + 32 * set; a < nr; a += 32 * sets) {
+            T rv[JT];
+#pragma unroll
+            for (int u = 0; u < G; ++u) {
+              const Item<T> t = ld_item(rbuf + (int64_t)a * JT + u * VL);
+#pragma unroll
+              for (int v = 0; v < VL; ++v) rv[u * VL + v] = t.v[v];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const T ph = m0 + i < 2 * k ? PhiT[(int64_t)(m0 + i) * d + c0 + a] : T(0);
+#pragma unroll
+              for (int j = 0; j < JT; ++j) acc[i][j] += ph * rv[j];
             }
           }
         }
-        const T s0 = warp_reduce_scatter32<T>(*reinterpret_cast<T(*)[32]>(&v[0]), lane);
-        red[j][lane][warp] = s0;
-        if constexpr (NVCAP == 64) {
-          const T s1 = warp_reduce_scatter32<T>(*reinterpret_cast<T(*)[32]>(&v[32]), lane);
-          red[j][32 + lane][warp] = s1;
-        }
-        warp_partial<T>(rr, wpf[j][warp], &wpd[j][warp], lane);
+        if (c0 + crows < d) __syncthreads();   // the next chunk overwrites the buffer
       }
-      __syncthreads();
-      for (int e = tid; e < JT * NVCAP; e += blockDim.x) {
-        const int j = e / NVCAP, vi = e % NVCAP;
-        if (vi == 0) {
-          redd[j][0] = combine_partials<T, NW>(wpf[j], wpd[j]);
-        } else {
-          T s = T(0);
+      warp_partials<T, KMAX>(sh, rr, warp, lane);
+      if (nq > 0 && set < sets) {
+        // reduce-scatter the 4 JT sums over the warp: first halve the values
+        // held per lane, then sum the lanes that hold the same value
+        constexpr int V = 4 * JT;   // 32 (FP32) or 8 (FP64)
+        T* v = &acc[0][0];
+        int idx = 0;
 #pragma unroll
-          for (int w = 0; w < NW; ++w) s += red[j][vi][w];
-          redd[j][vi] = (double)s;
+        for (int off = 16, w = V / 2; w >= 1; off >>= 1, w >>= 1) {
+          const bool up = (lane & off) != 0;
+#pragma unroll
+          for (int i = 0; i < w; ++i) {
+            const T send = up ? v[i] : v[i + w];
+            const T keep = up ? v[i + w] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+          }
+          if (up) idx += w;
         }
+#pragma unroll
+        for (int off = 16 / V; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+        if (V == 32 || (lane & 3) == 0) sh.red[set * 4 * nq + 4 * quad + idx / JT][idx % JT] = v[0];
       }
       __syncthreads();
-      if (tid < JT) {
-        const int j = tid;
-        const double rr = redd[j][0];
-        if (first) sh.bn2[j] = rr;
-        const bool was_active = sh.active[j];
+      if (warp < JT) {
+        const int j = warp;
+        const double rr_j = combine_partials<T, KMAX>(sh, j, lane);
+        const bool was_active = sh.active[j] != 0;
+        const double bn2 = first ? rr_j : sh.bn2[j];
+        __syncwarp();   // lane 0 writes both below
         bool act = was_active;
-        if (act && pr.fixed_iters <= 0 && !(rr > pr.tol * pr.tol * sh.bn2[j])) act = false;
-        if (act && !(rr > 0.0)) act = false;
-        if (act && !isfinite(rr)) act = false;
-        double rho = rr;
-        if (k > 0) {
-          double t[KMAX], t2[KMAX];
-          for (int m = 0; m < k; ++m) t[m] = redd[j][1 + m] / sh.thq[m];
-          double gt = 0.0, fc = 0.0;
-          for (int m = 0; m < k; ++m) {
-            double acc = redd[j][1 + KMAX + m] + sigma * redd[j][1 + m];
-            for (int i2 = 0; i2 < k; ++i2) acc -= sh.Gq[m * k + i2] * t[i2];
-            t2[m] = acc;
+        if (act && pr.fixed_iters <= 0 && !(rr_j > pr.tol * pr.tol * bn2)) act = false;
+        if (act && (!(rr_j > 0.0) || !isfinite(rr_j))) act = false;
+        double rho = rr_j;
+        if (k > 0 && act) {
+          T fs = T(0), gs = T(0);
+          if (lane < k)
+            for (int s = 0; s < sets; ++s) {
+              fs += sh.red[s * 4 * nq + lane][j];
+              gs += sh.red[s * 4 * nq + k + lane][j];
+            }
+          const double f = (double)fs, gg2 = (double)gs;
+          const double ith = lane < k ? sh.ith[lane] : 0.0;
+          const double t = f * ith;
+          if (lane < k) sh.ts[j][lane] = t;
+          __syncwarp();
+          double a0 = 0.0, a1 = 0.0;   // G_q t, two chains
+          if (lane < k) {
+            int i2 = 0;
+            for (; i2 + 1 < k; i2 += 2) {
+              a0 += sh.Gq[lane * k + i2] * sh.ts[j][i2];
+              a1 += sh.Gq[lane * k + i2 + 1] * sh.ts[j][i2 + 1];
+            }
+            if (i2 < k) a0 += sh.Gq[lane * k + i2] * sh.ts[j][i2];
           }
-          for (int m = 0; m < k; ++m) {
-            const double c = (sh.beta_lmp - sigma) * t[m] - t2[m] / sh.thq[m];
-            gt += redd[j][1 + KMAX + m] * t[m];
-            fc += redd[j][1 + m] * c;
-            sh.tco[j][m] = to_t<T>(t[m]);
-            sh.cco[j][m] = to_t<T>(c);
+          const double t2 = gg2 + sigma * f - (a0 + a1);
+          const double c = (sh.beta_lmp - sigma) * t - t2 * ith;
+          double df = lane < k ? f * c - gg2 * t : 0.0;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) df += __shfl_xor_sync(0xffffffffu, df, o);
+          rho = rr_j + df;
+          if (lane < k) {
+            sh.coef[lane][j] = to_t<T>(c);
+            sh.coef[k + lane][j] = to_t<T>(-t);
           }
-          rho = rr - gt + fc;
         }
-        if (!act) {
-          sh.beta[j] = T(0);
-          for (int m = 0; m < k; ++m) { sh.tco[j][m] = T(0); sh.cco[j][m] = T(0); }
-        } else if (first) {
-          sh.beta[j] = T(0);
-          sh.rho[j] = rho;
-        } else {
-          sh.beta[j] = to_t<T>(rho / sh.rho[j]);
-          sh.rho[j] = rho;
+        if (lane == 0) {
+          if (first) sh.bn2[j] = rr_j;
+          if (!act) {
+            sh.beta[j] = T(0);
+          } else {
+            sh.beta[j] = first ? T(0) : to_t<T>(rho / sh.rho[j]);
+            sh.rho[j] = rho;
+          }
+          if (was_active || first) sh.rr[j] = rr_j;
+          sh.active[j] = act;
         }
-        if (was_active || first) sh.rr[j] = rr;
-        sh.active[j] = act;
       }
       __syncthreads();
-      if (tid == 0) {
-        int any = 0;
-        for (int j = 0; j < JT; ++j) any |= sh.active[j];
-        sh.any_active = any;
-      }
-      __syncthreads();
+      int any = 0;
+#pragma unroll
+      for (int j = 0; j < JT; ++j) any |= sh.active[j];
+      return any != 0;
     };
 
-    // z = P^-1 r, p = z + beta p
+    // z = P^-1 r, p = z + beta p (a stopped system keeps its p)
     auto update_direction = [&]() {
-      for (int64_t a = tid; a < d; a += blockDim.x) {
-        const Row<T, JT> r = ld_row<T, JT>(vr, a);
-        Row<T, JT> p = ld_row<T, JT>(vp, a);
-        T z[JT];
+      T be[VL];
+      bool on[VL];
 #pragma unroll
-        for (int j = 0; j < JT; ++j) z[j] = r.v[j];
-        for (int m = 0; m < k; ++m) {
-          const T ph = Phi[a * pk + m], cp = CPhi[a * pk + m];
+      for (int v = 0; v < VL; ++v) {
+        be[v] = sh.beta[g * VL + v];
+        on[v] = sh.active[g * VL + v] != 0;
+      }
+      constexpr int kU = sizeof(T) == 4 ? 4 : 2;   // items side by side: one read of the coefficients serves all
+      for (int it = tid; it < d * G; it += kU * kPcgThreads) {
+        Item<T> z[kU];
+        int a[kU];
 #pragma unroll
-          for (int j = 0; j < JT; ++j) z[j] += ph * sh.cco[j][m] - cp * sh.tco[j][m];
+        for (int u = 0; u < kU; ++u) {
+          const int iu = it + u * kPcgThreads;
+          a[u] = iu < d * G ? iu / G : 0;
+          z[u] = ld_item(vr + (int64_t)a[u] * JT + g * VL);
+        }
+#pragma unroll 4
+        for (int m = 0; m < 2 * k; ++m) {
+          const Item<T> c = ld_item(&sh.coef[m][g * VL]);
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const T ph = PhiT[(int64_t)m * d + a[u]];
+#pragma unroll
+            for (int v = 0; v < VL; ++v) z[u].v[v] += ph * c.v[v];
+          }
         }
 #pragma unroll
-        for (int j = 0; j < JT; ++j) p.v[j] = sh.active[j] ? z[j] + sh.beta[j] * p.v[j] : p.v[j];
-        st_row<T, JT>(vp, a, p);
+        for (int u = 0; u < kU; ++u) {
+          if (it + u * kPcgThreads >= d * G) continue;
+          T* pp = vp + p_row<T>(a[u]) * JT + g * VL;
+          Item<T> p = ld_item(pp);
+#pragma unroll
+          for (int v = 0; v < VL; ++v) p.v[v] = on[v] ? z[u].v[v] + be[v] * p.v[v] : p.v[v];
+          st_item(pp, p);
+        }
       }
       __syncthreads();
     };
 
-    reduce_residual();
+    bool run = residual_pass();
     first = false;
-    if (sh.any_active) update_direction();
+    if (run) update_direction();
+
+    // FP32: C by quads of rows where the set-up made them (k_pcg_quads)
+    const bool quads = sizeof(T) == 4 && pr.qval && pr.status[2] == 0;
+    // items of the matvec, and threads per item: the largest power of two that
+    // still covers all items at once (small problems split a row's entries)
+    const int items = (quads ? (d + 3) / 4 : d) * G;
+    int tpi = 1;
+    while (tpi < 16 && 2 * tpi * items <= kPcgThreads) tpi *= 2;
+    const int per = 32 / tpi, sub = lane / per, ii = lane % per;
 
     int it = 0;
-    while (sh.any_active && it < maxit) {
+    while (run && it < maxit) {
       ++it;
       // ---- y = C_q p, p^T y ----
-      DotAcc<T> pap[JT];
-      for (int64_t a = tid; a < d; a += blockDim.x) {
-        const Row<T, JT> p = ld_row<T, JT>(vp, a);
-        T acc[JT];
+      DotAcc<T> pap[VL];
+      const int iend = (items + per - 1) / per * per;   // whole warps take part in the shuffles
+      if constexpr (sizeof(T) == 4) {
+        if (quads) {
+          const int nb = (d + 3) / 4;
+          const float4* __restrict__ qv = reinterpret_cast<const float4*>(pr.qval);
+          const int32_t* __restrict__ qc = pr.qcol;
+          for (int i = warp * per + ii; i < iend; i += kPcgWarps * per) {
+            const bool in = i < items;
+            const int blk = in ? i / G : 0;
+            float acc[4][VL] = {};
+            const int n = in ? pr.qn[blk] : 0;
+#pragma unroll 8
+            for (int e = sub; e < n; e += tpi) {
+              const float4 c = qv[(int64_t)e * nb + blk];
+              const Item<T> pb = ld_item(vp + qc[(int64_t)e * nb + blk] + g * VL);
+              const float cc[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
-        for (int j = 0; j < JT; ++j) acc[j] = sigma_t * p.v[j];
-        const int nnz = pr.oo_nnz[a];
-        for (int e = 0; e < nnz; ++e) {
-          const T c = val[(int64_t)e * d + a];
-          const int b = pr.oo_col[(int64_t)e * d + a];
-          const Row<T, JT> pb = ld_row<T, JT>(vp, b);
+              for (int w = 0; w < 4; ++w)
 #pragma unroll
-          for (int j = 0; j < JT; ++j) acc[j] += c * pb.v[j];
-        }
-        Row<T, JT> y;
+                for (int v = 0; v < VL; ++v) acc[w][v] = fmaf(cc[w], pb.v[v], acc[w][v]);
+            }
+            for (int o = 16; o >= per; o >>= 1)
 #pragma unroll
-        for (int j = 0; j < JT; ++j) {
-          y.v[j] = acc[j];
-          pap[j].add_prod(p.v[j], acc[j]);
-        }
-        st_row<T, JT>(vy, a, y);
-      }
+              for (int w = 0; w < 4; ++w)
 #pragma unroll
-      for (int j = 0; j < JT; ++j) warp_partial<T>(pap[j], wpf[j][warp], &wpd[j][warp], lane);
-      __syncthreads();
-      if (tid < JT) {
-        const int j = tid;
-        T alpha = T(0);
-        if (sh.active[j]) {
-          const double pAp = combine_partials<T, NW>(wpf[j], wpd[j]);
-          if (pAp > 0.0 && isfinite(pAp)) {
-            alpha = to_t<T>(sh.rho[j] / pAp);
-            sh.iters[j] = it;
-          } else {
-            sh.active[j] = 0;
-            atomicOr(&pr.status[0], kStatBreakdown);
+                for (int v = 0; v < VL; ++v) acc[w][v] += __shfl_xor_sync(0xffffffffu, acc[w][v], o);
+            if (in && sub == 0) {
+#pragma unroll
+              for (int w = 0; w < 4; ++w) {
+                const int a = 4 * blk + w;
+                if (a >= d) break;
+                const Item<T> p = ld_item(vp + p_row<T>(a) * JT + g * VL);
+                Item<T> y;
+#pragma unroll
+                for (int v = 0; v < VL; ++v) {
+                  y.v[v] = fmaf(sigma_t, p.v[v], acc[w][v]);
+                  pap[v].add_prod(p.v[v], y.v[v]);
+                }
+                st_item(vy + (int64_t)a * JT + g * VL, y);
+              }
+            }
           }
         }
-        sh.alpha[j] = alpha;
       }
-      __syncthreads();
-      // ---- x += alpha p, r -= alpha y ----
-      for (int64_t a = tid; a < d; a += blockDim.x) {
-        const Row<T, JT> p = ld_row<T, JT>(vp, a);
-        const Row<T, JT> y = ld_row<T, JT>(vy, a);
-        Row<T, JT> x = ld_row<T, JT>(vx, a);
-        Row<T, JT> r = ld_row<T, JT>(vr, a);
+      if (!quads) {
+        for (int i = warp * per + ii; i < iend; i += kPcgWarps * per) {
+          const bool in = i < items;
+          const int a = in ? i / G : 0;
+          Item<T> acc{};
+          const int nnz = in ? pr.oo_nnz[a] : 0;
+#pragma unroll 4
+          for (int e = sub; e < nnz; e += tpi) {
+            const T c = val[(int64_t)e * d + a];
+            const int b = col[(int64_t)e * d + a];
+            const Item<T> pb = ld_item(vp + p_row<T>(b) * JT + g * VL);
 #pragma unroll
-        for (int j = 0; j < JT; ++j) {
-          x.v[j] += sh.alpha[j] * p.v[j];
-          r.v[j] -= sh.alpha[j] * y.v[j];
+            for (int v = 0; v < VL; ++v) acc.v[v] += c * pb.v[v];
+          }
+          for (int o = 16; o >= per; o >>= 1)
+#pragma unroll
+            for (int v = 0; v < VL; ++v) acc.v[v] += __shfl_xor_sync(0xffffffffu, acc.v[v], o);
+          if (in && sub == 0) {
+            const Item<T> p = ld_item(vp + p_row<T>(a) * JT + g * VL);
+#pragma unroll
+            for (int v = 0; v < VL; ++v) {
+              acc.v[v] += sigma_t * p.v[v];
+              pap[v].add_prod(p.v[v], acc.v[v]);
+            }
+            st_item(vy + (int64_t)a * JT + g * VL, acc);
+          }
         }
-        st_row<T, JT>(vx, a, x);
-        st_row<T, JT>(vr, a, r);
+      }
+      warp_partials<T, KMAX>(sh, pap, warp, lane);
+      __syncthreads();
+      if (warp < JT) {
+        const int j = warp;
+        const double pAp = combine_partials<T, KMAX>(sh, j, lane);
+        if (lane == 0) {
+          T alpha = T(0);
+          if (sh.active[j]) {
+            if (pAp > 0.0 && isfinite(pAp)) {
+              alpha = to_t<T>(sh.rho[j] / pAp);
+              sh.iters[j] = it;
+            } else {
+              sh.active[j] = 0;
+              atomicOr(&pr.status[0], kStatBreakdown);
+            }
+          }
+          sh.alpha[j] = alpha;
+        }
       }
       __syncthreads();
-      reduce_residual();
-      if (!sh.any_active) break;
+      run = residual_pass();
+      if (!run) break;
       update_direction();
     }
 
@@ -419,7 +609,7 @@ k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* g
     const int64_t sid0 = gi.q < 0 ? 0 : pr.mean_sys + (int64_t)gi.q * N + gi.i0;
     T* U = reinterpret_cast<T*>(pr.U);
     for (int j = 0; j < gi.lanes; ++j)
-      for (int64_t a = tid; a < d; a += blockDim.x) U[(sid0 + j) * d + a] = vx[a * JT + j];
+      for (int a = tid; a < d; a += kPcgThreads) U[(sid0 + j) * d + a] = vx[(int64_t)a * JT + j];
     if (tid < gi.lanes) {
       const int64_t sidx = sid0 + tid;
       pr.iters[sidx] = sh.iters[tid];
@@ -431,71 +621,174 @@ k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* g
   }
 }
 
-int pcg_jt(int precision) { return precision == 0 ? 4 : 8; }
-
-static size_t vec_bytes(const ProblemTable& tab) {
-  int64_t dmax = 0;
-  for (int i = 0; i < tab.count; ++i) dmax = tab.p[i].d > dmax ? tab.p[i].d : dmax;
-  const int jt = pcg_jt(tab.p[0].precision);
-  const size_t esz = tab.p[0].precision == 0 ? 8 : 4;
-  return (size_t)4 * (size_t)dmax * jt * esz;
+// C by quads of rows for the FP32 matvec: block b holds rows 4 b .. 4 b + 3 over
+// the union of their columns in ascending order, entry e as the four rows'
+// values qval[e][b] (zero where a row lacks the column) and the column's offset
+// in the padded direction buffer qcol[e][b].  Neighbouring observations share
+// most columns (a union is 1.05 to 1.3 times one row's count on 1-D and layered
+// networks), so one 16-byte read of p and 20 bytes of C serve 16 FMAs; by rows
+// it was a read of p and 8 bytes of C per 4.  One warp per block: the union as a bitmap
+// in shared memory, a column's entry is its rank.  A union beyond the capacity sets
+// status[2] and the matvec takes the rows.
+constexpr int kQuadWarps = 4;
+__global__ void __launch_bounds__(32 * kQuadWarps) k_pcg_quads(const ProblemDev* tab) {
+  const ProblemDev& pr = tab[blockIdx.y];
+  if (!pr.qval) return;
+  constexpr int JT = PcgVec<float>::JT;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int d = (int)pr.d, nb = (d + 3) / 4;
+  const int blk = blockIdx.x * kQuadWarps + warp;
+  if (blk >= nb) return;
+  extern __shared__ uint32_t words_s[];   // per warp: bitmap, then the rank of each word's first bit
+  const int nw = (d + 31) / 32;
+  uint32_t* bits = words_s + (size_t)warp * 2 * nw;
+  uint32_t* rank = bits + nw;
+  for (int w = lane; w < nw; w += 32) bits[w] = 0;
+  __syncwarp();
+  const float* val = reinterpret_cast<const float*>(pr.oo_val);
+#pragma unroll 1
+  for (int i = 0; i < 4; ++i) {
+    const int a = 4 * blk + i;
+    const int nnz = a < d ? pr.oo_nnz[a] : 0;
+    for (int e = lane; e < nnz; e += 32) {
+      const int c = pr.oo_col[(int64_t)e * d + a];
+      atomicOr(&bits[c >> 5], 1u << (c & 31));
+    }
+  }
+  __syncwarp();
+  int n = 0;
+  for (int w0 = 0; w0 < nw; w0 += 32) {
+    const int w = w0 + lane;
+    const int cnt = w < nw ? __popc(bits[w]) : 0;
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    if (w < nw) rank[w] = (uint32_t)(n + incl - cnt);
+    n += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  __syncwarp();
+  if (n > pr.qcap) {
+    if (lane == 0) {
+      pr.qn[blk] = 0;
+      atomicExch(&pr.status[2], 1);
+    }
+    return;
+  }
+  if (lane == 0) pr.qn[blk] = n;
+  float4* qv = reinterpret_cast<float4*>(pr.qval);
+  for (int e = lane; e < n; e += 32) qv[(int64_t)e * nb + blk] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int w = lane; w < nw; w += 32) {
+    uint32_t b = bits[w];
+    int e = (int)rank[w];
+    while (b) {
+      const int c = 32 * w + __ffs(b) - 1;
+      pr.qcol[(int64_t)e * nb + blk] = (int32_t)(p_row<float>(c) * JT);
+      ++e;
+      b &= b - 1;
+    }
+  }
+  __syncwarp();   // the zeros before the values (same warp)
+#pragma unroll 1
+  for (int i = 0; i < 4; ++i) {
+    const int a = 4 * blk + i;
+    const int nnz = a < d ? pr.oo_nnz[a] : 0;
+    for (int e = lane; e < nnz; e += 32) {
+      const int c = pr.oo_col[(int64_t)e * d + a];
+      const int at = (int)(rank[c >> 5] + __popc(bits[c >> 5] & ((1u << (c & 31)) - 1u)));
+      pr.qval[((int64_t)at * nb + blk) * 4 + i] = val[(int64_t)e * d + a];
+    }
+  }
 }
 
-static constexpr size_t kSmemVecLimit = 160 * 1024;
+// Capacity of a problem's quads (0: none): FP32 problems that the general
+// kernel solves, up to the size whose bitmaps fit and whose copy stays within
+// 128 MB.
+int64_t pcg_quad_cap(const ProblemDev& p, int count, int32_t solver, int32_t cluster_size) {
+  if (p.precision != 1 || solver != 0 || p.d > 32768 || p.d < 1) return 0;
+  const bool band = cluster_size > 0 || (cluster_size == 0 && count == 1);
+  if (band && band1d_eligible(p)) return 0;
+  const int64_t cap = std::min<int64_t>(p.d, 2 * p.max_oo + 8);
+  return cap * ((p.d + 3) / 4) * 20 <= (int64_t(128) << 20) ? cap : 0;
+}
+
+void launch_pcg_quads(const ProblemTable& tab, const ProblemDev* dtab, cudaStream_t st) {
+  int64_t dmax = 0;
+  for (int i = 0; i < tab.count; ++i)
+    if (tab.p[i].qval) dmax = std::max<int64_t>(dmax, tab.p[i].d);
+  if (dmax < 1) return;
+  const int smem = kQuadWarps * 2 * (int)((dmax + 31) / 32) * 4;   // 32 KB at most
+  const unsigned nb = (unsigned)((dmax + 3) / 4);
+  k_pcg_quads<<<dim3((nb + kQuadWarps - 1) / kQuadWarps, (unsigned)tab.count), 32 * kQuadWarps, smem, st>>>(dtab);
+  note_launches(1);
+}
+
+// [Phi | C Phi] transposed, [2 k][d]: the columns that the kernel reads with
+// consecutive rows on consecutive lanes.
+template <typename T>
+__global__ void k_pcg_phit(const ProblemDev* tab) {
+  const ProblemDev& pr = tab[blockIdx.y];
+  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int k = pr.kR;
+  if (a >= pr.d || k <= 0) return;
+  const T* P = reinterpret_cast<const T*>(pr.Phi);
+  const T* A = reinterpret_cast<const T*>(pr.CPhi);
+  T* out = reinterpret_cast<T*>(pr.phiT);
+  for (int m = 0; m < k; ++m) {
+    out[(int64_t)m * pr.d + a] = P[a * k + m];
+    out[(int64_t)(k + m) * pr.d + a] = A[a * k + m];
+  }
+}
+
+int pcg_jt(int precision) { return precision == 0 ? PcgVec<double>::JT : PcgVec<float>::JT; }
+
+// Elements of one CTA's global slice: what the largest problem keeps there.
+static size_t slice_elems(const ProblemTable& tab) {
+  size_t most = 0;
+  for (int i = 0; i < tab.count; ++i) {
+    const bool f64 = tab.p[i].precision == 0;
+    const PcgLayout l = f64 ? pcg_layout<double>(tab.p[i].d) : pcg_layout<float>(tab.p[i].d);
+    const size_t need = l.level == 0 ? 0 : (l.level == 1 ? 3 * l.vec : 3 * l.vec + l.pvec);
+    most = std::max(most, need);
+  }
+  return (most + 31) / 32 * 32;
+}
 
 size_t pcg_scratch_bytes(const ProblemTable& tab, int num_sms) {
-  const size_t vb = vec_bytes(tab);
-  if (vb <= kSmemVecLimit) return 0;
-  int kmax = 0;
-  for (int i = 0; i < tab.count; ++i) kmax = tab.p[i].kR > kmax ? tab.p[i].kR : kmax;
-  const int per_sm = (tab.p[0].precision == 1 && kmax <= 12) ? kPcgFp32CtasPerSm : 1;
-  return vb * (size_t)num_sms * (size_t)per_sm;   // one slice per resident CTA
+  return slice_elems(tab) * (tab.p[0].precision == 0 ? 8 : 4) * (size_t)num_sms;   // one CTA per SM
 }
 
-template <typename T, int JT, int KMAX>
+template <typename T, int KMAX>
 static int launch_pcg_t(const ProblemTable& tab, const ProblemDev* dtab, int32_t* counter, void* scratch,
                         size_t scratch_bytes, int num_sms, cudaStream_t st, uint64_t band_mask,
                         const int32_t* band_fb) {
-  const size_t vb = vec_bytes(tab);
-  const int use_smem = vb <= kSmemVecLimit;
-  const size_t dyn = use_smem ? vb : 0;
-  // the attribute once per thread and device, the occupancy per dynamic size
+  const size_t slice = slice_elems(tab);
+  // the attribute once per thread and device
   constexpr int kMaxDev = 64;
   static thread_local bool attr_set[kMaxDev] = {};
-  static thread_local size_t occ_dyn[kMaxDev] = {};
-  static thread_local int occ_per_sm[kMaxDev] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
     cudaGetLastError();
     dev = -1;
   }
   if (dev < 0 || !attr_set[dev]) {
-    cudaFuncSetAttribute(k_pcg<T, JT, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemVecLimit);
+    cudaFuncSetAttribute(k_pcg<T, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPcgSmem);
     if (dev >= 0) attr_set[dev] = true;
   }
-  int per_sm = 0;
-  if (dev >= 0 && occ_per_sm[dev] > 0 && occ_dyn[dev] == dyn) per_sm = occ_per_sm[dev];
-  if (per_sm < 1) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg<T, JT, KMAX>, kThreads, dyn) != cudaSuccess ||
-        per_sm < 1) {
-      cudaGetLastError();
-      per_sm = 1;
-    }
-    if (dev >= 0) {
-      occ_dyn[dev] = dyn;
-      occ_per_sm[dev] = per_sm;
-    }
-  }
-  int64_t want = (int64_t)per_sm * num_sms;
-  if (!use_smem && vb > 0) want = std::min<int64_t>(want, (int64_t)(scratch_bytes / vb));   // scratch slices
-  int grid = (int)std::min<int64_t>(tab.total_groups, want);
-  if (!use_smem && grid < 1 && tab.total_groups > 0) return -1;
-  if (grid <= 0) return 0;
+  int64_t want = num_sms;
+  if (slice > 0) want = std::min<int64_t>(want, (int64_t)(scratch_bytes / (slice * sizeof(T))));   // scratch slices
+  const int grid = (int)std::min<int64_t>(tab.total_groups, want);
+  if (grid < 1) return tab.total_groups > 0 ? -1 : 0;
+  int64_t dmax = 1;
+  for (int i = 0; i < tab.count; ++i) dmax = std::max<int64_t>(dmax, tab.p[i].d);
+  k_pcg_phit<T><<<dim3((unsigned)((dmax + 255) / 256), (unsigned)tab.count), 256, 0, st>>>(dtab);
   cudaMemsetAsync(counter, 0, sizeof(int32_t), st);
-  k_pcg<T, JT, KMAX><<<grid, kThreads, dyn, st>>>(dtab, tab.count, tab.total_groups, counter,
-                                            reinterpret_cast<T*>(scratch), (int64_t)(vb / sizeof(T)),
-                                            use_smem, band_mask, band_fb);
-  note_launches(1);
+  k_pcg<T, KMAX><<<grid, kPcgThreads, kPcgSmem, st>>>(dtab, tab.count, tab.total_groups, counter,
+                                                       reinterpret_cast<T*>(scratch), (int64_t)slice, band_mask,
+                                                       band_fb);
+  note_launches(2);
   return 0;
 }
 
@@ -522,11 +815,11 @@ int launch_pcg(const ProblemTable& tab, const ProblemDev* dtab, int32_t* counter
     if (launch_pcg_band1d(p, dtab + i, CS, band_q + i, band_fb + i, num_sms, st) == 0) mask |= 1ull << i;
   }
   if (tab.p[0].precision == 0) {
-    if (small) return launch_pcg_t<double, 4, 12>(tab, dtab, counter, scratch, scratch_bytes, num_sms, st, mask, band_fb);
-    return launch_pcg_t<double, 4, 24>(tab, dtab, counter, scratch, scratch_bytes, num_sms, st, mask, band_fb);
+    if (small) return launch_pcg_t<double, 12>(tab, dtab, counter, scratch, scratch_bytes, num_sms, st, mask, band_fb);
+    return launch_pcg_t<double, 24>(tab, dtab, counter, scratch, scratch_bytes, num_sms, st, mask, band_fb);
   }
-  if (small) return launch_pcg_t<float, 8, 12>(tab, dtab, counter, scratch, scratch_bytes, num_sms, st, mask, band_fb);
-  return launch_pcg_t<float, 8, 24>(tab, dtab, counter, scratch, scratch_bytes, num_sms, st, mask, band_fb);
+  if (small) return launch_pcg_t<float, 12>(tab, dtab, counter, scratch, scratch_bytes, num_sms, st, mask, band_fb);
+  return launch_pcg_t<float, 24>(tab, dtab, counter, scratch, scratch_bytes, num_sms, st, mask, band_fb);
 }
 
 // ---------------------------------------------------------------------------

@@ -189,9 +189,10 @@ __global__ void k_tpcg_phit(const ProblemDev* dpr) {
   const float* P = reinterpret_cast<const float*>(pr.Phi);
   const float* A = reinterpret_cast<const float*>(pr.CPhi);
   const bool in = a < pr.d;
+  float* out = reinterpret_cast<float*>(pr.phiT);
   for (int m = 0; m < k; ++m) {
-    pr.phiT[(int64_t)m * pr.d_pad + a] = in ? P[a * k + m] : 0.f;
-    pr.phiT[(int64_t)(k + m) * pr.d_pad + a] = in ? A[a * k + m] : 0.f;
+    out[(int64_t)m * pr.d_pad + a] = in ? P[a * k + m] : 0.f;
+    out[(int64_t)(k + m) * pr.d_pad + a] = in ? A[a * k + m] : 0.f;
   }
 }
 
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_tpcg_update(const ProblemDev* d
     fence_mbar_init();
     if (k > 0) mbar_arrive_expect_tx(&bar, (uint32_t)(2 * k * nrow * 4));
     for (int m = 0; m < 2 * k; ++m)
-      bulk_load(phs_dyn4 + m * (kDotRows / 4), pr.phiT + (int64_t)m * dp + abase, (uint32_t)(nrow * 4), &bar);
+      bulk_load(phs_dyn4 + m * (kDotRows / 4), reinterpret_cast<const float*>(pr.phiT) + (int64_t)m * dp + abase, (uint32_t)(nrow * 4), &bar);
   }
   if (threadIdx.x < kSys) {
     const int64_t pos = g0 + threadIdx.x;
@@ -548,7 +549,7 @@ __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev
 #pragma unroll
     for (int i = 0; i < RPL; ++i) c[m][i] = 0.f;
     if (in) {
-      const float* src = pr.phiT + (int64_t)mm * dp + a;
+      const float* src = reinterpret_cast<const float*>(pr.phiT) + (int64_t)mm * dp + a;
       if constexpr (RPL == 4) {
         const float4 t = __ldg(reinterpret_cast<const float4*>(src));
         c[m][0] = t.x; c[m][1] = t.y; c[m][2] = t.z; c[m][3] = t.w;
