@@ -349,6 +349,7 @@ constexpr int kCounterInts = 256;
 static_assert(1 + 2 * kMaxProblems <= kCounterInts, "PCG counter area");
 
 int64_t pcg_quad_cap(const ProblemDev& p, int count, int32_t solver, int32_t cluster_size);
+void launch_pcg_phit(const ProblemTable& tab, const ProblemDev* dtab, cudaStream_t st);
 void launch_pcg_quads(const ProblemTable& tab, const ProblemDev* dtab, cudaStream_t st);
 
 // PCG vector scratch per CTA when vectors do not fit in shared memory.

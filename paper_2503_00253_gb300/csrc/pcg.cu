@@ -726,7 +726,8 @@ void launch_pcg_quads(const ProblemTable& tab, const ProblemDev* dtab, cudaStrea
 }
 
 // [Phi | C Phi] transposed, [2 k][d]: the columns that the kernel reads with
-// consecutive rows on consecutive lanes.
+// consecutive rows on consecutive lanes.  Last step of the eigensolver's
+// multi-kernel chain (the fused kernel writes it itself).
 template <typename T>
 __global__ void k_pcg_phit(const ProblemDev* tab) {
   const ProblemDev& pr = tab[blockIdx.y];
@@ -740,6 +741,15 @@ __global__ void k_pcg_phit(const ProblemDev* tab) {
     out[(int64_t)m * pr.d + a] = P[a * k + m];
     out[(int64_t)(k + m) * pr.d + a] = A[a * k + m];
   }
+}
+
+void launch_pcg_phit(const ProblemTable& tab, const ProblemDev* dtab, cudaStream_t st) {
+  int64_t dmax = 1;
+  for (int i = 0; i < tab.count; ++i) dmax = std::max<int64_t>(dmax, tab.p[i].d);
+  const dim3 grid((unsigned)((dmax + 255) / 256), (unsigned)tab.count);
+  if (tab.p[0].precision == 0) k_pcg_phit<double><<<grid, 256, 0, st>>>(dtab);
+  else k_pcg_phit<float><<<grid, 256, 0, st>>>(dtab);
+  note_launches(1);
 }
 
 int pcg_jt(int precision) { return precision == 0 ? PcgVec<double>::JT : PcgVec<float>::JT; }
@@ -781,14 +791,11 @@ static int launch_pcg_t(const ProblemTable& tab, const ProblemDev* dtab, int32_t
   if (slice > 0) want = std::min<int64_t>(want, (int64_t)(scratch_bytes / (slice * sizeof(T))));   // scratch slices
   const int grid = (int)std::min<int64_t>(tab.total_groups, want);
   if (grid < 1) return tab.total_groups > 0 ? -1 : 0;
-  int64_t dmax = 1;
-  for (int i = 0; i < tab.count; ++i) dmax = std::max<int64_t>(dmax, tab.p[i].d);
-  k_pcg_phit<T><<<dim3((unsigned)((dmax + 255) / 256), (unsigned)tab.count), 256, 0, st>>>(dtab);
   cudaMemsetAsync(counter, 0, sizeof(int32_t), st);
   k_pcg<T, KMAX><<<grid, kPcgThreads, kPcgSmem, st>>>(dtab, tab.count, tab.total_groups, counter,
                                                        reinterpret_cast<T*>(scratch), (int64_t)slice, band_mask,
                                                        band_fb);
-  note_launches(2);
+  note_launches(1);
   return 0;
 }
 

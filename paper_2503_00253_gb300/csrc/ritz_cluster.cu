@@ -406,6 +406,14 @@ __global__ void __launch_bounds__(kRT, 1) k_ritz_cluster(const ProblemDev* tab) 
     CPhi[(r0 + a) * k + j] = cp;
   }
   __syncthreads();
+  // transposed copy for the general PCG kernel (in the memory of buf, whose last
+  // reads lie before the cluster barriers above)
+  float* PhiT = reinterpret_cast<float*>(pr.phiT);
+  for (int e = tid; e < nrow * k; e += kRT) {
+    const int j = e / nrow, a = e % nrow;
+    PhiT[(int64_t)j * d + r0 + a] = ph_s[a][j];
+    PhiT[(int64_t)(k + j) * d + r0 + a] = cp_s[a][j];
+  }
   RITZ_PHASE(8);
   // ---- Gram matrices of Phi and A = C Phi: gram[0] = Phi^T Phi, [1] = A^T Phi, [2] = A^T A ----
   for (int w3 = 0; w3 < 3; ++w3) {

@@ -180,47 +180,148 @@ __device__ __forceinline__ bool h_row(const ProblemDev& pr, int64_t a, int64_t& 
   return true;
 }
 
-// W = H Z, one thread per (observation, member); the member-0 thread of each
-// observation also forms R^-1/2 and the mean right-hand side R^-1/2 (y - H mu).
+// W = H Z, one CTA per observation: its warps take the row's entries in turn,
+// lanes over members (coalesced rows of Z^T), and the warps' sums are added in
+// order; then R^-1/2 and the mean right-hand side R^-1/2 (y - H mu).  (One
+// thread per (observation, member) walked the whole row: 67 us at 100 rows of
+// 137 entries, on eight SMs.)
+constexpr int kHWarps = 8;
 template <typename T>
-__global__ void k_observe_H(const ProblemDev* tab) {
+__global__ void __launch_bounds__(32 * kHWarps) k_observe_H(const ProblemDev* tab) {
   const ProblemDev& pr = tab[blockIdx.y];
   if (!pr.H_rowptr) return;
-  const int64_t N = pr.N;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= pr.d * N) return;
-  const int64_t a = i / N, k = i - a * N;
+  const int64_t a = blockIdx.x, N = pr.N;
+  if (a >= pr.d) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double part[kHWarps][32];
+  __shared__ double mpart[kHWarps];
+  __shared__ int s_bad;
+  if (threadIdx.x == 0) s_bad = 0;
+  __syncthreads();
   int64_t e0, e1;
   bool bad = !h_row(pr, a, e0, e1);
   const T* Zt = tp<const T>(pr.Zt);
-  double w = 0.0, hmu = 0.0;
-  for (int64_t e = e0; e < e1; ++e) {
-    const int64_t c = pr.H_col[e];
-    if (c < 0 || c >= pr.n) {
-      bad = true;
-      continue;
+  double hmu = 0.0;
+  for (int64_t k0 = 0; k0 < N; k0 += 32) {
+    const int64_t k = k0 + lane;
+    double w = 0.0;
+#pragma unroll 4
+    for (int64_t e = e0 + warp; e < e1; e += kHWarps) {
+      const int64_t c = pr.H_col[e];
+      if (c < 0 || c >= pr.n) {
+        bad = true;
+        continue;
+      }
+      const double h = pr.H_val[e];
+      if (k < N) w += h * (double)Zt[c * N + k];
+      if (k == 0) hmu += h * pr.mu[c];
     }
-    const double h = pr.H_val[e];
-    w += h * (double)Zt[c * N + k];
-    if (k == 0) hmu += h * pr.mu[c];
+    part[warp][lane] = w;
+    if (k == 0) mpart[warp] = hmu;
+    __syncthreads();
+    if (warp == 0 && k < N) {
+      double t = 0.0;
+#pragma unroll
+      for (int u = 0; u < kHWarps; ++u) t += part[u][lane];
+      tp<T>(pr.W)[a * N + k] = to_t<T>(t);
+    }
+    __syncthreads();
   }
-  tp<T>(pr.W)[i] = to_t<T>(w);
-  if (k != 0) return;
+  if (bad) s_bad = 1;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int u = 1; u < kHWarps; ++u) hmu += mpart[u];   // thread 0 holds warp 0's sum
   const double r = pr.R[a];
   const bool bad_r = !(r > 0.0) || !isfinite(r);
   const double ri = bad_r ? 0.0 : 1.0 / sqrt(r);
   pr.rinv[a] = ri;
   if (pr.do_mean) pr.bmean[a] = ri * (pr.y[a] - hmu);
-  if (bad) atomicOr(&pr.status[0], kStatBadObs);
+  if (s_bad) atomicOr(&pr.status[0], kStatBadObs);
   if (bad_r) atomicOr(&pr.status[0], kStatBadR);
 }
 
-// Sxh(x, b) = sum_j H(b, j) L(x, j) z_x . z_j, thread x (consecutive, so that
-// the ELL writes are coalesced) of observation column b = blockIdx.y.
+// Sxh(x, b) = sum_j H(b, j) L(x, j) z_x . z_j.  A CTA owns kXB consecutive grid
+// points: it forms their rows G_x(j) = L(x, j) z_x . z_j over all grid points
+// once in shared memory (zero outside the support), then takes H G_x^T row by
+// row, one warp per observation with its lanes over the row's entries; rows
+// that miss the supports cost no arithmetic.  (Each (x, b) formed its own
+// products z_x . z_j, so every pair (x, j) was formed once per observation
+// that sees j: 656 to 865 us at n = 2000, d = 100, rows of 137 entries.)
+constexpr int kXB = 4;
+constexpr size_t kSxhSmem = 200 * 1024;
 template <typename T>
-__global__ void k_sxh_H(const ProblemDev* tab) {
-  const ProblemDev& pr = tab[blockIdx.z];
+__global__ void __launch_bounds__(256) k_sxh_H(const ProblemDev* tab) {
+  const ProblemDev& pr = tab[blockIdx.y];
   if (!pr.H_rowptr) return;
+  extern __shared__ double Gx[];   // [n][kXB]
+  const int64_t n = pr.n, N = pr.N, d = pr.d;
+  const int64_t x0 = (int64_t)blockIdx.x * kXB;
+  if (x0 >= n || (size_t)n * kXB * 8 > kSxhSmem) return;   // larger grids: k_sxh_H_direct
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const GridDev& g = pr.grid;
+  const T* Zt = tp<const T>(pr.Zt);
+  Coord3 px[kXB];
+#pragma unroll
+  for (int u = 0; u < kXB; ++u) px[u] = flat_to_coord(g, x0 + u < n ? x0 + u : x0);
+  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+    const Coord3 pj = flat_to_coord(g, j);
+    const T* zj = Zt + j * N;
+    for (int u = 0; u < kXB; ++u) {
+      double v = 0.0;
+      if (x0 + u < n) {
+        const double r2 = scaled_r2_tab(g, pr.d2tab, px[u], pj);
+        if (r2 < 4.0) {
+          DotAcc<T> dot;
+          const T* zx = Zt + (x0 + u) * N;
+          for (int64_t k = 0; k < N; ++k) dot.add_prod(zx[k], zj[k]);
+          const double gc = sizeof(T) == 8 ? gaspari_cohn(sqrt(r2)) : (double)gaspari_cohn_f(sqrtf((float)r2));
+          v = gc * dot.value();
+        }
+      }
+      Gx[j * kXB + u] = v;
+    }
+  }
+  __syncthreads();
+  for (int64_t b = warp; b < d; b += nw) {
+    int64_t e0, e1;
+    h_row(pr, b, e0, e1);
+    double acc[kXB] = {};
+    bool hit = false;
+    for (int64_t e = e0 + lane; e < e1; e += 32) {
+      const int64_t c = pr.H_col[e];
+      if (c < 0 || c >= n) continue;
+      const double* gx = Gx + c * kXB;
+      bool any = false;
+#pragma unroll
+      for (int u = 0; u < kXB; ++u) any |= __double_as_longlong(gx[u]) != 0;
+      if (!any) continue;
+      hit = true;
+      const double h = pr.H_val[e];
+#pragma unroll
+      for (int u = 0; u < kXB; ++u) acc[u] += h * gx[u];
+    }
+    if (__any_sync(0xffffffffu, hit)) {
+#pragma unroll
+      for (int u = 0; u < kXB; ++u) acc[u] = warp_sum(acc[u]);
+    }
+    if (lane < kXB && x0 + lane < n) {
+      double v = acc[0];
+#pragma unroll
+      for (int u = 1; u < kXB; ++u) v = lane == u ? acc[u] : v;
+      tp<T>(pr.xo_val)[b * n + x0 + lane] = to_t<T>(v);
+      pr.xo_col[b * n + x0 + lane] = (int32_t)b;
+      if (b == 0) pr.xo_nnz[x0 + lane] = (int32_t)d;
+    }
+  }
+}
+
+// The same for grids whose rows do not fit shared memory: thread x
+// (consecutive, so that the ELL writes are coalesced) of observation column
+// b = blockIdx.y forms its own products.
+template <typename T>
+__global__ void k_sxh_H_direct(const ProblemDev* tab) {
+  const ProblemDev& pr = tab[blockIdx.z];
+  if (!pr.H_rowptr || (size_t)pr.n * kXB * 8 <= kSxhSmem) return;
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t b = blockIdx.y;
   const int64_t n = pr.n, N = pr.N;
@@ -248,29 +349,31 @@ __global__ void k_sxh_H(const ProblemDev* tab) {
   if (b == 0) pr.xo_nnz[x] = (int32_t)pr.d;
 }
 
-// C(a, b) = R_a^-1/2 R_b^-1/2 sum_x H(a, x) Sxh(x, b), one warp per row a with
-// the lanes over b; the Gershgorin bound, the minimum and the sum of the
-// diagonal as in k_band.
+// C(a, b) = R_a^-1/2 R_b^-1/2 sum_x H(a, x) Sxh(x, b), one CTA per row a: a warp
+// per entry with its lanes over the row of H (a column of Sxh is contiguous);
+// the Gershgorin bound, the minimum and the sum of the diagonal as in k_band.
 template <typename T>
-__global__ void k_c_H(const ProblemDev* tab) {
+__global__ void __launch_bounds__(32 * kHWarps) k_c_H(const ProblemDev* tab) {
   const ProblemDev& pr = tab[blockIdx.y];
   if (!pr.H_rowptr) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t a = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t n = pr.n, d = pr.d;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t a = blockIdx.x, n = pr.n, d = pr.d;
   if (a >= d) return;
+  __shared__ double part[kHWarps];
   int64_t e0, e1;
   h_row(pr, a, e0, e1);
   const T* S = tp<const T>(pr.xo_val);
   const double ra = pr.rinv[a];
   double rowsum = 0.0;
-  for (int64_t b = lane; b < d; b += 32) {
+  for (int64_t b = warp; b < d; b += kHWarps) {
     double acc = 0.0;
-    for (int64_t e = e0; e < e1; ++e) {
+    for (int64_t e = e0 + lane; e < e1; e += 32) {
       const int64_t c = pr.H_col[e];
       if (c < 0 || c >= n) continue;
       acc += pr.H_val[e] * (double)S[b * n + c];
     }
+    acc = warp_sum(acc);
+    if (lane != 0) continue;
     const double v = ra * pr.rinv[b] * acc;
     tp<T>(pr.oo_val)[b * d + a] = to_t<T>(v);
     pr.oo_col[b * d + a] = (int32_t)b;
@@ -280,36 +383,33 @@ __global__ void k_c_H(const ProblemDev* tab) {
       atomicAdd(&pr.scal[4], v);
     }
   }
-  rowsum = warp_sum(rowsum);
-  if (lane == 0) {
-    pr.oo_nnz[a] = (int32_t)d;
-    atomic_max_nonneg(&pr.scal[0], rowsum);
-  }
-}
-
-static bool any_general_h(const ProblemTable& tab) {
-  for (int i = 0; i < tab.count; ++i)
-    if (tab.p[i].H_rowptr) return true;
-  return false;
+  if (lane == 0) part[warp] = rowsum;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int u = 1; u < kHWarps; ++u) rowsum += part[u];
+  pr.oo_nnz[a] = (int32_t)d;
+  atomic_max_nonneg(&pr.scal[0], rowsum);
 }
 
 void launch_anomalies(const ProblemTable& tab, const ProblemDev* dtab, cudaStream_t st) {
-  int64_t nmax = 0, dnmax = 0;
+  int64_t nmax = 0, dnmax = 0, dh = 0;   // dh: most observations of a general H
   for (int i = 0; i < tab.count; ++i) {
+    if (tab.p[i].H_rowptr) dh = std::max<int64_t>(dh, tab.p[i].d);
     nmax = tab.p[i].n > nmax ? tab.p[i].n : nmax;
     dnmax = tab.p[i].d * tab.p[i].N > dnmax ? tab.p[i].d * tab.p[i].N : dnmax;
   }
   const bool f64 = tab.p[0].precision == 0;
   dim3 g1((unsigned)((nmax + kAnomPts - 1) / kAnomPts), tab.count);
   dim3 g2((unsigned)((dnmax + 255) / 256), tab.count);
+  const dim3 gh((unsigned)dh, tab.count);
   if (f64) {
     k_anomalies<double><<<g1, 256, 0, st>>>(dtab); note_launches(1);
     k_observe<double><<<g2, 256, 0, st>>>(dtab); note_launches(1);
-    if (any_general_h(tab)) { k_observe_H<double><<<g2, 256, 0, st>>>(dtab); note_launches(1); }
+    if (dh > 0) { k_observe_H<double><<<gh, 32 * kHWarps, 0, st>>>(dtab); note_launches(1); }
   } else {
     k_anomalies<float><<<g1, 256, 0, st>>>(dtab); note_launches(1);
     k_observe<float><<<g2, 256, 0, st>>>(dtab); note_launches(1);
-    if (any_general_h(tab)) { k_observe_H<float><<<g2, 256, 0, st>>>(dtab); note_launches(1); }
+    if (dh > 0) { k_observe_H<float><<<gh, 32 * kHWarps, 0, st>>>(dtab); note_launches(1); }
   }
 }
 
@@ -416,24 +516,45 @@ void launch_band_obs(const ProblemTable& tab, const ProblemDev* dtab, cudaStream
   if (tab.p[0].precision == 0) k_band<double, true><<<go, 256, 0, st>>>(dtab);
   else k_band<float, true><<<go, 256, 0, st>>>(dtab);
   note_launches(1);
-  if (any_general_h(tab)) {
+  int64_t dh = 0;   // most observations of a general H
+  for (int i = 0; i < tab.count; ++i)
+    if (tab.p[i].H_rowptr) dh = std::max<int64_t>(dh, tab.p[i].d);
+  if (dh > 0) {
     // dense Sxh first (C is formed from it), then C
-    int64_t nmax = 0, dh = 0;
+    // grids whose rows of L o Z Z^T fit shared memory, then the others
+    const size_t row = (size_t)kXB * 8;
+    int64_t nfit = 0, nbig = 0;
     for (int i = 0; i < tab.count; ++i)
       if (tab.p[i].H_rowptr) {
-        nmax = std::max<int64_t>(nmax, tab.p[i].n);
-        dh = std::max<int64_t>(dh, tab.p[i].d);
+        int64_t& most = (size_t)tab.p[i].n * row <= kSxhSmem ? nfit : nbig;
+        most = std::max<int64_t>(most, tab.p[i].n);
       }
-    const dim3 gs((unsigned)((nmax + 127) / 128), (unsigned)dh, tab.count);
-    const dim3 gc((unsigned)((dh * 32 + 255) / 256), tab.count);
-    if (tab.p[0].precision == 0) {
-      k_sxh_H<double><<<gs, 128, 0, st>>>(dtab);
-      k_c_H<double><<<gc, 256, 0, st>>>(dtab);
-    } else {
-      k_sxh_H<float><<<gs, 128, 0, st>>>(dtab);
-      k_c_H<float><<<gc, 256, 0, st>>>(dtab);
+    const bool f64 = tab.p[0].precision == 0;
+    if (nfit > 0) {
+      const dim3 gs((unsigned)((nfit + kXB - 1) / kXB), tab.count);
+      const size_t smem = (size_t)nfit * row;
+      static thread_local int raised = -1;
+      int dev = 0;
+      cudaGetDevice(&dev);
+      if (raised != dev) {
+        cudaFuncSetAttribute(k_sxh_H<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSxhSmem);
+        cudaFuncSetAttribute(k_sxh_H<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSxhSmem);
+        raised = dev;
+      }
+      if (f64) k_sxh_H<double><<<gs, 256, smem, st>>>(dtab);
+      else k_sxh_H<float><<<gs, 256, smem, st>>>(dtab);
+      note_launches(1);
     }
-    note_launches(2);
+    if (nbig > 0) {
+      const dim3 gs((unsigned)((nbig + 127) / 128), (unsigned)dh, tab.count);
+      if (f64) k_sxh_H_direct<double><<<gs, 128, 0, st>>>(dtab);
+      else k_sxh_H_direct<float><<<gs, 128, 0, st>>>(dtab);
+      note_launches(1);
+    }
+    const dim3 gc((unsigned)dh, tab.count);
+    if (f64) k_c_H<double><<<gc, 32 * kHWarps, 0, st>>>(dtab);
+    else k_c_H<float><<<gc, 32 * kHWarps, 0, st>>>(dtab);
+    note_launches(1);
   }
 }
 
@@ -665,8 +786,8 @@ void launch_philox(uint64_t seed, int64_t count, double* out, cudaStream_t st) {
 // summed with DotAcc<T> and kept in FP64.  Orthonormalization is CholeskyQR2
 // (each pass: G = X^T X, G = R^T R, X <- X R^-1, the Cholesky factor formed
 // redundantly by every row block).  The l x l eigenproblem uses cyclic
-// Jacobi with one thread per matrix entry and l/2 disjoint rotations per
-// round (round-robin ordering), in the bulk precision.
+// Jacobi with l/2 disjoint rotations per round (round-robin ordering) in
+// FP32, refined by products on the FP64 path.
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ T* ritz_buf(const ProblemDev& pr, int which) {
@@ -832,52 +953,266 @@ __global__ void k_ritz_orth(const ProblemDev* tab, int src) {
     if (j < l) Y[a * l + j] = row[j];
 }
 
-// Element-parallel cyclic Jacobi on B = sym(Om^T C Om) (Gm holds Om^T (C Om)),
-// one thread per entry.  The round-robin pairing of every round is tabulated
-// once; a round is then two barriers (rotations, then the two-sided update).
-// Output: ev (descending) and Rm (eigenvectors).
-template <typename T>
-__device__ __forceinline__ void jacobi_rotation(T app, T aqq, T apq, T& c, T& s) {
-  c = T(1);
-  s = T(0);
-  if (apq != T(0)) {
-    const T theta = (aqq - app) / (T(2) * apq);
-    const T t = (theta >= T(0) ? T(1) : T(-1)) / (fabs(theta) + sqrt(theta * theta + T(1)));
-    c = T(1) / sqrt(t * t + T(1));
-    s = t * c;
+// The same for the FP64 path.  Every block factors G redundantly in float-float arithmetic
+// (right-looking, one barrier per column, one thread per entry) and applies the same elimination to the identity,
+// which leaves W = R^-T; then one thread per entry of X_dst takes its dot
+// product with a column of R^-1.  (One thread per row solved the triangular
+// system as a chain of l^2 / 2 dependent steps: 29 us a call at 60 rows and 37 us
+// at 1024.)  A non-positive pivot
+// zeroes that column (rank loss) and flags kStatEigFail.
+constexpr int kOrthThreads = kMaxRitz * kMaxRitz;   // one thread per entry of G and W
+constexpr int kOrthEntries = kOrthThreads;          // entries of X_dst per block
+__global__ void __launch_bounds__(kOrthThreads) k_ritz_orth64(const ProblemDev* tab, int src) {
+  const ProblemDev& pr = tab[blockIdx.y];
+  const int l = pr.l;
+  const int64_t e0 = (int64_t)blockIdx.x * kOrthEntries, total = pr.d * l;
+  if (l <= 0 || e0 >= total) return;
+  __shared__ FF G[kMaxRitz][kMaxRitz + 1];   // upper triangle
+  __shared__ FF W[kMaxRitz][kMaxRitz + 1];   // lower triangle: R^-T
+  __shared__ double Ri[kMaxRitz][kMaxRitz + 1];   // R^-1, upper triangle
+  __shared__ float s_tiny;
+  const int t = threadIdx.x;
+  const int i = t / kMaxRitz, c = t % kMaxRitz;
+  const bool mine = i < l && c < l;
+  if (mine) {
+    if (i <= c) G[i][c] = ff_from(pr.Gm[i * l + c]);
+    W[i][c] = FF{i == c ? 1.f : 0.f, 0.f};
+  }
+  if (t < 32) {
+    float tr = t < l ? (float)pr.Gm[t * (l + 1)] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+    if (t == 0) s_tiny = 1e-28f * (tr > 0.f ? tr : 1.f);
+  }
+  __syncthreads();
+  const float tiny = s_tiny;
+  for (int j = 0; j < l; ++j) {
+    // eliminate below the pivot, row i > j: G[i][c] -= f G[j][c] (c >= i) and
+    // W[i][c] -= f W[j][c] (c <= j) with f = G[j][i] / G[j][j]
+    const FF gjj = G[j][j];
+    const bool ok = gjj.h > tiny;
+    if (t == 0 && !ok && blockIdx.x == 0) atomicOr(&pr.status[0], kStatEigFail);
+    if (mine && i > j && ok && (c <= j || c >= i)) {
+      const FF f = ff_div(G[j][i], gjj);
+      if (c <= j) W[i][c] = ff_sub(W[i][c], ff_mul(f, W[j][c]));
+      else G[i][c] = ff_sub(G[i][c], ff_mul(f, G[j][c]));
+    }
+    __syncthreads();
+  }
+  // R^-1[i][c] = W[c][i] / sqrt(G[c][c]), i <= c
+  if (mine) {
+    const FF gcc = G[c][c];
+    const FF v = gcc.h > tiny && i <= c ? ff_mul(W[c][i], ff_rsqrt(gcc)) : FF{0.f, 0.f};
+    Ri[i][c] = (double)v.h + (double)v.l;
+  }
+  __syncthreads();
+  const double* X = ritz_buf<double>(pr, src);
+  double* Y = ritz_buf<double>(pr, 1 - src);
+  const int64_t e = e0 + t;
+  if (e < total) {
+    const int64_t a = e / l;
+    const int j = (int)(e - a * l);
+    double s0 = 0.0, s1 = 0.0;   // two chains
+    int u = 0;
+    for (; u + 1 <= j; u += 2) {
+      s0 += X[a * l + u] * Ri[u][j];
+      s1 += X[a * l + u + 1] * Ri[u + 1][j];
+    }
+    if (u <= j) s0 += X[a * l + u] * Ri[u][j];
+    Y[e] = s0 + s1;
   }
 }
-template <>
-__device__ __forceinline__ void jacobi_rotation<float>(float app, float aqq, float apq, float& c, float& s) {
-  c = 1.f;
-  s = 0.f;
-  if (apq != 0.f) {
-    const float theta = __fdividef(aqq - app, 2.f * apq);
-    const float t = copysignf(1.f, theta) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f)));
-    c = rsqrtf(fmaf(t, t, 1.f));
+
+// One-sided (Hestenes) cyclic Jacobi in FP32, one warp per column pair of a
+// round (lane i holds row i): U = B and V = I on entry; each round rotates its
+// pairs so that their columns of U become orthogonal.  At convergence
+// B V = U with orthogonal columns, so the columns of V are eigenvectors and
+// lambda_c = v_c . u_c (sign kept).  Squared column norms are carried through
+// the rotations (alpha' = alpha - t g, beta' = beta + t g) and recomputed once
+// per sweep.  Called by all threads of the block.
+struct JacobiPairs {
+  float U[kMaxRitz][kMaxRitz + 1], V[kMaxRitz][kMaxRitz + 1];
+  float nrm[kMaxRitz];
+  float scale;
+  int8_t pair_p[kMaxRitz][kMaxRitz / 2], pair_q[kMaxRitz][kMaxRitz / 2];
+};
+__device__ void jacobi_pairs(JacobiPairs& jp, int l, int sweeps) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int m = (l + 1) & ~1, npairs = m / 2;
+  // round-robin schedule (circle method): slot 0 fixed, slot s > 0 holds
+  // ((s - 1 + round) mod (m - 1)) + 1; pair w of a round joins slots w and m - 1 - w
+  for (int e = tid; e < (m - 1) * npairs; e += blockDim.x) {
+    const int round = e / npairs, w = e % npairs;
+    const int s1 = w, s2 = m - 1 - w;
+    int p = s1 == 0 ? 0 : ((s1 - 1 + round) % (m - 1)) + 1;
+    int q = ((s2 - 1 + round) % (m - 1)) + 1;
+    if (p > q) { const int x = p; p = q; q = x; }
+    jp.pair_p[round][w] = (int8_t)p;
+    jp.pair_q[round][w] = (int8_t)q;
+  }
+  __syncthreads();
+  auto refresh_norms = [&]() {
+    for (int c = warp; c < l; c += nw) {
+      const float u = lane < l ? jp.U[lane][c] : 0.f;
+      float a = u * u;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane == 0) jp.nrm[c] = a;
+    }
+  };
+  refresh_norms();
+  __syncthreads();
+  if (tid == 0) {
+    float mx = 0.f;
+    for (int c = 0; c < l; ++c) mx = fmaxf(mx, jp.nrm[c]);
+    jp.scale = mx;
+  }
+  __syncthreads();
+  // a pair stays unconverged while the cosine of its columns exceeds 1e-5 and
+  // |u_p . u_q| exceeds 2e-6 of the largest squared column norm (below that it
+  // is FP32 rounding noise of the small columns)
+  const float gabs = 2e-6f * jp.scale;
+  // cyclic Jacobi is quadratically convergent; a round costs a few hundred
+  // cycles of dependent latency, so the sweep count is the cost (FP32 path: four,
+  // the Ritz pairs only shape the preconditioner)
+  for (int sweep = 0; sweep < sweeps; ++sweep) {
+    int busy = 0;
+    for (int round = 0; round < m - 1; ++round) {
+      for (int w = warp; w < npairs; w += nw) {
+        const int p = jp.pair_p[round][w], q = jp.pair_q[round][w];
+        if (q >= l) continue;
+        const float up = lane < l ? jp.U[lane][p] : 0.f, uq = lane < l ? jp.U[lane][q] : 0.f;
+        float g = up * uq;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        const float al = jp.nrm[p], be = jp.nrm[q];
+        if (g == 0.f) continue;
+        busy |= fabsf(g) > gabs && fabsf(g) > 1e-5f * sqrtf(al * be);
+        // rotation from approximate reciprocals and roots: any orthogonal rotation
+        // keeps B V = U exact; these only change how fast the pair converges
+        const float zeta = __fdividef(be - al, 2.f * g);
+        const float z2 = fmaf(zeta, zeta, 1.f);
+        const float tt = copysignf(1.f, zeta) * __fdividef(1.f, fabsf(zeta) + z2 * rsqrtf(z2));
+        const float cs = rsqrtf(fmaf(tt, tt, 1.f)), sn = cs * tt;
+        if (lane < l) {
+          jp.U[lane][p] = cs * up - sn * uq;
+          jp.U[lane][q] = sn * up + cs * uq;
+          const float vp = jp.V[lane][p], vq = jp.V[lane][q];
+          jp.V[lane][p] = cs * vp - sn * vq;
+          jp.V[lane][q] = sn * vp + cs * vq;
+        }
+        if (lane == 0) {
+          jp.nrm[p] = fmaxf(al - tt * g, 0.f);
+          jp.nrm[q] = fmaxf(be + tt * g, 0.f);
+        }
+      }
+      __syncthreads();
+    }
+    refresh_norms();
+    if (!__syncthreads_or(busy)) break;
+  }
+  __syncthreads();
+}
+
+// The FP32 path's eigenpairs of B = sym(Om^T C Om) (Gm holds Om^T (C Om)): ev
+// (descending) and Rm (eigenvectors).
+__global__ void k_ritz_jacobi_pairs(const ProblemDev* tab) {
+  const ProblemDev& pr = tab[blockIdx.x];
+  const int l = pr.l;
+  if (l <= 0) return;
+  __shared__ JacobiPairs jp;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  for (int e = tid; e < l * l; e += blockDim.x) {
+    const int i = e / l, c = e % l;
+    jp.U[i][c] = (float)(0.5 * (pr.Gm[i * l + c] + pr.Gm[c * l + i]));
+    jp.V[i][c] = i == c ? 1.f : 0.f;
+  }
+  jacobi_pairs(jp, l, 4);
+  // eigenvalues (Rayleigh quotients) and the descending order
+  __shared__ float lam[kMaxRitz];
+  for (int c = warp; c < l; c += nw) {
+    float a = lane < l ? jp.V[lane][c] * jp.U[lane][c] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) lam[c] = a;
+  }
+  __syncthreads();
+  if (tid < l) {
+    const float di = lam[tid];
+    int rank = 0;
+    for (int u = 0; u < l; ++u) rank += (lam[u] > di) || (lam[u] == di && u < tid);
+    pr.ev[rank] = (double)di;
+    for (int u = 0; u < l; ++u) pr.Rm[u * l + rank] = (double)jp.V[u][tid];
+  }
+}
+
+
+// The FP64 path's eigenpairs of B.  On this GPU an FP64 instruction of a warp
+// holds the SM's FP64 pipe for about 16 clocks, so cyclic Jacobi in FP64 (nine
+// sweeps of l - 1 rounds) took 486 us at l = 20.  Instead: the FP32 one-sided
+// Jacobi above, then two steps of the quadratically convergent refinement of a
+// symmetric eigenvector matrix by products (Ogita & Aishima 2018): with
+// R = I - X^T X, S = X^T B X and lambda_i = S_ii / (1 - R_ii),
+//   X <- X + X E,  E_ij = (S_ij + lambda_j R_ij) / (lambda_j - lambda_i),
+// R_ij / 2 where the eigenvalues are too close to separate: 1e-6 -> 1e-12 ->
+// rounding.  FP64 Jacobi sweeps on (X^T B X, X), one thread per entry and l / 2
+// disjoint rotations per round, finish what is left, if anything
+// (unseparated eigenvalues).
+constexpr int kEigThreads = kMaxRitz * kMaxRitz;
+__device__ __forceinline__ void jacobi_rotation(double app, double aqq, double apq, double& c, double& s) {
+  c = 1.0;
+  s = 0.0;
+  if (apq != 0.0) {
+    const double theta = (aqq - app) / (2.0 * apq);
+    const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+    c = 1.0 / sqrt(t * t + 1.0);
     s = t * c;
   }
 }
 
-template <typename T>
-__global__ void k_ritz_jacobi(const ProblemDev* tab) {
+// C = A B or A^T B of l x l matrices, one thread per entry; the caller synchronizes.
+template <bool TRANS>
+__device__ __forceinline__ void eig_product(const double (*A)[kMaxRitz + 1], const double (*Bm)[kMaxRitz + 1],
+                                            double (*Cm)[kMaxRitz + 1], int l) {
+  for (int e = threadIdx.x; e < l * l; e += kEigThreads) {
+    const int i = e / l, j = e % l;
+    double s0 = 0.0, s1 = 0.0;
+    int u = 0;
+    for (; u + 1 < l; u += 2) {
+      s0 += (TRANS ? A[u][i] : A[i][u]) * Bm[u][j];
+      s1 += (TRANS ? A[u + 1][i] : A[i][u + 1]) * Bm[u + 1][j];
+    }
+    if (u < l) s0 += (TRANS ? A[u][i] : A[i][u]) * Bm[u][j];
+    Cm[i][j] = s0 + s1;
+  }
+}
+
+__global__ void __launch_bounds__(kEigThreads) k_ritz_jacobi(const ProblemDev* tab) {
   const ProblemDev& pr = tab[blockIdx.x];
   const int l = pr.l;
   if (l <= 0) return;
-  __shared__ T A[2][kMaxRitz][kMaxRitz + 1];
-  __shared__ T V[2][kMaxRitz][kMaxRitz + 1];
-  __shared__ T cs[kMaxRitz][2];                 // (c, s) of the pair containing index x
-  __shared__ int8_t partner[kMaxRitz][kMaxRitz];  // [round][x]
-  __shared__ T red_off[kMaxRitz], red_tot[kMaxRitz];
+  __shared__ double A[2][kMaxRitz][kMaxRitz + 1];
+  __shared__ double V[2][kMaxRitz][kMaxRitz + 1];
+  __shared__ union Scratch {
+    JacobiPairs jp;                                  // FP32 start
+    struct {
+      double B[kMaxRitz][kMaxRitz + 1], lam[kMaxRitz];   // refinement (from the end of the FP32 start on)
+    } r;
+    __device__ Scratch() {}
+  } sc;
+  __shared__ double cs[kMaxRitz][2];                 // (c, s) of the pair containing index x
+  __shared__ int8_t partner[kMaxRitz][kMaxRitz];     // [round][x]
+  __shared__ double red_off[kMaxRitz], red_tot[kMaxRitz];
+  __shared__ float row_sum[kMaxRitz], row_lam[kMaxRitz];
   __shared__ int go_on;
   const int tid = threadIdx.x;
   const int i = tid / kMaxRitz, j = tid % kMaxRitz;
   const bool mine = i < l && j < l;
   const int m = (l + 1) & ~1;   // even count; index l is a dummy when l is odd
+  const double bij = mine ? 0.5 * (pr.Gm[i * l + j] + pr.Gm[j * l + i]) : 0.0;
   if (mine) {
-    const double b = 0.5 * (pr.Gm[i * l + j] + pr.Gm[j * l + i]);
-    A[0][i][j] = to_t<T>(b);
-    V[0][i][j] = i == j ? T(1) : T(0);
+    sc.jp.U[i][j] = (float)bij;
+    sc.jp.V[i][j] = i == j ? 1.f : 0.f;
   }
   // circle method: position 0 fixed, the others rotate by one per round
   if (i < m - 1 && j < m) {
@@ -886,17 +1221,80 @@ __global__ void k_ritz_jacobi(const ProblemDev* tab) {
     const int ppos = m - 1 - pos;
     partner[round][x] = (int8_t)(ppos == 0 ? 0 : ((ppos - 1 + round) % (m - 1)) + 1);
   }
+  __syncthreads();
+  jacobi_pairs(sc.jp, l, 8);
+  if (mine) V[0][i][j] = (double)sc.jp.V[i][j];
+  __syncthreads();
+  if (mine) sc.r.B[i][j] = bij;
+  __syncthreads();
+  // two refinement steps; X in V[0], scratch V[1], A[0], A[1]
+  bool usable = true;
+  for (int step = 0; step < 2; ++step) {
+    eig_product<false>(sc.r.B, V[0], A[0], l);          // B X
+    eig_product<true>(V[0], V[0], A[1], l);             // X^T X
+    __syncthreads();
+    eig_product<true>(V[0], A[0], V[1], l);             // S = X^T B X
+    __syncthreads();
+    if (tid < l) sc.r.lam[tid] = V[1][tid][tid] / A[1][tid][tid];
+    __syncthreads();
+    // the separation below which a pair is left alone: twice the largest row
+    // sum of |S - Lambda| + |Lambda| |R| (FP32 will do for it)
+    const double r = mine ? (i == j ? 1.0 : 0.0) - A[1][i][j] : 0.0;
+    if (i < l) {
+      const float li = fabsf((float)sc.r.lam[i]);
+      float v = mine ? fabsf((float)(V[1][i][j] - (i == j ? sc.r.lam[i] : 0.0))) + li * fabsf((float)r) : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (j == 0) {
+        row_sum[i] = v;
+        row_lam[i] = li;
+      }
+    }
+    __syncthreads();
+    float delta = 0.f, lmax = 0.f;
+    for (int u = 0; u < l; ++u) {
+      delta = fmaxf(delta, row_sum[u]);
+      lmax = fmaxf(lmax, row_lam[u]);
+    }
+    delta *= 2.f;
+    // a start that is no near eigenbasis (values beyond FP32's range, say):
+    // FP64 Jacobi from the beginning
+    if (step == 0 && !(delta <= 1e-2f * lmax)) {
+      usable = false;
+      break;
+    }
+    if (mine) {
+      // E to FP32's relative accuracy: it is the size of the error that this step
+      // removes.  Entries above 1e-4 (close eigenvalues) would cost orthogonality
+      // in second order and are left to the sweeps below.
+      const float gap = (float)(sc.r.lam[j] - sc.r.lam[i]);
+      const float e = (float)(V[1][i][j] + sc.r.lam[j] * r) / gap;
+      A[0][i][j] = i != j && fabsf(gap) > delta && fabsf(e) < 1e-4f ? (double)e : 0.5 * r;
+    }
+    __syncthreads();
+    eig_product<false>(V[0], A[0], V[1], l);            // X E
+    __syncthreads();
+    if (mine) V[0][i][j] += V[1][i][j];
+    __syncthreads();
+  }
+  if (usable) {
+    eig_product<false>(sc.r.B, V[0], A[1], l);
+    __syncthreads();
+    eig_product<true>(V[0], A[1], A[0], l);             // X^T B X
+  } else if (mine) {
+    A[0][i][j] = bij;
+    V[0][i][j] = i == j ? 1.0 : 0.0;
+  }
   int cur = 0;
   __syncthreads();
-  // cyclic Jacobi converges quadratically; six sweeps reach FP32 rounding for
-  // l <= 32 (the Ritz pairs only shape the preconditioner)
-  const int max_sweeps = sizeof(T) == 4 ? 6 : 30;
-  const T eps = sizeof(T) == 4 ? T(1e-11) : T(1e-30);
+  // off-diagonal norm within 1e-14 of the whole: done, usually before the first sweep
+  const int max_sweeps = 30;
+  const double eps = 1e-28;
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     {
       // off-diagonal and total squared norms: warp i holds row i
-      T v = mine ? A[cur][i][j] * A[cur][i][j] : T(0);
-      T o = (mine && i != j) ? v : T(0);
+      double v = mine ? A[cur][i][j] * A[cur][i][j] : 0.0;
+      double o = (mine && i != j) ? v : 0.0;
 #pragma unroll
       for (int sh = 16; sh > 0; sh >>= 1) {
         v += __shfl_xor_sync(0xffffffffu, v, sh);
@@ -905,7 +1303,7 @@ __global__ void k_ritz_jacobi(const ProblemDev* tab) {
       if (j == 0) { red_tot[i] = v; red_off[i] = o; }
       __syncthreads();
       if (tid < 32) {
-        T to = red_tot[tid], of = red_off[tid];
+        double to = red_tot[tid], of = red_off[tid];
 #pragma unroll
         for (int sh = 16; sh > 0; sh >>= 1) {
           to += __shfl_xor_sync(0xffffffffu, to, sh);
@@ -920,30 +1318,30 @@ __global__ void k_ritz_jacobi(const ProblemDev* tab) {
       if (tid < l) {
         const int x = tid, y = partner[round][x];
         if (x < y && y < l) {
-          T c, s;
-          jacobi_rotation<T>(A[cur][x][x], A[cur][y][y], A[cur][x][y], c, s);
+          double c, s;
+          jacobi_rotation(A[cur][x][x], A[cur][y][y], A[cur][x][y], c, s);
           cs[x][0] = c; cs[x][1] = s;
           cs[y][0] = c; cs[y][1] = s;
         } else if (y >= l) {
-          cs[x][0] = T(1); cs[x][1] = T(0);
+          cs[x][0] = 1.0; cs[x][1] = 0.0;
         }
       }
       __syncthreads();
       if (mine) {
         // coefficients of row/column index u: new_u = al * X_p + be * X_q for its pair (p < q)
-        auto coef = [&](int u, int& p, int& q, T& al, T& be) {
+        auto coef = [&](int u, int& p, int& q, double& al, double& be) {
           const int v2 = partner[round][u];
-          if (v2 >= l) { p = u; q = u; al = T(1); be = T(0); return; }
-          const T c = cs[u][0], s = cs[u][1];
+          if (v2 >= l) { p = u; q = u; al = 1.0; be = 0.0; return; }
+          const double c = cs[u][0], s = cs[u][1];
           if (u < v2) { p = u; q = v2; al = c; be = -s; }
           else { p = v2; q = u; al = s; be = c; }
         };
         int pi, qi, pj, qj;
-        T ai, bi, aj, bj;
+        double ai, bi, aj, bj;
         coef(i, pi, qi, ai, bi);
         coef(j, pj, qj, aj, bj);
-        const T(*Ac)[kMaxRitz + 1] = A[cur];
-        T nv;
+        const double (*Ac)[kMaxRitz + 1] = A[cur];
+        double nv;
         if (pi == qi && pj == qj) nv = Ac[i][j];
         else if (pi == qi) nv = aj * Ac[i][pj] + bj * Ac[i][qj];
         else if (pj == qj) nv = ai * Ac[pi][j] + bi * Ac[qi][j];
@@ -957,164 +1355,46 @@ __global__ void k_ritz_jacobi(const ProblemDev* tab) {
   }
   // descending order: rank of each diagonal entry
   if (tid < l) {
-    const T di = A[cur][tid][tid];
+    const double di = A[cur][tid][tid];
     int rank = 0;
     for (int u = 0; u < l; ++u) {
-      const T du = A[cur][u][u];
+      const double du = A[cur][u][u];
       rank += (du > di) || (du == di && u < tid);
     }
-    pr.ev[rank] = (double)di;
-    for (int u = 0; u < l; ++u) pr.Rm[u * l + rank] = (double)V[cur][u][tid];
+    pr.ev[rank] = di;
+    for (int u = 0; u < l; ++u) pr.Rm[u * l + rank] = V[cur][u][tid];
   }
 }
 
-// One-sided (Hestenes) cyclic Jacobi for the FP32 path: one warp per column
-// pair of a round (lane i holds row i), U = B, V = I initially; each round
-// rotates its pairs so that their columns of U become orthogonal.  At
-// convergence B V = U with orthogonal columns, so the columns of V are
-// eigenvectors and lambda_c = v_c . u_c (sign kept).  Squared column norms are
-// carried through the rotations (alpha' = alpha - t g, beta' = beta + t g) and
-// recomputed once per sweep.
-__global__ void k_ritz_jacobi_pairs(const ProblemDev* tab) {
-  const ProblemDev& pr = tab[blockIdx.x];
-  const int l = pr.l;
-  if (l <= 0) return;
-  __shared__ float U[kMaxRitz][kMaxRitz + 1], V[kMaxRitz][kMaxRitz + 1];
-  __shared__ float nrm[kMaxRitz];
-  __shared__ float s_scale;
-  __shared__ int8_t pair_p[kMaxRitz][kMaxRitz / 2], pair_q[kMaxRitz][kMaxRitz / 2];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  for (int e = tid; e < l * l; e += blockDim.x) {
-    const int i = e / l, c = e % l;
-    U[i][c] = (float)(0.5 * (pr.Gm[i * l + c] + pr.Gm[c * l + i]));
-    V[i][c] = i == c ? 1.f : 0.f;
-  }
-  const int m = (l + 1) & ~1, npairs = m / 2;
-  // round-robin schedule (circle method): slot 0 fixed, slot s > 0 holds
-  // ((s - 1 + round) mod (m - 1)) + 1; pair w of a round joins slots w and m - 1 - w
-  for (int e = tid; e < (m - 1) * npairs; e += blockDim.x) {
-    const int round = e / npairs, w = e % npairs;
-    const int s1 = w, s2 = m - 1 - w;
-    int p = s1 == 0 ? 0 : ((s1 - 1 + round) % (m - 1)) + 1;
-    int q = ((s2 - 1 + round) % (m - 1)) + 1;
-    if (p > q) { const int x = p; p = q; q = x; }
-    pair_p[round][w] = (int8_t)p;
-    pair_q[round][w] = (int8_t)q;
-  }
-  __syncthreads();
-  auto refresh_norms = [&]() {
-    for (int c = warp; c < l; c += nw) {
-      const float u = lane < l ? U[lane][c] : 0.f;
-      float a = u * u;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-      if (lane == 0) nrm[c] = a;
-    }
-  };
-  refresh_norms();
-  __syncthreads();
-  if (tid == 0) {
-    float mx = 0.f;
-    for (int c = 0; c < l; ++c) mx = fmaxf(mx, nrm[c]);
-    s_scale = mx;
-  }
-  __syncthreads();
-  // a pair stays unconverged while the cosine of its columns exceeds 1e-5 and
-  // |u_p . u_q| exceeds 2e-6 of the largest squared column norm (below that it
-  // is FP32 rounding noise of the small columns)
-  const float gabs = 2e-6f * s_scale;
-  // four sweeps: cyclic Jacobi is quadratically convergent, and the Ritz pairs
-  // only shape the preconditioner (a round costs a few hundred cycles of
-  // dependent latency, so the sweep count is the cost)
-  for (int sweep = 0; sweep < 4; ++sweep) {
-    int busy = 0;
-    for (int round = 0; round < m - 1; ++round) {
-      for (int w = warp; w < npairs; w += nw) {
-        const int p = pair_p[round][w], q = pair_q[round][w];
-        if (q >= l) continue;
-        const float up = lane < l ? U[lane][p] : 0.f, uq = lane < l ? U[lane][q] : 0.f;
-        float g = up * uq;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        const float al = nrm[p], be = nrm[q];
-        if (g == 0.f) continue;
-        busy |= fabsf(g) > gabs && fabsf(g) > 1e-5f * sqrtf(al * be);
-        // rotation from approximate reciprocals and roots: any orthogonal rotation
-        // keeps B V = U exact; these only change how fast the pair converges
-        const float zeta = __fdividef(be - al, 2.f * g);
-        const float z2 = fmaf(zeta, zeta, 1.f);
-        const float tt = copysignf(1.f, zeta) * __fdividef(1.f, fabsf(zeta) + z2 * rsqrtf(z2));
-        const float cs = rsqrtf(fmaf(tt, tt, 1.f)), sn = cs * tt;
-        if (lane < l) {
-          U[lane][p] = cs * up - sn * uq;
-          U[lane][q] = sn * up + cs * uq;
-          const float vp = V[lane][p], vq = V[lane][q];
-          V[lane][p] = cs * vp - sn * vq;
-          V[lane][q] = sn * vp + cs * vq;
-        }
-        if (lane == 0) {
-          nrm[p] = fmaxf(al - tt * g, 0.f);
-          nrm[q] = fmaxf(be + tt * g, 0.f);
-        }
-      }
-      __syncthreads();
-    }
-    refresh_norms();
-    if (!__syncthreads_or(busy)) break;
-  }
-  // eigenvalues (Rayleigh quotients) and the descending order
-  __shared__ float lam[kMaxRitz];
-  for (int c = warp; c < l; c += nw) {
-    float a = lane < l ? V[lane][c] * U[lane][c] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) lam[c] = a;
-  }
-  __syncthreads();
-  if (tid < l) {
-    const float di = lam[tid];
-    int rank = 0;
-    for (int u = 0; u < l; ++u) rank += (lam[u] > di) || (lam[u] == di && u < tid);
-    pr.ev[rank] = (double)di;
-    for (int u = 0; u < l; ++u) pr.Rm[u * l + rank] = (double)V[u][tid];
-  }
-}
-
-// Phi = basis V_k, C Phi = image V_k (stored in T), theta = top k eigenvalues.
+// Phi = basis V_k, C Phi = image V_k (stored in T), theta = top k eigenvalues;
+// one thread per entry of both (a thread per row ran 2 l k dependent steps on a
+// couple of SMs: 25 us in FP64 at 60 rows, 50 us at 1024).
+constexpr int kVecEntries = 128;
 template <typename T>
-__global__ void k_ritz_vectors(const ProblemDev* tab, int basis) {
+__global__ void __launch_bounds__(kVecEntries) k_ritz_vectors(const ProblemDev* tab, int basis) {
   const ProblemDev& pr = tab[blockIdx.y];
   const int l = pr.l, k = pr.kR;
-  if (k <= 0) return;
+  const int64_t e0 = (int64_t)blockIdx.x * kVecEntries, total = pr.d * k;
+  if (k <= 0 || e0 >= total) return;
   __shared__ T Vk[kMaxRitz][kMaxK];
-  for (int e = threadIdx.x; e < l * k; e += blockDim.x) Vk[e / k][e % k] = to_t<T>(pr.Rm[(e / k) * l + e % k]);
+  for (int e = threadIdx.x; e < l * k; e += kVecEntries) Vk[e / k][e % k] = to_t<T>(pr.Rm[(e / k) * l + e % k]);
   __syncthreads();
-  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= pr.d) return;
-  const T* Qb = ritz_buf<T>(pr, basis);
-  const T* Pb = ritz_buf<T>(pr, 1 - basis);
-  T* Phi = tp<T>(pr.Phi);
-  T* CPhi = tp<T>(pr.CPhi);
-  T q[kMaxRitz], c[kMaxRitz];
-#pragma unroll
-  for (int i = 0; i < kMaxRitz; ++i) {
-    q[i] = i < l ? Qb[a * l + i] : T(0);
-    c[i] = i < l ? Pb[a * l + i] : T(0);
-  }
-  for (int j = 0; j < k; ++j) {
+  const int64_t e = e0 + threadIdx.x;
+  if (e < total) {
+    const int64_t a = e / k;
+    const int j = (int)(e - a * k);
+    const T* q = ritz_buf<T>(pr, basis) + a * l;
+    const T* c = ritz_buf<T>(pr, 1 - basis) + a * l;
     T ph = T(0), cp = T(0);
-#pragma unroll
-    for (int i = 0; i < kMaxRitz; ++i) {
-      if (i < l) {
-        ph += q[i] * Vk[i][j];
-        cp += c[i] * Vk[i][j];
-      }
+#pragma unroll 4
+    for (int i = 0; i < l; ++i) {
+      ph += q[i] * Vk[i][j];
+      cp += c[i] * Vk[i][j];
     }
-    Phi[a * k + j] = ph;
-    CPhi[a * k + j] = cp;
+    tp<T>(pr.Phi)[e] = ph;
+    tp<T>(pr.CPhi)[e] = cp;
+    if (a == 0) pr.theta[j] = pr.ev[j];
   }
-  if (a == 0)
-    for (int j = 0; j < k; ++j) pr.theta[j] = pr.ev[j];
 }
 
 // Gram matrices of the stored Phi and A = C Phi in FP64:
@@ -1155,6 +1435,8 @@ static void launch_ritz_t(const ProblemTable& tab, const ProblemDev* dtab, cudaS
   if (lmax <= 0 || kmax <= 0) return;
   const dim3 gdl((unsigned)((dl + 255) / 256), tab.count);
   const dim3 gd((unsigned)((dmax + 255) / 256), tab.count);
+  const dim3 go((unsigned)((dl + kOrthEntries - 1) / kOrthEntries), tab.count);
+  const dim3 gv((unsigned)((dmax * kmax + kVecEntries - 1) / kVecEntries), tab.count);
   const dim3 gdw((unsigned)((dmax * 32 + 255) / 256), tab.count);   // one warp per row
   const dim3 gll((unsigned)(lmax * lmax), tab.count);
   int cur = 0;   // buffer holding the current basis candidate
@@ -1166,11 +1448,15 @@ static void launch_ritz_t(const ProblemTable& tab, const ProblemDev* dtab, cudaS
     k_ritz_matvec<T><<<gdw, 256, 0, st>>>(dtab, cur);
     note_launches(1);
   };
+  auto orth = [&](int x) {
+    if constexpr (sizeof(T) == 8) k_ritz_orth64<<<go, kOrthThreads, 0, st>>>(dtab, x);
+    else k_ritz_orth<T><<<gd, 256, 0, st>>>(dtab, x);
+  };
   auto orth2 = [&](int x) {   // orthonormalize buf[x] in place (scratch: the other buffer)
     k_ritz_gram<T><<<gll, 256, 0, st>>>(dtab, x, x, 1);
-    k_ritz_orth<T><<<gd, 256, 0, st>>>(dtab, x);          // buf[1-x] = buf[x] R^-1
+    orth(x);                                              // buf[1-x] = buf[x] R^-1
     k_ritz_gram<T><<<gll, 256, 0, st>>>(dtab, 1 - x, 1 - x, 1);
-    k_ritz_orth<T><<<gd, 256, 0, st>>>(dtab, 1 - x);      // buf[x] = buf[1-x] R^-1
+    orth(1 - x);                                          // buf[x] = buf[1-x] R^-1
     note_launches(4);
   };
   k_ritz_omega<T><<<gdl, 256, 0, st>>>(dtab);               // buf0 = Omega
@@ -1186,10 +1472,11 @@ static void launch_ritz_t(const ProblemTable& tab, const ProblemDev* dtab, cudaS
   matvec();                                                 // image in buf[1-cur]
   k_ritz_gram<T><<<gll, 256, 0, st>>>(dtab, cur, 1 - cur, 0);   // Gm = Q^T (C Q)
   if (sizeof(T) == 4) k_ritz_jacobi_pairs<<<tab.count, 32 * ((lmax + 1) / 2), 0, st>>>(dtab);
-  else k_ritz_jacobi<T><<<tab.count, kMaxRitz * kMaxRitz, 0, st>>>(dtab);
-  k_ritz_vectors<T><<<gd, 256, 0, st>>>(dtab, cur);
+  else k_ritz_jacobi<<<tab.count, kEigThreads, 0, st>>>(dtab);
+  k_ritz_vectors<T><<<gv, kVecEntries, 0, st>>>(dtab, cur);
   k_ritz_grams<T><<<dim3(3 * kmax * kmax, tab.count), 256, 0, st>>>(dtab);
   note_launches(4);
+  if (!tile) launch_pcg_phit(tab, dtab, st);
 }
 
 void launch_ritz(const ProblemTable& tab, const ProblemDev* dtab, cudaStream_t st) {
