@@ -20,6 +20,8 @@
 // the stencil and the network), a fixed-order reduction over samples, Adam.
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "info_esrf.h"
 #include "info_esrf_stages.h"
@@ -141,146 +143,256 @@ __global__ void k_learn_coef(const float* theta, int nshift, const float* feat, 
   for (int j = 1; j < kLearnOut; ++j) coef[(int64_t)s * kLearnOut + j] = out[j] * rs;
 }
 
+// What the parameter gradient of one sample is made of: every entry is the
+// product of two of these floats (k_learn_reduce).
+constexpr int kRecH1 = 0, kRecH2 = kRecH1 + kHid, kRecG2 = kRecH2 + kHid, kRecG1 = kRecG2 + kHid,
+              kRecOut = kRecG1 + kHid, kRecPhi = kRecOut + kLearnOut, kRecOne = kRecPhi + kIn, kRec = 152;
+static_assert(kRecOne < kRec && kRec <= kLearnParams, "record layout");
+
+// h1, h2: hidden layers; ga2, ga1: gradients before their activations; gout:
+// gradient of the network's output.
+__device__ __forceinline__ void write_record(float* r, int tid, const float* h1, const float* h2, const float* ga2,
+                                             const float* ga1, const float* gout, const float* phi) {
+  if (tid < kHid) {
+    r[kRecH1 + tid] = h1[tid];
+    r[kRecH2 + tid] = h2[tid];
+    r[kRecG2 + tid] = ga2[tid];
+    r[kRecG1 + tid] = ga1[tid];
+    if (tid < kLearnOut) r[kRecOut + tid] = gout[tid];
+    if (tid < kIn) r[kRecPhi + tid] = phi[tid];
+    if (tid == 0) r[kRecOne] = 1.f;
+  }
+}
+
+// Sum over a quad of lanes (each lane returns it).
+__device__ __forceinline__ float quad_sum(float v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
+
 // ---------------------------------------------------------------------------
-// Loss and gradient, one block per sample.  Vectors in dynamic shared memory.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads)
-k_learn_loss_grad(const float* theta, int nsamp, int64_t d, const float* feat, const float* V, const float* Y,
-                  const float* Z, float* G, double* sample_loss) {
+// Loss and gradient, one block per sample at a time.
+//
+// With u = S y and e = a z + S^T u - v, the derivative of ||e||^2 / 2 by tap j is
+// e^T S_j^T S y + (S e)^T S_j y = sum_k w_k (X(k - j) + X(j - k)) with the cross-
+// correlations X(m) = sum_a e_a y_{a + m}: 17 float-float sums of
+// e_a (y_{a+m} + y_{a-m}), m = 0..16, in place of the 34 sums of e against
+// shifted u and of S e against shifted y (and S e is not formed).
+//
+// A thread owns four consecutive rows, so that a window of 20 (stencils) or 36
+// (correlations) values is read into registers with 16-byte loads; y and u lie
+// in shared memory with their periodic halos written out, so no index is
+// wrapped in the loops.  The sums dominate (11 FP32 instructions each): issue-
+// bound.  Network in shared memory, four lanes per unit; theta is staged once per block.
+constexpr int kLgThreads = 128;
+constexpr int kLgBlocks = 4;   // resident per SM (registers)
+constexpr int kLgSums = 3 + kLearnTaps;   // ||v||^2, ||e||^2, e.z, X(m) + X(-m)
+static_assert(kLgThreads == 4 * kHid && kLgSums <= 32, "layout");
+
+__global__ void __launch_bounds__(kLgThreads, kLgBlocks)
+k_learn_loss_grad(const float* theta, int nsamp, int d, const float* feat, const float* V, const float* Y,
+                  const float* Z, float* rec, double* sample_loss) {
+  constexpr int H = kLearnH;
   extern __shared__ __align__(16) float sm[];
-  float* y = sm;
-  float* z = y + d;
-  float* v = z + d;
-  float* u = v + d;
-  float* e = u + d;
-  float* se = e + d;
-  __shared__ float h1[kHid], h2[kHid], out[kLearnOut], gout[kLearnOut], ga2[kHid], ga1[kHid];
-  __shared__ float phi[kIn];
-  __shared__ double red_scratch[2 * (3 + 2 * kLearnTaps) * (kThreads / 32)];
-  const int s = blockIdx.x;
-  const int tid = threadIdx.x;
-  if (s >= nsamp) return;
-  const float* th = theta;
-  if (tid < kIn) phi[tid] = feat[(int64_t)s * kIn + tid];
-  __syncthreads();
-  if (tid < kHid) {
-    float a = th[kOB1 + tid];
-    for (int c = 0; c < kIn; ++c) a = fmaf(th[kOW1 + tid * kIn + c], phi[c], a);
-    h1[tid] = tanhf(a);
-  }
-  __syncthreads();
-  if (tid < kHid) {
-    float a = th[kOB2 + tid];
-    for (int j = 0; j < kHid; ++j) a = fmaf(th[kOW2 + tid * kHid + j], h1[j], a);
-    h2[tid] = tanhf(a);
-  }
-  __syncthreads();
-  if (tid < kLearnOut) {
-    float a = th[kOB3 + tid];
-    for (int j = 0; j < kHid; ++j) a = fmaf(th[kOW3 + tid * kHid + j], h2[j], a);
-    out[tid] = a;
-  }
-  for (int64_t a = tid; a < d; a += blockDim.x) {
-    y[a] = Y[s * d + a];
-    z[a] = Z[s * d + a];
-    v[a] = V[s * d + a];
-  }
+  const int d4 = (d + 3) & ~3;
+  float* yx = sm;                    // y_{a}, a = -2h .. d4 + 2h - 1, at a + 2h
+  float* ux = sm + d4 + 4 * H;       // u_{a}, a = -h .. d4 + h - 1, at a + h
+  __shared__ float W1[kHid * kIn], B1[kHid], W2[kHid][kHid + 1], B2[kHid], W3[kLearnOut][kHid + 1], B3[kLearnOut];
+  __shared__ float h1[kHid], h2[kHid], out[kLearnOut], gout[kLearnOut], ga2[kHid], ga1[kHid], phi[kIn];
   __shared__ float wsc[kLearnTaps];
-  const float rs = expf(-2.5f * phi[0]);       // sigma^-1/2
-  if (tid < kLearnTaps) wsc[tid] = out[1 + tid] * rs;
-  __syncthreads();
-  const float sa = expf(out[0]) * rs * rs;
-  const float* w = wsc;
-  // u = S y
-  for (int64_t a = tid; a < d; a += blockDim.x) {
-    float acc = 0.f;
-    for (int j = 0; j < kLearnTaps; ++j) {
-      int64_t b = (a + j - kLearnH) % d;
-      if (b < 0) b += d;
-      acc = fmaf(w[j], y[b], acc);
-    }
-    u[a] = acc;
+  __shared__ float part[kLgThreads / 32][32][2];
+  __shared__ double tot[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int unit = tid >> 2, sub = tid & 3;   // four lanes per hidden unit
+  for (int p = tid; p < kLearnParams; p += kLgThreads) {
+    const float t = theta[p];
+    if (p < kOB1) W1[p] = t;
+    else if (p < kOW2) B1[p - kOB1] = t;
+    else if (p < kOB2) W2[(p - kOW2) / kHid][(p - kOW2) % kHid] = t;
+    else if (p < kOW3) B2[p - kOB2] = t;
+    else if (p < kOB3) W3[(p - kOW3) / kHid][(p - kOW3) % kHid] = t;
+    else B3[p - kOB3] = t;
   }
-  __syncthreads();
-  // e = a z + S^T u - v
-  for (int64_t a = tid; a < d; a += blockDim.x) {
-    float acc = 0.f;
-    for (int j = 0; j < kLearnTaps; ++j) {
-      int64_t b = (a - (j - kLearnH)) % d;
-      if (b < 0) b += d;
-      acc = fmaf(w[j], u[b], acc);
+  // 16-byte loads where every sample's row starts on a 16-byte boundary
+  const bool vec = d % 4 == 0 && ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(Z)) & 15) == 0;
+  auto load4 = [&](const float* p, int a0) {
+    if (vec) return *reinterpret_cast<const float4*>(p + a0);
+    return make_float4(p[a0], a0 + 1 < d ? p[a0 + 1] : 0.f, a0 + 2 < d ? p[a0 + 2] : 0.f,
+                       a0 + 3 < d ? p[a0 + 3] : 0.f);
+  };
+  for (int s = blockIdx.x; s < nsamp; s += gridDim.x) {
+    const float* y = Y + (int64_t)s * d;
+    const float* z = Z + (int64_t)s * d;
+    const float* v = V + (int64_t)s * d;
+    for (int i = tid; i < d4 + 4 * H; i += kLgThreads) {
+      int a = i - 2 * H;
+      if (a < 0 || a >= d) {   // halo, and the rows that fill the last four
+        a %= d;
+        if (a < 0) a += d;
+      }
+      yx[i] = y[a];
     }
-    e[a] = sa * z[a] + acc - v[a];
-  }
-  __syncthreads();
-  // S e
-  for (int64_t a = tid; a < d; a += blockDim.x) {
-    float acc = 0.f;
-    for (int j = 0; j < kLearnTaps; ++j) {
-      int64_t b = (a + j - kLearnH) % d;
-      if (b < 0) b += d;
-      acc = fmaf(w[j], e[b], acc);
+    float4 zn = make_float4(0.f, 0.f, 0.f, 0.f), vn = zn;   // rows 4 tid .. of z and v, a run ahead
+    if (4 * tid < d) {
+      zn = load4(z, 4 * tid);
+      vn = load4(v, 4 * tid);
     }
-    se[a] = acc;
-  }
-  __syncthreads();
-  // sums: ||v||^2, ||e||^2, e.z, and per tap c1 = sum e_a u_{a-delta}, c2 = sum (Se)_b y_{b+delta}
-  constexpr int NV = 3 + 2 * kLearnTaps;
-  DotAcc<float> acc[NV];
-  for (int64_t a = tid; a < d; a += blockDim.x) {
-    acc[0].add_prod(v[a], v[a]);
-    acc[1].add_prod(e[a], e[a]);
-    acc[2].add_prod(e[a], z[a]);
+    if (tid < kIn) phi[tid] = feat[(int64_t)s * kIn + tid];
+    __syncthreads();
+    // network forward
+    {
+      const float a = quad_sum(W1[unit * kIn + sub] * phi[sub]);
+      if (sub == 0) h1[unit] = tanhf(a + B1[unit]);
+    }
+    __syncthreads();
+    {
+      float a = 0.f;
 #pragma unroll
-    for (int j = 0; j < kLearnTaps; ++j) {
-      const int dl = j - kLearnH;
-      int64_t am = (a - dl) % d;
-      if (am < 0) am += d;
-      int64_t bp = (a + dl) % d;
-      if (bp < 0) bp += d;
-      acc[3 + j].add_prod(e[a], u[am]);
-      acc[3 + kLearnTaps + j].add_prod(se[a], y[bp]);
+      for (int j = 0; j < kHid / 4; ++j) a = fmaf(W2[unit][sub * (kHid / 4) + j], h1[sub * (kHid / 4) + j], a);
+      a = quad_sum(a);
+      if (sub == 0) h2[unit] = tanhf(a + B2[unit]);
     }
+    __syncthreads();
+    const float rs = expf(-2.5f * phi[0]);       // sigma^-1/2
+    {
+      float a = 0.f;
+      if (unit < kLearnOut)
+#pragma unroll
+        for (int j = 0; j < kHid / 4; ++j) a = fmaf(W3[unit][sub * (kHid / 4) + j], h2[sub * (kHid / 4) + j], a);
+      a = quad_sum(a);
+      if (unit < kLearnOut && sub == 0) {
+        a += B3[unit];
+        out[unit] = a;
+        if (unit > 0) wsc[unit - 1] = a * rs;
+      }
+    }
+    __syncthreads();
+    const float sa = expf(out[0]) * rs * rs;
+    // u = S y, also on the halo
+    for (int a0 = 4 * tid - H; a0 < d4 + H; a0 += 4 * kLgThreads) {
+      float win[4 + 2 * H];
+#pragma unroll
+      for (int i = 0; i < 1 + H / 2; ++i) {
+        const float4 t = *reinterpret_cast<const float4*>(yx + a0 + H + 4 * i);   // from y_{a0 - h} on
+        win[4 * i] = t.x; win[4 * i + 1] = t.y; win[4 * i + 2] = t.z; win[4 * i + 3] = t.w;
+      }
+      float acc[4] = {};
+#pragma unroll
+      for (int j = 0; j < kLearnTaps; ++j) {
+        const float w = wsc[j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = fmaf(w, win[i + j], acc[i]);
+      }
+      *reinterpret_cast<float4*>(ux + a0 + H) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    }
+    __syncthreads();
+    // e = a z + S^T u - v and the sums
+    DotAcc<float> acc[kLgSums];
+    for (int a0 = 4 * tid; a0 < d; a0 += 4 * kLgThreads) {
+      const float zr[4] = {zn.x, zn.y, zn.z, zn.w}, vr[4] = {vn.x, vn.y, vn.z, vn.w};
+      if (a0 + 4 * kLgThreads < d) {
+        zn = load4(z, a0 + 4 * kLgThreads);
+        vn = load4(v, a0 + 4 * kLgThreads);
+      }
+      float e[4] = {};
+      {
+        float win[4 + 2 * H];   // u from a0 - h on
+#pragma unroll
+        for (int i = 0; i < 1 + H / 2; ++i) {
+          const float4 t = *reinterpret_cast<const float4*>(ux + a0 + 4 * i);
+          win[4 * i] = t.x; win[4 * i + 1] = t.y; win[4 * i + 2] = t.z; win[4 * i + 3] = t.w;
+        }
+#pragma unroll
+        for (int j = 0; j < kLearnTaps; ++j) {
+          const float w = wsc[j];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) e[i] = fmaf(w, win[i + 2 * H - j], e[i]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        e[i] = a0 + i < d ? sa * zr[i] + e[i] - vr[i] : 0.f;   // z and v are zero there as well
+        acc[0].add_prod(vr[i], vr[i]);
+        acc[1].add_prod(e[i], e[i]);
+        acc[2].add_prod(e[i], zr[i]);
+      }
+      float win[4 + 4 * H];   // y from a0 - 2h on
+#pragma unroll
+      for (int i = 0; i < 1 + H; ++i) {
+        const float4 t = *reinterpret_cast<const float4*>(yx + a0 + 4 * i);
+        win[4 * i] = t.x; win[4 * i + 1] = t.y; win[4 * i + 2] = t.z; win[4 * i + 3] = t.w;
+      }
+#pragma unroll
+      for (int m = 0; m < kLearnTaps; ++m)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[3 + m].add_prod(e[i], win[i + 2 * H + m] + win[i + 2 * H - m]);
+    }
+    // reduce-scatter of the float-float sums over the warp (lane l ends with sum l), then over the warps
+    {
+      float hi[32], lo[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        hi[i] = i < kLgSums ? acc[i].hi : 0.f;
+        lo[i] = i < kLgSums ? acc[i].lo : 0.f;
+      }
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < off; ++i) {
+          const float sh = __shfl_xor_sync(0xffffffffu, up ? hi[i] : hi[i + off], off);
+          const float sl = __shfl_xor_sync(0xffffffffu, up ? lo[i] : lo[i + off], off);
+          hi[i] = up ? hi[i + off] : hi[i];
+          lo[i] = up ? lo[i + off] : lo[i];
+          ff_merge(hi[i], lo[i], sh, sl);
+        }
+      }
+      part[warp][lane][0] = hi[0];
+      part[warp][lane][1] = lo[0];
+    }
+    __syncthreads();
+    if (warp == 0) {
+      float hi = part[0][lane][0], lo = part[0][lane][1];
+#pragma unroll
+      for (int w = 1; w < kLgThreads / 32; ++w) ff_merge(hi, lo, part[w][lane][0], part[w][lane][1]);
+      tot[lane] = (double)hi + (double)lo;
+    }
+    __syncthreads();
+    const double vv = tot[0] > 0 ? tot[0] : 1.0;
+    const double scale = 2.0 / ((double)nsamp * vv);
+    {
+      // tap j = unit: sum_k w_k (X(k - j) + X(j - k)); X(0) + X(0) is what sum 0 holds
+      double g = 0.0;
+      if (unit < kLearnTaps)
+        for (int k = sub; k < kLearnTaps; k += 4) g += (double)wsc[k] * tot[3 + (k < unit ? unit - k : k - unit)];
+      g += __shfl_xor_sync(0xffffffffu, g, 1);
+      g += __shfl_xor_sync(0xffffffffu, g, 2);
+      if (unit < kLearnTaps && sub == 0) gout[1 + unit] = (float)(scale * g) * rs;
+      if (tid == kLgThreads - 1) {
+        sample_loss[s] = tot[1] / vv / (double)nsamp;
+        gout[0] = (float)(scale * (double)sa * tot[2]);
+      }
+    }
+    __syncthreads();
+    // backward through the network
+    {
+      float g = 0.f;
+      for (int o = sub; o < kLearnOut; o += 4) g = fmaf(W3[o][unit], gout[o], g);
+      g = quad_sum(g);
+      if (sub == 0) ga2[unit] = g * (1.f - h2[unit] * h2[unit]);
+    }
+    __syncthreads();
+    {
+      float g = 0.f;
+#pragma unroll
+      for (int i = 0; i < kHid / 4; ++i) g = fmaf(W2[sub * (kHid / 4) + i][unit], ga2[sub * (kHid / 4) + i], g);
+      g = quad_sum(g);
+      if (sub == 0) ga1[unit] = g * (1.f - h1[unit] * h1[unit]);
+    }
+    __syncthreads();
+    write_record(rec + (int64_t)s * kRec, tid, h1, h2, ga2, ga1, gout, phi);
+    __syncthreads();   // the next sample overwrites phi and the layers
   }
-  double sums[NV];
-  block_sum<NV>(acc, sums, red_scratch);
-  const double vv = sums[0] > 0 ? sums[0] : 1.0;
-  const double scale = 2.0 / ((double)nsamp * vv);
-  if (tid == 0) {
-    sample_loss[s] = sums[1] / vv / (double)nsamp;
-    gout[0] = (float)(scale * (double)sa * sums[2]);
-  }
-  if (tid < kLearnTaps) gout[1 + tid] = (float)(scale * (sums[3 + tid] + sums[3 + kLearnTaps + tid])) * rs;
-  __syncthreads();
-  // backward through the network
-  float* g = G + (int64_t)s * kLearnParams;
-  for (int e2 = tid; e2 < kLearnOut * kHid; e2 += blockDim.x) {
-    const int o = e2 / kHid, j = e2 % kHid;
-    g[kOW3 + e2] = gout[o] * h2[j];
-  }
-  if (tid < kLearnOut) g[kOB3 + tid] = gout[tid];
-  if (tid < kHid) {
-    float gh = 0.f;
-    for (int o = 0; o < kLearnOut; ++o) gh = fmaf(th[kOW3 + o * kHid + tid], gout[o], gh);
-    ga2[tid] = gh * (1.f - h2[tid] * h2[tid]);
-  }
-  __syncthreads();
-  for (int e2 = tid; e2 < kHid * kHid; e2 += blockDim.x) {
-    const int i = e2 / kHid, j = e2 % kHid;
-    g[kOW2 + e2] = ga2[i] * h1[j];
-  }
-  if (tid < kHid) {
-    g[kOB2 + tid] = ga2[tid];
-    float gh = 0.f;
-    for (int i = 0; i < kHid; ++i) gh = fmaf(th[kOW2 + i * kHid + tid], ga2[i], gh);
-    ga1[tid] = gh * (1.f - h1[tid] * h1[tid]);
-  }
-  __syncthreads();
-  for (int e2 = tid; e2 < kHid * kIn; e2 += blockDim.x) {
-    const int i = e2 / kIn, c = e2 % kIn;
-    g[kOW1 + e2] = ga1[i] * phi[c];
-  }
-  if (tid < kHid) g[kOB1 + tid] = ga1[tid];
 }
 
 // ---------------------------------------------------------------------------
@@ -311,7 +423,7 @@ __device__ __forceinline__ void lat_points(int a, int Lx, int Ly, const int (&of
 
 __global__ void __launch_bounds__(kThreads)
 k_learn_loss_grad_lat(const float* theta, int nsamp, int Lx, int Ly, const float* feat, const float* V,
-                      const float* Y, const float* Z, float* G, double* sample_loss, float* tmp) {
+                      const float* Y, const float* Z, float* rec, double* sample_loss, float* tmp) {
   __shared__ float h1[kHid], h2[kHid], out[kLearnOut], gout[kLearnOut], ga2[kHid], ga1[kHid];
   __shared__ float phi[kIn];
   __shared__ float wsc[kLatBins];
@@ -410,49 +522,83 @@ k_learn_loss_grad_lat(const float* theta, int nsamp, int Lx, int Ly, const float
   if (tid < kLearnTaps) gout[1 + tid] = (tid < kLatBins && sums[0] > 0) ? (float)(scale * sums[3 + tid]) * rs : 0.f;
   __syncthreads();
   // backward through the network
-  float* g = G + (int64_t)s * kLearnParams;
-  for (int e2 = tid; e2 < kLearnOut * kHid; e2 += blockDim.x) {
-    const int o = e2 / kHid, j = e2 % kHid;
-    g[kOW3 + e2] = gout[o] * h2[j];
-  }
-  if (tid < kLearnOut) g[kOB3 + tid] = gout[tid];
   if (tid < kHid) {
     float gh = 0.f;
     for (int o = 0; o < kLearnOut; ++o) gh = fmaf(th[kOW3 + o * kHid + tid], gout[o], gh);
     ga2[tid] = gh * (1.f - h2[tid] * h2[tid]);
   }
   __syncthreads();
-  for (int e2 = tid; e2 < kHid * kHid; e2 += blockDim.x) {
-    const int i = e2 / kHid, j = e2 % kHid;
-    g[kOW2 + e2] = ga2[i] * h1[j];
-  }
   if (tid < kHid) {
-    g[kOB2 + tid] = ga2[tid];
     float gh = 0.f;
     for (int i = 0; i < kHid; ++i) gh = fmaf(th[kOW2 + i * kHid + tid], ga2[i], gh);
     ga1[tid] = gh * (1.f - h1[tid] * h1[tid]);
   }
   __syncthreads();
-  for (int e2 = tid; e2 < kHid * kIn; e2 += blockDim.x) {
-    const int i = e2 / kIn, c = e2 % kIn;
-    g[kOW1 + e2] = ga1[i] * phi[c];
-  }
-  if (tid < kHid) g[kOB1 + tid] = ga1[tid];
+  write_record(rec + (int64_t)s * kRec, tid, h1, h2, ga2, ga1, gout, phi);
 }
 
-// grad[p] = sum_s G[s][p] in sample order; loss = sum_s sample_loss[s].
-__global__ void k_learn_reduce(int nsamp, const float* G, const double* sample_loss, float* grad, double* loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < kLearnParams) {
-    float acc = 0.f;
-    for (int s = 0; s < nsamp; ++s) acc += G[(int64_t)s * kLearnParams + p];
-    grad[p] = acc;
-  }
-  if (p == 0 && loss) {
+// grad[p] = sum_s left(s, p) right(s, p) over the samples' records, and loss =
+// sum_s sample_loss[s], in a fixed order.  Warp g of a block takes the samples
+// g, g + 32, ... for 32 consecutive parameters (one row of a weight matrix:
+// the left factor is one broadcast, the right factors are coalesced), then the
+// warps' sums are added.  One more block sums the loss.  Latency-bound: 36 samples a
+// thread at 1152, with eight in flight.  (The products used to be written out,
+// 8.3 MB at 1152 samples, and one thread per parameter walked all samples.)
+constexpr int kRedWarps = 32;
+__global__ void __launch_bounds__(32 * kRedWarps) k_learn_reduce(int nsamp, const float* rec,
+                                                                 const double* sample_loss, float* grad,
+                                                                 double* loss) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (blockIdx.x == gridDim.x - 1) {
+    __shared__ double lp[kRedWarps];
+    if (!loss) return;
     double l = 0.0;
-    for (int s = 0; s < nsamp; ++s) l += sample_loss[s];
-    *loss = l;
+    for (int s = threadIdx.x; s < nsamp; s += 32 * kRedWarps) l += sample_loss[s];
+    l = warp_sum(l);
+    if (lane == 0) lp[warp] = l;
+    __syncthreads();
+    if (warp != 0) return;
+    l = warp_sum(lp[lane]);
+    if (lane == 0) *loss = l;
+    return;
   }
+  __shared__ float part[kRedWarps][33];
+  const int p = blockIdx.x * 32 + lane;
+  int left = kRecOne, right = kRecOne;
+  if (p < kOB1) {
+    left = kRecG1 + p / kIn;
+    right = kRecPhi + p % kIn;
+  } else if (p < kOW2) {
+    left = kRecG1 + p - kOB1;
+  } else if (p < kOB2) {
+    left = kRecG2 + (p - kOW2) / kHid;
+    right = kRecH1 + (p - kOW2) % kHid;
+  } else if (p < kOW3) {
+    left = kRecG2 + p - kOB2;
+  } else if (p < kOB3) {
+    left = kRecOut + (p - kOW3) / kHid;
+    right = kRecH2 + (p - kOW3) % kHid;
+  } else if (p < kLearnParams) {
+    left = kRecOut + p - kOB3;
+  }
+  float acc = 0.f;
+#pragma unroll 8
+  for (int s = warp; s < nsamp; s += kRedWarps) {
+    const float* r = rec + (int64_t)s * kRec;
+    acc = fmaf(r[left], r[right], acc);
+  }
+  part[warp][lane] = acc;
+  __syncthreads();
+  float v = part[lane][warp];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const int pw = blockIdx.x * 32 + warp;
+  if (lane == 0 && pw < kLearnParams) grad[pw] = v;
+}
+
+static void launch_learn_reduce(int nsamp, const float* rec, const double* sample_loss, float* grad, double* loss,
+                                cudaStream_t st) {
+  k_learn_reduce<<<(kLearnParams + 31) / 32 + 1, 32 * kRedWarps, 0, st>>>(nsamp, rec, sample_loss, grad, loss);
 }
 
 __global__ void k_learn_adam(float* theta, float* m, float* v, const float* grad, int step, float lr, float b1,
@@ -673,12 +819,19 @@ int info_esrf_learn_loss_grad(const float* theta_dev, int32_t nsamp, int64_t d, 
   const size_t dyn = (size_t)6 * d * sizeof(float);
   if (dyn > 200 * 1024) return INFO_ESRF_ERR_UNSUPPORTED;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  float* G = reinterpret_cast<float*>(scratch_dev);
-  double* sl = reinterpret_cast<double*>(G + (size_t)nsamp * kLearnParams);
+  float* rec = reinterpret_cast<float*>(scratch_dev);
+  double* sl = reinterpret_cast<double*>(rec + (size_t)nsamp * kLearnParams);
   cudaGetLastError();
-  cudaFuncSetAttribute(k_learn_loss_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  k_learn_loss_grad<<<nsamp, kThreads, dyn, st>>>(theta_dev, nsamp, d, feat_dev, V_dev, Y_dev, Z_dev, G, sl);
-  k_learn_reduce<<<(kLearnParams + 255) / 256, 256, 0, st>>>(nsamp, G, sl, grad_dev, loss_dev);
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return INFO_ESRF_ERR_CUDA;
+  const int64_t d4 = (d + 3) / 4 * 4;
+  const size_t smem = (size_t)(2 * d4 + 6 * kLearnH) * sizeof(float);   // y and u with their halos
+  if (smem > 32 * 1024) cudaFuncSetAttribute(k_learn_loss_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int grid = (int)std::min<int64_t>(nsamp, (int64_t)sms * kLgBlocks);
+  k_learn_loss_grad<<<grid, kLgThreads, smem, st>>>(theta_dev, nsamp, (int)d, feat_dev, V_dev, Y_dev, Z_dev, rec, sl);
+  launch_learn_reduce(nsamp, rec, sl, grad_dev, loss_dev, st);
   note_launches(2);
   return cudaGetLastError() == cudaSuccess ? 0 : INFO_ESRF_ERR_CUDA;
 }
@@ -701,15 +854,15 @@ int info_esrf_learn_loss_grad_lattice(const float* theta_dev, int32_t nsamp, int
       (reinterpret_cast<uintptr_t>(scratch_dev) % 16) != 0)
     return INFO_ESRF_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  float* G = reinterpret_cast<float*>(scratch_dev);
-  double* sl = reinterpret_cast<double*>(G + (size_t)nsamp * kLearnParams);
+  float* rec = reinterpret_cast<float*>(scratch_dev);
+  double* sl = reinterpret_cast<double*>(rec + (size_t)nsamp * kLearnParams);
   uintptr_t t = reinterpret_cast<uintptr_t>(sl + nsamp);
   t = (t + 255) & ~(uintptr_t)255;
   float* tmp = reinterpret_cast<float*>(t);
   cudaGetLastError();
-  k_learn_loss_grad_lat<<<nsamp, kThreads, 0, st>>>(theta_dev, nsamp, Lx, Ly, feat_dev, V_dev, Y_dev, Z_dev, G, sl,
+  k_learn_loss_grad_lat<<<nsamp, kThreads, 0, st>>>(theta_dev, nsamp, Lx, Ly, feat_dev, V_dev, Y_dev, Z_dev, rec, sl,
                                                      tmp);
-  k_learn_reduce<<<(kLearnParams + 255) / 256, 256, 0, st>>>(nsamp, G, sl, grad_dev, loss_dev);
+  launch_learn_reduce(nsamp, rec, sl, grad_dev, loss_dev, st);
   note_launches(2);
   return cudaGetLastError() == cudaSuccess ? 0 : INFO_ESRF_ERR_CUDA;
 }
