@@ -1246,7 +1246,7 @@ __global__ void __launch_bounds__(kEigThreads) k_ritz_jacobi(const ProblemDev* t
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (j == 0) {
-        row_sum[i] = v;
+        row_sum[i] = v < INFINITY ? v : INFINITY;   // NaN as infinity: the maximum below would drop it
         row_lam[i] = li;
       }
     }
@@ -1259,7 +1259,7 @@ __global__ void __launch_bounds__(kEigThreads) k_ritz_jacobi(const ProblemDev* t
     delta *= 2.f;
     // a start that is no near eigenbasis (values beyond FP32's range, say):
     // FP64 Jacobi from the beginning
-    if (step == 0 && !(delta <= 1e-2f * lmax)) {
+    if (step == 0 && !(delta <= 1e-2f * lmax && delta < INFINITY)) {
       usable = false;
       break;
     }
