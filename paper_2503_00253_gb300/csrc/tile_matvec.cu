@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(128, 1)
   float* sg = red + 4 * BN;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  grid_dependency_wait();
   // an overflowed block pattern is not read (uniform across the grid)
   if (args.status && (*reinterpret_cast<volatile int32_t*>(args.status) & kStatTileOverflow)) return;
   const int chunk = (int)(blockIdx.x % (unsigned)args.nchunks);
@@ -249,7 +250,7 @@ int launch_tile_mm_t(TileMmArgs a, int units, const void* chi, const void* clo, 
     raised_dev = dev;
   }
   const int64_t grid = (int64_t)a.nrt * a.nchunks;
-  k_tile_mm<BN, S><<<(unsigned)grid, 128, Shape::kSmem, st>>>(mh, ml, mp, a);
+  launch_overlapped(k_tile_mm<BN, S>, dim3((unsigned)grid), 128, Shape::kSmem, st, mh, ml, mp, a);
   note_launches(1);
   return cudaGetLastError() == cudaSuccess ? INFO_ESRF_OK : INFO_ESRF_ERR_CUDA;
 }

@@ -149,6 +149,36 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// --- overlapped launches ------------------------------------------------------
+
+// Start of a kernel that launch_overlapped may start early: waits until the
+// kernels before it in the stream have finished and their results are visible,
+// then lets the next one be scheduled.  No memory that they write, or read, is
+// touched before it.
+__device__ __forceinline__ void grid_dependency_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launches a kernel that begins with grid_dependency_wait so that its CTAs may
+// be placed while the kernel before it in the stream still runs (programmatic
+// dependent launch): the gap between two launches of a PCG iteration is then a
+// wait on the chip instead of a launch after a drain.
+template <typename... P, typename... A>
+inline void launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // --- operand staging shared by the tcgen05 kernels -------------------------
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {

@@ -227,6 +227,7 @@ struct VecStep {
 template <int NV32, int SPT>
 __global__ void __launch_bounds__(kUpdThreads) k_tpcg_update(const ProblemDev* dpr, int update, const int32_t* list,
                                                              int it) {
+  grid_dependency_wait();
   constexpr int kSys = kUpdSlots * SPT;
   extern __shared__ float4 phs_dyn4[];   // [2 k][kDotRows / 4]
   __shared__ alignas(8) uint64_t bar;
@@ -379,6 +380,7 @@ constexpr int kScalThreads = 256;
 __global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev* dpr, int nsub, int last,
                                                                const int32_t* list, int32_t* next, int32_t* src,
                                                                int it) {
+  grid_dependency_wait();
   const ProblemDev& pr = *dpr;
   const int64_t pos = blockIdx.x;
   const int64_t j = pos < list_count(pr, list, it) ? (list ? list[pos] : pos) : -1;
@@ -391,14 +393,34 @@ __global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev*
   __shared__ double t_s[kMaxK], ti_s[kMaxK];
   __shared__ double gt_s[kMaxK][kMaxK + 1];
   __shared__ int go;
+  // everything that does not depend on the sums is loaded before them, so that
+  // the launch costs few of the memory's latencies one after another
+  const double sigma = sys_sigma(pr, j);
+  double* sd = pr.sysd + j * 8;
+  const double rho0 = sd[kRho], bn20 = sd[kBn2];
+  const bool first = sd[kFirst] != 0.0;
+  const bool lrn = pr.learn_on && pr.learn_on[j] == 1;
+  float la = 0.f;
+  if (lrn) la = pr.learn_coef[(j < pr.mean_sys ? pr.Q : (j - pr.mean_sys) / pr.N) * kLearnOut];
+  const double beta0 = pr.scal[1];   // beta_lmp - sigma
+  // G_q = A^T A + sigma (A^T Phi + Phi^T A) + sigma^2 Phi^T Phi, entries tid, tid + 256, ..
+  constexpr int kGramPer = (kMaxK * kMaxK + kScalThreads - 1) / kScalThreads;
+  double G[kGramPer];
+#pragma unroll
+  for (int i = 0; i < kGramPer; ++i) {
+    const int e = tid + i * kScalThreads;
+    if (e < k * k)
+      G[i] = pr.gram[2 * k * k + e] + sigma * (pr.gram[k * k + e] + pr.gram[k * k + (e % k) * k + e / k]) +
+             sigma * sigma * pr.gram[e];
+  }
+  if (tid < k) ti_s[tid] = 1.0 / (pr.theta[tid] + sigma);
   for (int e = lane; e < NVD; e += 32) {
     double sum = 0.0;
     const float* d = pr.dots + pos * nsub * NVD + e;
+#pragma unroll 4
     for (int cb = warp; cb < nsub; cb += kScalThreads / 32) sum += (double)d[(int64_t)cb * NVD];
     part[warp][e] = sum;
   }
-  const double sigma = sys_sigma(pr, j);
-  if (tid < k) ti_s[tid] = 1.0 / (pr.theta[tid] + sigma);
   __syncthreads();
   if (tid < NVD) {
     double sum = 0.0;
@@ -408,13 +430,10 @@ __global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev*
     if (tid >= 1 && tid <= k) t_s[tid - 1] = sum * ti_s[tid - 1];
   }
   __syncthreads();
-  double* sd = pr.sysd + j * 8;
   const double rr = v[0];
-  const bool first = sd[kFirst] != 0.0;
-  const bool lrn = pr.learn_on && pr.learn_on[j] == 1;
   if (tid == 0) {
     go = 0;
-    const double bn2 = first ? rr : sd[kBn2];
+    const double bn2 = first ? rr : bn20;
     if (first) sd[kBn2] = rr;
     sd[kRr] = rr;
     pr.relres[j] = bn2 > 0.0 ? sqrt(rr / bn2) : 0.0;
@@ -439,15 +458,16 @@ __global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev*
       go = act ? 1 : 0;
     }
   }
-  // G_q t, one product per thread: G_q = A^T A + sigma (A^T Phi + Phi^T A) + sigma^2 Phi^T Phi
-  for (int e = tid; e < k * k; e += kScalThreads) {
-    const int m = e / k, i2 = e - m * k;
-    const double G = pr.gram[2 * k * k + e] + sigma * (pr.gram[k * k + e] + pr.gram[k * k + i2 * k + m]) +
-                     sigma * sigma * pr.gram[e];
-    gt_s[m][i2] = G * t_s[i2];
+  // G_q t, one product per thread
+#pragma unroll
+  for (int i = 0; i < kGramPer; ++i) {
+    const int e = tid + i * kScalThreads;
+    if (e < k * k) gt_s[e / k][e % k] = G[i] * t_s[e % k];
   }
   __syncthreads();
   if (!go || warp != 0) return;
+  int at = 0;   // the system's position in the next list; needed last
+  if (lane == 0) at = atomicAdd(&pr.nactive[(it + 1) % 3], 1);
   float* lc = pr.lcoef + pos * 2 * kMaxK;
   double gt = 0.0, fc = 0.0;
   if (lane < k) {
@@ -460,7 +480,7 @@ __global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev*
     }
     if (i2 < k) s0 += gt_s[lane][i2];
     const double t2 = (g + sigma * f) - (s0 + s1);
-    const double cc = pr.scal[1] * t - t2 * ti_s[lane];   // (beta_lmp - sigma) t - T^-1 t2
+    const double cc = beta0 * t - t2 * ti_s[lane];   // (beta_lmp - sigma) t - T^-1 t2
     gt = g * t;
     fc = f * cc;
     lc[lane] = (float)cc;   // Phi columns take c, C Phi columns -t
@@ -473,14 +493,10 @@ __global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev*
   }
   if (lane != 0) return;
   double rho = k > 0 ? rr - gt + fc : rr;
-  if (lrn) {   // rho = r^T (a P^-1 + S S) r = a r^T P^-1 r + u^T u
-    const int64_t q = j < pr.mean_sys ? pr.Q : (j - pr.mean_sys) / pr.N;
-    rho = (double)pr.learn_coef[q * kLearnOut] * rho + v[2 * k + 1];
-  }
-  pr.betaf[pos] = first ? 0.f : (float)(rho / sd[kRho]);
+  if (lrn) rho = (double)la * rho + v[2 * k + 1];   // r^T (a P^-1 + S S) r = a r^T P^-1 r + u^T u
+  pr.betaf[pos] = first ? 0.f : (float)(rho / rho0);
   sd[kRho] = rho;
   sd[kFirst] = 0.0;
-  const int at = atomicAdd(&pr.nactive[(it + 1) % 3], 1);
   next[at] = (int32_t)j;
   src[at] = (int32_t)pos;
 }
@@ -498,6 +514,7 @@ template <int K, int RPL>
 __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev* dpr, const int32_t* list,
                                                                 const int32_t* src, int group, int learned, int it) {
   constexpr int kBatch = 4;
+  grid_dependency_wait();
   const ProblemDev& pr = *dpr;
   const int k = pr.kR;
   const int64_t dp = pr.d_pad;
@@ -704,15 +721,17 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
     // gives every SM two CTAs; 64 dot values (k > 15) leave registers for one
     const int spt = p.kR <= 15 && nsub * count >= 32 * (int64_t)sms ? 2 : 1;
     const dim3 grid((unsigned)nsub, (unsigned)((count + kUpdSlots * spt - 1) / (kUpdSlots * spt)));
-    if (p.kR > 15) k_tpcg_update<2, 1><<<grid, kUpdThreads, usm, st>>>(dp, mode, list, it);
-    else if (spt == 2) k_tpcg_update<1, 2><<<grid, kUpdThreads, usm, st>>>(dp, mode, list, it);
-    else k_tpcg_update<1, 1><<<grid, kUpdThreads, usm, st>>>(dp, mode, list, it);
+    if (p.kR > 15) launch_overlapped(k_tpcg_update<2, 1>, grid, kUpdThreads, usm, st, dp, mode, list, it);
+    else if (spt == 2) launch_overlapped(k_tpcg_update<1, 2>, grid, kUpdThreads, usm, st, dp, mode, list, it);
+    else launch_overlapped(k_tpcg_update<1, 1>, grid, kUpdThreads, usm, st, dp, mode, list, it);
   };
   auto direction = [&](const int32_t* list, int64_t count, int it) {
     const int group = dir_group(dchunks, count, sms);
     const dim3 grid((unsigned)((dchunks + kVecWarps - 1) / kVecWarps), (unsigned)((count + group - 1) / group));
-    if (wide) k_tpcg_direction<24, 2><<<grid, kVecThreads, 0, st>>>(dp, list, srcs, group, learned ? 1 : 0, it);
-    else k_tpcg_direction<12, 2><<<grid, kVecThreads, 0, st>>>(dp, list, srcs, group, learned ? 1 : 0, it);
+    const int32_t* from = srcs;
+    const int lrn = learned ? 1 : 0;
+    if (wide) launch_overlapped(k_tpcg_direction<24, 2>, grid, kVecThreads, 0, st, dp, list, from, group, lrn, it);
+    else launch_overlapped(k_tpcg_direction<12, 2>, grid, kVecThreads, 0, st, dp, list, from, group, lrn, it);
   };
   // iteration 0, the first direction of every running system: r = b, z = M r, p = z
   auto start = [&]() {
@@ -771,7 +790,8 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
       }
       update(fused_alpha ? 2 : 1, list, bound, it);
       if (learned) launch_tile_learn_u(p, dp, list, bound, nsub, it, st);
-      k_tpcg_scalars<<<(unsigned)bound, kScalThreads, 0, st>>>(dp, nsub, it == maxit ? 1 : 0, list, next, srcs, it);
+      launch_overlapped(k_tpcg_scalars, dim3((unsigned)bound), kScalThreads, 0, st, dp, nsub, it == maxit ? 1 : 0, list,
+                        next, srcs, it);
       cudaEventRecord(counted[it & 1], st);
       direction(next, bound, it);
       note_launches(3);
