@@ -340,7 +340,6 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
   ProblemDev* dtab = cv.take<ProblemDev>(sizeof(ProblemDev) * count);
   int32_t* counter = cv.take<int32_t>(kCounterInts * sizeof(int32_t));
   int group_base = 0, sys_base = 0;
-  const int JT = pcg_jt(o.precision);
   for (int i = 0; i < count; ++i) {
     const info_esrf_problem& P = probs[i];
     ProblemDev& pr = tab.p[i];
@@ -413,8 +412,8 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
     pr.R = P.R_diag;
     pr.mu_a = P.mu_a;
     pr.A_a = P.A_a;
-    pr.JT = JT;
-    pr.groups_per_q = (int32_t)((pr.N + JT - 1) / JT);
+    pr.JT = pcg_jt(o.precision, (pr.do_pert ? pr.Q * pr.N : 0) + (pr.do_mean ? 1 : 0), num_sms);
+    pr.groups_per_q = (int32_t)((pr.N + pr.JT - 1) / pr.JT);
     pr.num_groups = (pr.do_pert ? pr.Q * pr.groups_per_q : 0) + (pr.do_mean ? 1 : 0);
     pr.group_base = group_base;
     group_base += pr.num_groups;

@@ -43,8 +43,12 @@ namespace infoesrf {
 constexpr int kPcgThreads = 512;
 constexpr int kPcgWarps = kPcgThreads / 32;
 template <typename T> struct PcgVec;
-template <> struct PcgVec<float> { static constexpr int VL = 4, JT = 8; };
-template <> struct PcgVec<double> { static constexpr int VL = 1, JT = 2; };
+template <> struct PcgVec<float> { static constexpr int VL = 4; };
+template <> struct PcgVec<double> { static constexpr int VL = 1; };
+// Systems per group: two items a row (an entry of C and a column of Phi serve
+// both); in FP64 one for problems of few groups (pcg_jt).
+template <typename T> constexpr int kJTWide = 2 * PcgVec<T>::VL;
+template <typename T> constexpr int kJTNarrow = sizeof(T) == 8 ? 1 : kJTWide<T>;
 
 template <typename T>
 struct Item {
@@ -92,9 +96,8 @@ __device__ __forceinline__ GroupInfo decode_group(const ProblemDev* tab, int cou
   return gi;
 }
 
-template <typename T, int KMAX>
+template <typename T, int KMAX, int JT>
 struct PcgShared {
-  static constexpr int JT = PcgVec<T>::JT;
   alignas(16) T coef[2 * KMAX][JT];        // direction: c for the Phi columns, -t for the C Phi columns
   T red[4 * kPcgWarps][JT];                // projections: [set][4 nq columns]
   double Gq[KMAX * KMAX + 1];
@@ -105,16 +108,15 @@ struct PcgShared {
   double wpd[JT][kPcgWarps];
   double ts[JT][KMAX + 1];
   int active[JT], iters[JT];
-  int any_active, group;
   double sigma, beta_lmp;
 };
 
 // Sums acc over the lanes of a warp that serve the same systems (lane mod G)
 // and writes the warp's partial of each system.
-template <typename T, int KMAX>
-__device__ __forceinline__ void warp_partials(PcgShared<T, KMAX>& sh, const DotAcc<T> (&acc)[PcgVec<T>::VL], int warp,
-                                              int lane) {
-  constexpr int VL = PcgVec<T>::VL, G = PcgVec<T>::JT / VL;
+template <typename T, int KMAX, int JT>
+__device__ __forceinline__ void warp_partials(PcgShared<T, KMAX, JT>& sh, const DotAcc<T> (&acc)[PcgVec<T>::VL],
+                                              int warp, int lane) {
+  constexpr int VL = PcgVec<T>::VL, G = JT / VL;
 #pragma unroll
   for (int v = 0; v < VL; ++v) {
     if constexpr (sizeof(T) == 4) {
@@ -141,8 +143,8 @@ __device__ __forceinline__ void warp_partials(PcgShared<T, KMAX>& sh, const DotA
 // Sum of the warps' partials of system j, by one warp.  Every lane returns lane
 // 0's value: the callers branch on it, and all lanes must take the same way
 // (the low parts of a float-float butterfly may differ between lanes).
-template <typename T, int KMAX>
-__device__ __forceinline__ double combine_partials(const PcgShared<T, KMAX>& sh, int j, int lane) {
+template <typename T, int KMAX, int JT>
+__device__ __forceinline__ double combine_partials(const PcgShared<T, KMAX, JT>& sh, int j, int lane) {
   static_assert(kPcgWarps <= 32, "one lane per warp partial");
   double s;
   if constexpr (sizeof(T) == 4) {
@@ -182,8 +184,7 @@ constexpr size_t kPcgSmem = 200 * 1024;   // dynamic shared memory of a CTA (one
 constexpr int kPcgChunk = 1024;           // rows of r staged at a time for the projections (levels 1 and 2)
 
 template <typename T>
-__host__ __device__ __forceinline__ PcgLayout pcg_layout(int64_t d) {
-  constexpr int JT = PcgVec<T>::JT;
+__host__ __device__ __forceinline__ PcgLayout pcg_layout(int64_t d, int JT) {
   PcgLayout l;
   l.vec = (size_t)d * JT;
   l.pvec = (size_t)p_row<T>(d + 3) * JT;
@@ -194,15 +195,420 @@ __host__ __device__ __forceinline__ PcgLayout pcg_layout(int64_t d) {
   return l;
 }
 
+// One group to convergence, by all threads of the CTA.
+template <typename T, int KMAX, int JT>
+__device__ __forceinline__ void solve_group(const ProblemDev& pr, const GroupInfo& gi, T* sm, T* slice,
+                                            PcgShared<T, KMAX, JT>& sh) {
+  constexpr int VL = PcgVec<T>::VL, G = JT / VL;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = tid % G;   // which systems of a row this thread serves, in every item loop
+  const int d = (int)pr.d;
+  const int64_t N = pr.N;
+  const int k = pr.kR < KMAX ? pr.kR : KMAX;
+  const PcgLayout lay = pcg_layout<T>(d, JT);
+  T* vp = lay.level <= 1 ? sm : slice + 3 * lay.vec;
+  T* vr = lay.level == 0 ? sm + lay.pvec : slice;
+  T* vy = vr + lay.vec;
+  T* vx = vy + lay.vec;
+  T* rbuf = lay.level == 0 ? vr : (lay.level == 1 ? sm + lay.pvec : sm);   // rows of r under projection
+  const int crows = lay.level == 0 ? d : kPcgChunk;
+  const T* __restrict__ val = reinterpret_cast<const T*>(pr.oo_val);
+  const int32_t* __restrict__ col = pr.oo_col;
+  const T* __restrict__ PhiT = reinterpret_cast<const T*>(pr.phiT);   // [2 k][d]
+  const T* __restrict__ W = reinterpret_cast<const T*>(pr.W);
+
+  // ---- group setup: shift, LMP constants, G_q ----
+  if (tid == 0) {
+    const double s = gi.q < 0 ? 0.0 : pr.s[gi.q];
+    sh.sigma = s + 1.0;
+    sh.beta_lmp = sh.sigma + pr.scal[1];
+  }
+  __syncthreads();
+  const double sigma = sh.sigma;
+  const T sigma_t = to_t<T>(sigma);
+  for (int e = tid; e < k * k; e += kPcgThreads) {
+    const int i = e / k, j = e % k;
+    const int kk = pr.kR;   // gram matrices are stored with the problem's k
+    const int ge = i * kk + j, gt = j * kk + i;
+    // G_q = A^T A + sigma (A^T Phi + Phi^T A) + sigma^2 Phi^T Phi
+    sh.Gq[e] = pr.gram[2 * kk * kk + ge] + sigma * (pr.gram[kk * kk + ge] + pr.gram[kk * kk + gt]) +
+               sigma * sigma * pr.gram[ge];
+  }
+  for (int m = tid; m < k; m += kPcgThreads) sh.ith[m] = 1.0 / (pr.theta[m] + sigma);
+  if (tid < JT) {
+    sh.active[tid] = tid < gi.lanes;
+    sh.iters[tid] = 0;
+    sh.beta[tid] = T(0);
+    sh.rr[tid] = 0.0;
+    sh.alpha[tid] = T(0);
+  }
+
+  // ---- x = 0, r = b, p = 0 ----
+  for (int e = tid; e < d * JT; e += kPcgThreads) {
+    const int a = e / JT, j = e % JT;
+    T b = T(0);
+    if (j < gi.lanes) {
+      if (gi.q < 0) b = to_t<T>(pr.bmean[a]);
+      else b = W[a * N + gi.i0 + j] * to_t<T>(pr.rinv[a]);
+    }
+    vr[e] = b;
+    vx[e] = T(0);
+    vp[p_row<T>(a) * JT + j] = T(0);
+  }
+  __syncthreads();
+
+  bool first = true;
+  const int maxit = pr.fixed_iters > 0 ? pr.fixed_iters : pr.max_iter;
+  const int nq = (2 * k + 3) / 4;              // column quads of [Phi | C Phi]
+  const int sets = nq > 0 ? kPcgWarps / nq : 1;   // warps per quad
+  const int quad = nq > 0 ? warp % nq : 0, set = nq > 0 ? warp / nq : 0;
+
+  // The update x += alpha p, r -= alpha y (not on the first call), then
+  // r^T r, f = Phi^T r and g = A^T r, in one pass: rows of r go through
+  // shared memory, where warp (quad, set) projects them on its four columns
+  // with 4 JT register accumulators, lanes over rows (coalesced columns).
+  // Then the scalars, one warp per system.
+  auto residual_pass = [&]() {
+    DotAcc<T> rr[VL];
+    T acc[4][JT];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < JT; ++j) acc[i][j] = T(0);
+    T al[VL];
+#pragma unroll
+    for (int v = 0; v < VL; ++v) al[v] = sh.alpha[g * VL + v];
+    for (int c0 = 0; c0 < d; c0 += crows) {
+      const int nr = d - c0 < crows ? d - c0 : crows;
+      // kU items at once: their loads are all in flight before the first use
+      // (levels 1 and 2 stream the vectors from L2)
+      constexpr int kU = 2;
+      for (int it0 = tid; it0 < nr * G; it0 += kU * kPcgThreads) {
+        Item<T> r[kU], y[kU], x[kU], p[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int it = it0 + u * kPcgThreads;
+          if (it >= nr * G) continue;
+          const int64_t o = ((int64_t)c0 * G + it) * VL;
+          r[u] = ld_item(vr + o);
+          if (first) continue;
+          y[u] = ld_item(vy + o);
+          x[u] = ld_item(vx + o);
+          p[u] = ld_item(vp + p_row<T>(c0 + it / G) * JT + g * VL);
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int it = it0 + u * kPcgThreads;
+          if (it >= nr * G) continue;
+          const int64_t o = ((int64_t)c0 * G + it) * VL;
+          if (!first) {
+#pragma unroll
+            for (int v = 0; v < VL; ++v) {
+              x[u].v[v] += al[v] * p[u].v[v];
+              r[u].v[v] -= al[v] * y[u].v[v];
+            }
+            st_item(vx + o, x[u]);
+            st_item(vr + o, r[u]);
+          }
+          if (lay.level != 0) st_item(rbuf + (int64_t)it * VL, r[u]);
+#pragma unroll
+          for (int v = 0; v < VL; ++v) rr[v].add_prod(r[u].v[v], r[u].v[v]);
+        }
+      }
+      if (nq == 0) continue;
+      __syncthreads();
+      if (set < sets) {
+        const int m0 = 4 * quad;
+#pragma unroll 2
+        for (int a = lane + 32 * set; a < nr; a += 32 * sets) {
+          T rv[JT];
+#pragma unroll
+          for (int u = 0; u < G; ++u) {
+            const Item<T> t = ld_item(rbuf + (int64_t)a * JT + u * VL);
+#pragma unroll
+            for (int v = 0; v < VL; ++v) rv[u * VL + v] = t.v[v];
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const T ph = m0 + i < 2 * k ? PhiT[(int64_t)(m0 + i) * d + c0 + a] : T(0);
+#pragma unroll
+            for (int j = 0; j < JT; ++j) acc[i][j] += ph * rv[j];
+          }
+        }
+      }
+      if (c0 + crows < d) __syncthreads();   // the next chunk overwrites the buffer
+    }
+    warp_partials<T, KMAX, JT>(sh, rr, warp, lane);
+    if (nq > 0 && set < sets) {
+      // reduce-scatter the 4 JT sums over the warp: first halve the values
+      // held per lane, then sum the lanes that hold the same value
+      constexpr int V = 4 * JT;   // 32 (FP32), 8 or 4 (FP64)
+      T* v = &acc[0][0];
+      int idx = 0;
+#pragma unroll
+      for (int off = 16, w = V / 2; w >= 1; off >>= 1, w >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+          const T send = up ? v[i] : v[i + w];
+          const T keep = up ? v[i + w] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+        if (up) idx += w;
+      }
+#pragma unroll
+      for (int off = 16 / V; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+      if ((lane & (32 / V - 1)) == 0) sh.red[set * 4 * nq + 4 * quad + idx / JT][idx % JT] = v[0];
+    }
+    __syncthreads();
+    if (warp < JT) {
+      const int j = warp;
+      const double rr_j = combine_partials<T, KMAX, JT>(sh, j, lane);
+      const bool was_active = sh.active[j] != 0;
+      const double bn2 = first ? rr_j : sh.bn2[j];
+      __syncwarp();   // lane 0 writes both below
+      bool act = was_active;
+      if (act && pr.fixed_iters <= 0 && !(rr_j > pr.tol * pr.tol * bn2)) act = false;
+      if (act && (!(rr_j > 0.0) || !isfinite(rr_j))) act = false;
+      double rho = rr_j;
+      if (k > 0 && act) {
+        T fs = T(0), gs = T(0);
+        if (lane < k)
+          for (int s = 0; s < sets; ++s) {
+            fs += sh.red[s * 4 * nq + lane][j];
+            gs += sh.red[s * 4 * nq + k + lane][j];
+          }
+        const double f = (double)fs, gg2 = (double)gs;
+        const double ith = lane < k ? sh.ith[lane] : 0.0;
+        const double t = f * ith;
+        if (lane < k) sh.ts[j][lane] = t;
+        __syncwarp();
+        double a0 = 0.0, a1 = 0.0;   // G_q t, two chains
+        if (lane < k) {
+          int i2 = 0;
+          for (; i2 + 1 < k; i2 += 2) {
+            a0 += sh.Gq[lane * k + i2] * sh.ts[j][i2];
+            a1 += sh.Gq[lane * k + i2 + 1] * sh.ts[j][i2 + 1];
+          }
+          if (i2 < k) a0 += sh.Gq[lane * k + i2] * sh.ts[j][i2];
+        }
+        const double t2 = gg2 + sigma * f - (a0 + a1);
+        const double c = (sh.beta_lmp - sigma) * t - t2 * ith;
+        double df = lane < k ? f * c - gg2 * t : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) df += __shfl_xor_sync(0xffffffffu, df, o);
+        rho = rr_j + df;
+        if (lane < k) {
+          sh.coef[lane][j] = to_t<T>(c);
+          sh.coef[k + lane][j] = to_t<T>(-t);
+        }
+      }
+      if (lane == 0) {
+        if (first) sh.bn2[j] = rr_j;
+        if (!act) {
+          sh.beta[j] = T(0);
+        } else {
+          sh.beta[j] = first ? T(0) : to_t<T>(rho / sh.rho[j]);
+          sh.rho[j] = rho;
+        }
+        if (was_active || first) sh.rr[j] = rr_j;
+        sh.active[j] = act;
+      }
+    }
+    __syncthreads();
+    int any = 0;
+#pragma unroll
+    for (int j = 0; j < JT; ++j) any |= sh.active[j];
+    return any != 0;
+  };
+
+  // z = P^-1 r, p = z + beta p (a stopped system keeps its p)
+  auto update_direction = [&]() {
+    T be[VL];
+    bool on[VL];
+#pragma unroll
+    for (int v = 0; v < VL; ++v) {
+      be[v] = sh.beta[g * VL + v];
+      on[v] = sh.active[g * VL + v] != 0;
+    }
+    constexpr int kU = sizeof(T) == 4 ? 4 : 2;   // items side by side: one read of the coefficients serves all
+    for (int it = tid; it < d * G; it += kU * kPcgThreads) {
+      Item<T> z[kU];
+      int a[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int iu = it + u * kPcgThreads;
+        a[u] = iu < d * G ? iu / G : 0;
+        z[u] = ld_item(vr + (int64_t)a[u] * JT + g * VL);
+      }
+#pragma unroll 4
+      for (int m = 0; m < 2 * k; ++m) {
+        const Item<T> c = ld_item(&sh.coef[m][g * VL]);
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const T ph = PhiT[(int64_t)m * d + a[u]];
+#pragma unroll
+          for (int v = 0; v < VL; ++v) z[u].v[v] += ph * c.v[v];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        if (it + u * kPcgThreads >= d * G) continue;
+        T* pp = vp + p_row<T>(a[u]) * JT + g * VL;
+        Item<T> p = ld_item(pp);
+#pragma unroll
+        for (int v = 0; v < VL; ++v) p.v[v] = on[v] ? z[u].v[v] + be[v] * p.v[v] : p.v[v];
+        st_item(pp, p);
+      }
+    }
+    __syncthreads();
+  };
+
+  bool run = residual_pass();
+  first = false;
+  if (run) update_direction();
+
+  // FP32: C by quads of rows where the set-up made them (k_pcg_quads)
+  const bool quads = sizeof(T) == 4 && pr.qval && pr.status[2] == 0;
+  // items of the matvec, and threads per item: the largest power of two that
+  // still covers all items at once (small problems split a row's entries)
+  const int items = (quads ? (d + 3) / 4 : d) * G;
+  int tpi = 1;
+  while (tpi < 16 && 2 * tpi * items <= kPcgThreads) tpi *= 2;
+  const int per = 32 / tpi, sub = lane / per, ii = lane % per;
+
+  int it = 0;
+  while (run && it < maxit) {
+    ++it;
+    // ---- y = C_q p, p^T y ----
+    DotAcc<T> pap[VL];
+    const int iend = (items + per - 1) / per * per;   // whole warps take part in the shuffles
+    if constexpr (sizeof(T) == 4) {
+      if (quads) {
+        const int nb = (d + 3) / 4;
+        const float4* __restrict__ qv = reinterpret_cast<const float4*>(pr.qval);
+        const int32_t* __restrict__ qc = pr.qcol;
+        for (int i = warp * per + ii; i < iend; i += kPcgWarps * per) {
+          const bool in = i < items;
+          const int blk = in ? i / G : 0;
+          float acc[4][VL] = {};
+          const int n = in ? pr.qn[blk] : 0;
+#pragma unroll 8
+          for (int e = sub; e < n; e += tpi) {
+            const float4 c = qv[(int64_t)e * nb + blk];
+            const Item<T> pb = ld_item(vp + qc[(int64_t)e * nb + blk] + g * VL);
+            const float cc[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+#pragma unroll
+              for (int v = 0; v < VL; ++v) acc[w][v] = fmaf(cc[w], pb.v[v], acc[w][v]);
+          }
+          for (int o = 16; o >= per; o >>= 1)
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+#pragma unroll
+              for (int v = 0; v < VL; ++v) acc[w][v] += __shfl_xor_sync(0xffffffffu, acc[w][v], o);
+          if (in && sub == 0) {
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              const int a = 4 * blk + w;
+              if (a >= d) break;
+              const Item<T> p = ld_item(vp + p_row<T>(a) * JT + g * VL);
+              Item<T> y;
+#pragma unroll
+              for (int v = 0; v < VL; ++v) {
+                y.v[v] = fmaf(sigma_t, p.v[v], acc[w][v]);
+                pap[v].add_prod(p.v[v], y.v[v]);
+              }
+              st_item(vy + (int64_t)a * JT + g * VL, y);
+            }
+          }
+        }
+      }
+    }
+    if (!quads) {
+      for (int i = warp * per + ii; i < iend; i += kPcgWarps * per) {
+        const bool in = i < items;
+        const int a = in ? i / G : 0;
+        Item<T> acc{};
+        const int nnz = in ? pr.oo_nnz[a] : 0;
+#pragma unroll 4
+        for (int e = sub; e < nnz; e += tpi) {
+          const T c = val[(int64_t)e * d + a];
+          const int b = col[(int64_t)e * d + a];
+          const Item<T> pb = ld_item(vp + p_row<T>(b) * JT + g * VL);
+#pragma unroll
+          for (int v = 0; v < VL; ++v) acc.v[v] += c * pb.v[v];
+        }
+        for (int o = 16; o >= per; o >>= 1)
+#pragma unroll
+          for (int v = 0; v < VL; ++v) acc.v[v] += __shfl_xor_sync(0xffffffffu, acc.v[v], o);
+        if (in && sub == 0) {
+          const Item<T> p = ld_item(vp + p_row<T>(a) * JT + g * VL);
+#pragma unroll
+          for (int v = 0; v < VL; ++v) {
+            acc.v[v] += sigma_t * p.v[v];
+            pap[v].add_prod(p.v[v], acc.v[v]);
+          }
+          st_item(vy + (int64_t)a * JT + g * VL, acc);
+        }
+      }
+    }
+    warp_partials<T, KMAX, JT>(sh, pap, warp, lane);
+    __syncthreads();
+    if (warp < JT) {
+      const int j = warp;
+      const double pAp = combine_partials<T, KMAX, JT>(sh, j, lane);
+      if (lane == 0) {
+        T alpha = T(0);
+        if (sh.active[j]) {
+          if (pAp > 0.0 && isfinite(pAp)) {
+            alpha = to_t<T>(sh.rho[j] / pAp);
+            sh.iters[j] = it;
+          } else {
+            sh.active[j] = 0;
+            atomicOr(&pr.status[0], kStatBreakdown);
+          }
+        }
+        sh.alpha[j] = alpha;
+      }
+    }
+    __syncthreads();
+    run = residual_pass();
+    if (!run) break;
+    update_direction();
+  }
+
+  // ---- results ----
+  // lane j holds system sid0 + j (the mean group has one lane, sid 0)
+  const int64_t sid0 = gi.q < 0 ? 0 : pr.mean_sys + (int64_t)gi.q * N + gi.i0;
+  T* U = reinterpret_cast<T*>(pr.U);
+  for (int j = 0; j < gi.lanes; ++j)
+    for (int a = tid; a < d; a += kPcgThreads) U[(sid0 + j) * d + a] = vx[(int64_t)a * JT + j];
+  if (tid < gi.lanes) {
+    const int64_t sidx = sid0 + tid;
+    pr.iters[sidx] = sh.iters[tid];
+    const double bn = sh.bn2[tid];
+    pr.relres[sidx] = bn > 0 ? sqrt(sh.rr[tid] / bn) : 0.0;
+    if (sh.active[tid] && pr.fixed_iters <= 0) atomicOr(&pr.status[0], kStatNotConverged);
+  }
+  __syncthreads();
+}
+
 template <typename T, int KMAX>
 __global__ void __launch_bounds__(kPcgThreads, 1)
 k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* gscratch,
       int64_t scratch_stride, uint64_t band_mask, const int32_t* band_fb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int JT = PcgVec<T>::JT, VL = PcgVec<T>::VL, G = JT / VL;
-  __shared__ PcgShared<T, KMAX> sh;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int g = tid % G;   // which systems of a row this thread serves, in every item loop
+  __shared__ union Shared {
+    PcgShared<T, KMAX, kJTWide<T>> wide;
+    PcgShared<T, KMAX, kJTNarrow<T>> narrow;
+    __device__ Shared() {}
+  } sh;
+  __shared__ int s_group;
+  const int tid = threadIdx.x;
+  T* sm = reinterpret_cast<T*>(smem_raw);
+  T* slice = gscratch + (int64_t)blockIdx.x * scratch_stride;
   // Problems in band_mask were given to the band kernel first; this kernel
   // solves them only where it fell back (band_fb[p] != 0).
   auto band_solved = [&](int p) { return ((band_mask >> p) & 1ull) && band_fb[p] == 0; };
@@ -213,9 +619,9 @@ k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* g
   }
 
   for (;;) {
-    if (tid == 0) sh.group = atomicAdd(counter, 1);
+    if (tid == 0) s_group = atomicAdd(counter, 1);
     __syncthreads();
-    const int gg = sh.group;
+    const int gg = s_group;
     if (gg >= total_groups) break;
     const GroupInfo gi = decode_group(tab, count, gg);
     const ProblemDev& pr = tab[gi.prob];
@@ -225,399 +631,11 @@ k_pcg(const ProblemDev* tab, int count, int total_groups, int32_t* counter, T* g
       __syncthreads();
       continue;
     }
-    const int d = (int)pr.d;
-    const int64_t N = pr.N;
-    const int k = pr.kR < KMAX ? pr.kR : KMAX;
-    const PcgLayout lay = pcg_layout<T>(d);
-    T* sm = reinterpret_cast<T*>(smem_raw);
-    T* slice = gscratch + (int64_t)blockIdx.x * scratch_stride;
-    T* vp = lay.level <= 1 ? sm : slice + 3 * lay.vec;
-    T* vr = lay.level == 0 ? sm + lay.pvec : slice;
-    T* vy = vr + lay.vec;
-    T* vx = vy + lay.vec;
-    T* rbuf = lay.level == 0 ? vr : (lay.level == 1 ? sm + lay.pvec : sm);   // rows of r under projection
-    const int crows = lay.level == 0 ? d : kPcgChunk;
-    const T* __restrict__ val = reinterpret_cast<const T*>(pr.oo_val);
-    const int32_t* __restrict__ col = pr.oo_col;
-    const T* __restrict__ PhiT = reinterpret_cast<const T*>(pr.phiT);   // [2 k][d]
-    const T* __restrict__ W = reinterpret_cast<const T*>(pr.W);
-
-    // ---- group setup: shift, LMP constants, G_q ----
-    if (tid == 0) {
-      const double s = gi.q < 0 ? 0.0 : pr.s[gi.q];
-      sh.sigma = s + 1.0;
-      sh.beta_lmp = sh.sigma + pr.scal[1];
+    if (pr.JT == kJTWide<T>) {
+      solve_group<T, KMAX, kJTWide<T>>(pr, gi, sm, slice, sh.wide);
+    } else if constexpr (kJTNarrow<T> != kJTWide<T>) {
+      solve_group<T, KMAX, kJTNarrow<T>>(pr, gi, sm, slice, sh.narrow);
     }
-    __syncthreads();
-    const double sigma = sh.sigma;
-    const T sigma_t = to_t<T>(sigma);
-    for (int e = tid; e < k * k; e += kPcgThreads) {
-      const int i = e / k, j = e % k;
-      const int kk = pr.kR;   // gram matrices are stored with the problem's k
-      const int ge = i * kk + j, gt = j * kk + i;
-      // G_q = A^T A + sigma (A^T Phi + Phi^T A) + sigma^2 Phi^T Phi
-      sh.Gq[e] = pr.gram[2 * kk * kk + ge] + sigma * (pr.gram[kk * kk + ge] + pr.gram[kk * kk + gt]) +
-                 sigma * sigma * pr.gram[ge];
-    }
-    for (int m = tid; m < k; m += kPcgThreads) sh.ith[m] = 1.0 / (pr.theta[m] + sigma);
-    if (tid < JT) {
-      sh.active[tid] = tid < gi.lanes;
-      sh.iters[tid] = 0;
-      sh.beta[tid] = T(0);
-      sh.rr[tid] = 0.0;
-      sh.alpha[tid] = T(0);
-    }
-
-    // ---- x = 0, r = b, p = 0 ----
-    for (int e = tid; e < d * JT; e += kPcgThreads) {
-      const int a = e / JT, j = e % JT;
-      T b = T(0);
-      if (j < gi.lanes) {
-        if (gi.q < 0) b = to_t<T>(pr.bmean[a]);
-        else b = W[a * N + gi.i0 + j] * to_t<T>(pr.rinv[a]);
-      }
-      vr[e] = b;
-      vx[e] = T(0);
-      vp[p_row<T>(a) * JT + j] = T(0);
-    }
-    __syncthreads();
-
-    bool first = true;
-    const int maxit = pr.fixed_iters > 0 ? pr.fixed_iters : pr.max_iter;
-    const int nq = (2 * k + 3) / 4;              // column quads of [Phi | C Phi]
-    const int sets = nq > 0 ? kPcgWarps / nq : 1;   // warps per quad
-    const int quad = nq > 0 ? warp % nq : 0, set = nq > 0 ? warp / nq : 0;
-
-    // The update x += alpha p, r -= alpha y (not on the first call), then
-    // r^T r, f = Phi^T r and g = A^T r, in one pass: rows of r go through
-    // shared memory, where warp (quad, set) projects them on its four columns
-    // with 4 JT register accumulators, lanes over rows (coalesced columns).
-    // Then the scalars, one warp per system.
-    auto residual_pass = [&]() {
-      DotAcc<T> rr[VL];
-      T acc[4][JT];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < JT; ++j) acc[i][j] = T(0);
-      T al[VL];
-#pragma unroll
-      for (int v = 0; v < VL; ++v) al[v] = sh.alpha[g * VL + v];
-      for (int c0 = 0; c0 < d; c0 += crows) {
-        const int nr = d - c0 < crows ? d - c0 : crows;
-        // kU items at once: their loads are all in flight before the first use
-        // (levels 1 and 2 stream the vectors from L2)
-        constexpr int kU = 2;
-        for (int it0 = tid; it0 < nr * G; it0 += kU * kPcgThreads) {
-          Item<T> r[kU], y[kU], x[kU], p[kU];
-#pragma unroll
-          for (int u = 0; u < kU; ++u) {
-            const int it = it0 + u * kPcgThreads;
-            if (it >= nr * G) continue;
-            const int64_t o = ((int64_t)c0 * G + it) * VL;
-            r[u] = ld_item(vr + o);
-            if (first) continue;
-            y[u] = ld_item(vy + o);
-            x[u] = ld_item(vx + o);
-            p[u] = ld_item(vp + p_row<T>(c0 + it / G) * JT + g * VL);
-          }
-#pragma unroll
-          for (int u = 0; u < kU; ++u) {
-            const int it = it0 + u * kPcgThreads;
-            if (it >= nr * G) continue;
-            const int64_t o = ((int64_t)c0 * G + it) * VL;
-            if (!first) {
-#pragma unroll
-              for (int v = 0; v < VL; ++v) {
-                x[u].v[v] += al[v] * p[u].v[v];
-                r[u].v[v] -= al[v] * y[u].v[v];
-              }
-              st_item(vx + o, x[u]);
-              st_item(vr + o, r[u]);
-            }
-            if (lay.level != 0) st_item(rbuf + (int64_t)it * VL, r[u]);
-#pragma unroll
-            for (int v = 0; v < VL; ++v) rr[v].add_prod(r[u].v[v], r[u].v[v]);
-          }
-        }
-        if (nq == 0) continue;
-        __syncthreads();
-        if (set < sets) {
-          const int m0 = 4 * quad;
-#pragma unroll 2
-          for (int a = lane + 32 * set; a < nr; a += 32 * sets) {
-            T rv[JT];
-#pragma unroll
-            for (int u = 0; u < G; ++u) {
-              const Item<T> t = ld_item(rbuf + (int64_t)a * JT + u * VL);
-#pragma unroll
-              for (int v = 0; v < VL; ++v) rv[u * VL + v] = t.v[v];
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const T ph = m0 + i < 2 * k ? PhiT[(int64_t)(m0 + i) * d + c0 + a] : T(0);
-#pragma unroll
-              for (int j = 0; j < JT; ++j) acc[i][j] += ph * rv[j];
-            }
-          }
-        }
-        if (c0 + crows < d) __syncthreads();   // the next chunk overwrites the buffer
-      }
-      warp_partials<T, KMAX>(sh, rr, warp, lane);
-      if (nq > 0 && set < sets) {
-        // reduce-scatter the 4 JT sums over the warp: first halve the values
-        // held per lane, then sum the lanes that hold the same value
-        constexpr int V = 4 * JT;   // 32 (FP32) or 8 (FP64)
-        T* v = &acc[0][0];
-        int idx = 0;
-#pragma unroll
-        for (int off = 16, w = V / 2; w >= 1; off >>= 1, w >>= 1) {
-          const bool up = (lane & off) != 0;
-#pragma unroll
-          for (int i = 0; i < w; ++i) {
-            const T send = up ? v[i] : v[i + w];
-            const T keep = up ? v[i + w] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-          }
-          if (up) idx += w;
-        }
-#pragma unroll
-        for (int off = 16 / V; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
-        if (V == 32 || (lane & 3) == 0) sh.red[set * 4 * nq + 4 * quad + idx / JT][idx % JT] = v[0];
-      }
-      __syncthreads();
-      if (warp < JT) {
-        const int j = warp;
-        const double rr_j = combine_partials<T, KMAX>(sh, j, lane);
-        const bool was_active = sh.active[j] != 0;
-        const double bn2 = first ? rr_j : sh.bn2[j];
-        __syncwarp();   // lane 0 writes both below
-        bool act = was_active;
-        if (act && pr.fixed_iters <= 0 && !(rr_j > pr.tol * pr.tol * bn2)) act = false;
-        if (act && (!(rr_j > 0.0) || !isfinite(rr_j))) act = false;
-        double rho = rr_j;
-        if (k > 0 && act) {
-          T fs = T(0), gs = T(0);
-          if (lane < k)
-            for (int s = 0; s < sets; ++s) {
-              fs += sh.red[s * 4 * nq + lane][j];
-              gs += sh.red[s * 4 * nq + k + lane][j];
-            }
-          const double f = (double)fs, gg2 = (double)gs;
-          const double ith = lane < k ? sh.ith[lane] : 0.0;
-          const double t = f * ith;
-          if (lane < k) sh.ts[j][lane] = t;
-          __syncwarp();
-          double a0 = 0.0, a1 = 0.0;   // G_q t, two chains
-          if (lane < k) {
-            int i2 = 0;
-            for (; i2 + 1 < k; i2 += 2) {
-              a0 += sh.Gq[lane * k + i2] * sh.ts[j][i2];
-              a1 += sh.Gq[lane * k + i2 + 1] * sh.ts[j][i2 + 1];
-            }
-            if (i2 < k) a0 += sh.Gq[lane * k + i2] * sh.ts[j][i2];
-          }
-          const double t2 = gg2 + sigma * f - (a0 + a1);
-          const double c = (sh.beta_lmp - sigma) * t - t2 * ith;
-          double df = lane < k ? f * c - gg2 * t : 0.0;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) df += __shfl_xor_sync(0xffffffffu, df, o);
-          rho = rr_j + df;
-          if (lane < k) {
-            sh.coef[lane][j] = to_t<T>(c);
-            sh.coef[k + lane][j] = to_t<T>(-t);
-          }
-        }
-        if (lane == 0) {
-          if (first) sh.bn2[j] = rr_j;
-          if (!act) {
-            sh.beta[j] = T(0);
-          } else {
-            sh.beta[j] = first ? T(0) : to_t<T>(rho / sh.rho[j]);
-            sh.rho[j] = rho;
-          }
-          if (was_active || first) sh.rr[j] = rr_j;
-          sh.active[j] = act;
-        }
-      }
-      __syncthreads();
-      int any = 0;
-#pragma unroll
-      for (int j = 0; j < JT; ++j) any |= sh.active[j];
-      return any != 0;
-    };
-
-    // z = P^-1 r, p = z + beta p (a stopped system keeps its p)
-    auto update_direction = [&]() {
-      T be[VL];
-      bool on[VL];
-#pragma unroll
-      for (int v = 0; v < VL; ++v) {
-        be[v] = sh.beta[g * VL + v];
-        on[v] = sh.active[g * VL + v] != 0;
-      }
-      constexpr int kU = sizeof(T) == 4 ? 4 : 2;   // items side by side: one read of the coefficients serves all
-      for (int it = tid; it < d * G; it += kU * kPcgThreads) {
-        Item<T> z[kU];
-        int a[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int iu = it + u * kPcgThreads;
-          a[u] = iu < d * G ? iu / G : 0;
-          z[u] = ld_item(vr + (int64_t)a[u] * JT + g * VL);
-        }
-#pragma unroll 4
-        for (int m = 0; m < 2 * k; ++m) {
-          const Item<T> c = ld_item(&sh.coef[m][g * VL]);
-#pragma unroll
-          for (int u = 0; u < kU; ++u) {
-            const T ph = PhiT[(int64_t)m * d + a[u]];
-#pragma unroll
-            for (int v = 0; v < VL; ++v) z[u].v[v] += ph * c.v[v];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          if (it + u * kPcgThreads >= d * G) continue;
-          T* pp = vp + p_row<T>(a[u]) * JT + g * VL;
-          Item<T> p = ld_item(pp);
-#pragma unroll
-          for (int v = 0; v < VL; ++v) p.v[v] = on[v] ? z[u].v[v] + be[v] * p.v[v] : p.v[v];
-          st_item(pp, p);
-        }
-      }
-      __syncthreads();
-    };
-
-    bool run = residual_pass();
-    first = false;
-    if (run) update_direction();
-
-    // FP32: C by quads of rows where the set-up made them (k_pcg_quads)
-    const bool quads = sizeof(T) == 4 && pr.qval && pr.status[2] == 0;
-    // items of the matvec, and threads per item: the largest power of two that
-    // still covers all items at once (small problems split a row's entries)
-    const int items = (quads ? (d + 3) / 4 : d) * G;
-    int tpi = 1;
-    while (tpi < 16 && 2 * tpi * items <= kPcgThreads) tpi *= 2;
-    const int per = 32 / tpi, sub = lane / per, ii = lane % per;
-
-    int it = 0;
-    while (run && it < maxit) {
-      ++it;
-      // ---- y = C_q p, p^T y ----
-      DotAcc<T> pap[VL];
-      const int iend = (items + per - 1) / per * per;   // whole warps take part in the shuffles
-      if constexpr (sizeof(T) == 4) {
-        if (quads) {
-          const int nb = (d + 3) / 4;
-          const float4* __restrict__ qv = reinterpret_cast<const float4*>(pr.qval);
-          const int32_t* __restrict__ qc = pr.qcol;
-          for (int i = warp * per + ii; i < iend; i += kPcgWarps * per) {
-            const bool in = i < items;
-            const int blk = in ? i / G : 0;
-            float acc[4][VL] = {};
-            const int n = in ? pr.qn[blk] : 0;
-#pragma unroll 8
-            for (int e = sub; e < n; e += tpi) {
-              const float4 c = qv[(int64_t)e * nb + blk];
-              const Item<T> pb = ld_item(vp + qc[(int64_t)e * nb + blk] + g * VL);
-              const float cc[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-              for (int w = 0; w < 4; ++w)
-#pragma unroll
-                for (int v = 0; v < VL; ++v) acc[w][v] = fmaf(cc[w], pb.v[v], acc[w][v]);
-            }
-            for (int o = 16; o >= per; o >>= 1)
-#pragma unroll
-              for (int w = 0; w < 4; ++w)
-#pragma unroll
-                for (int v = 0; v < VL; ++v) acc[w][v] += __shfl_xor_sync(0xffffffffu, acc[w][v], o);
-            if (in && sub == 0) {
-#pragma unroll
-              for (int w = 0; w < 4; ++w) {
-                const int a = 4 * blk + w;
-                if (a >= d) break;
-                const Item<T> p = ld_item(vp + p_row<T>(a) * JT + g * VL);
-                Item<T> y;
-#pragma unroll
-                for (int v = 0; v < VL; ++v) {
-                  y.v[v] = fmaf(sigma_t, p.v[v], acc[w][v]);
-                  pap[v].add_prod(p.v[v], y.v[v]);
-                }
-                st_item(vy + (int64_t)a * JT + g * VL, y);
-              }
-            }
-          }
-        }
-      }
-      if (!quads) {
-        for (int i = warp * per + ii; i < iend; i += kPcgWarps * per) {
-          const bool in = i < items;
-          const int a = in ? i / G : 0;
-          Item<T> acc{};
-          const int nnz = in ? pr.oo_nnz[a] : 0;
-#pragma unroll 4
-          for (int e = sub; e < nnz; e += tpi) {
-            const T c = val[(int64_t)e * d + a];
-            const int b = col[(int64_t)e * d + a];
-            const Item<T> pb = ld_item(vp + p_row<T>(b) * JT + g * VL);
-#pragma unroll
-            for (int v = 0; v < VL; ++v) acc.v[v] += c * pb.v[v];
-          }
-          for (int o = 16; o >= per; o >>= 1)
-#pragma unroll
-            for (int v = 0; v < VL; ++v) acc.v[v] += __shfl_xor_sync(0xffffffffu, acc.v[v], o);
-          if (in && sub == 0) {
-            const Item<T> p = ld_item(vp + p_row<T>(a) * JT + g * VL);
-#pragma unroll
-            for (int v = 0; v < VL; ++v) {
-              acc.v[v] += sigma_t * p.v[v];
-              pap[v].add_prod(p.v[v], acc.v[v]);
-            }
-            st_item(vy + (int64_t)a * JT + g * VL, acc);
-          }
-        }
-      }
-      warp_partials<T, KMAX>(sh, pap, warp, lane);
-      __syncthreads();
-      if (warp < JT) {
-        const int j = warp;
-        const double pAp = combine_partials<T, KMAX>(sh, j, lane);
-        if (lane == 0) {
-          T alpha = T(0);
-          if (sh.active[j]) {
-            if (pAp > 0.0 && isfinite(pAp)) {
-              alpha = to_t<T>(sh.rho[j] / pAp);
-              sh.iters[j] = it;
-            } else {
-              sh.active[j] = 0;
-              atomicOr(&pr.status[0], kStatBreakdown);
-            }
-          }
-          sh.alpha[j] = alpha;
-        }
-      }
-      __syncthreads();
-      run = residual_pass();
-      if (!run) break;
-      update_direction();
-    }
-
-    // ---- results ----
-    // lane j holds system sid0 + j (the mean group has one lane, sid 0)
-    const int64_t sid0 = gi.q < 0 ? 0 : pr.mean_sys + (int64_t)gi.q * N + gi.i0;
-    T* U = reinterpret_cast<T*>(pr.U);
-    for (int j = 0; j < gi.lanes; ++j)
-      for (int a = tid; a < d; a += kPcgThreads) U[(sid0 + j) * d + a] = vx[(int64_t)a * JT + j];
-    if (tid < gi.lanes) {
-      const int64_t sidx = sid0 + tid;
-      pr.iters[sidx] = sh.iters[tid];
-      const double bn = sh.bn2[tid];
-      pr.relres[sidx] = bn > 0 ? sqrt(sh.rr[tid] / bn) : 0.0;
-      if (sh.active[tid] && pr.fixed_iters <= 0) atomicOr(&pr.status[0], kStatNotConverged);
-    }
-    __syncthreads();
   }
 }
 
@@ -634,9 +652,8 @@ constexpr int kQuadWarps = 4;
 __global__ void __launch_bounds__(32 * kQuadWarps) k_pcg_quads(const ProblemDev* tab) {
   const ProblemDev& pr = tab[blockIdx.y];
   if (!pr.qval) return;
-  constexpr int JT = PcgVec<float>::JT;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int d = (int)pr.d, nb = (d + 3) / 4;
+  const int JT = pr.JT, d = (int)pr.d, nb = (d + 3) / 4;
   const int blk = blockIdx.x * kQuadWarps + warp;
   if (blk >= nb) return;
   extern __shared__ uint32_t words_s[];   // per warp: bitmap, then the rank of each word's first bit
@@ -752,14 +769,26 @@ void launch_pcg_phit(const ProblemTable& tab, const ProblemDev* dtab, cudaStream
   note_launches(1);
 }
 
-int pcg_jt(int precision) { return precision == 0 ? PcgVec<double>::JT : PcgVec<float>::JT; }
+// Systems per group of a problem with `systems` of them.  A CTA takes a group
+// to its end, so the hardest group's iterations bound the call from below.
+// FP64, whose pipe is the bound: groups of one halve that time where groups of
+// two leave CTAs without work (100 weighted sums, 161 systems: 1.30 -> 1.12
+// ms; at 321 systems, more groups of two than CTAs, 0.57 -> 0.61).  FP32: half
+// a group's iteration costs almost what a whole one does (layered 961 systems 7.0 -> 7.3 ms).
+// The rule looks at the problem alone, and so a batched call solves it in the
+// same way as a call of its own.
+int pcg_jt(int precision, int64_t systems, int num_sms) {
+  if (precision != 0) return kJTWide<float>;
+  return (systems + 1) / 2 <= num_sms ? kJTNarrow<double> : kJTWide<double>;
+}
 
 // Elements of one CTA's global slice: what the largest problem keeps there.
 static size_t slice_elems(const ProblemTable& tab) {
   size_t most = 0;
   for (int i = 0; i < tab.count; ++i) {
     const bool f64 = tab.p[i].precision == 0;
-    const PcgLayout l = f64 ? pcg_layout<double>(tab.p[i].d) : pcg_layout<float>(tab.p[i].d);
+    const PcgLayout l =
+        f64 ? pcg_layout<double>(tab.p[i].d, tab.p[i].JT) : pcg_layout<float>(tab.p[i].d, tab.p[i].JT);
     const size_t need = l.level == 0 ? 0 : (l.level == 1 ? 3 * l.vec : 3 * l.vec + l.pvec);
     most = std::max(most, need);
   }
