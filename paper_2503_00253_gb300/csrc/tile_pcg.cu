@@ -257,24 +257,13 @@ __global__ void __launch_bounds__(kUpdThreads) k_tpcg_update(const ProblemDev* d
     sys[threadIdx.x] = j >= 0 && (list || pr.active[j]) ? (int32_t)j : -1;
   }
   __syncthreads();
-  if (update == 2) {
-    for (int s = warp; s < kSys; s += kUpdThreads / 32) {
-      const int j = sys[s];
-      if (j < 0) continue;
-      const double al = warp_alpha(pr, j, g0 + s, it, blockIdx.x == 0, lane);
-      if (lane == 0) als[s] = (float)al;
-    }
-    __syncthreads();
-  }
   const int slot = threadIdx.x / kRowLanes, r0 = threadIdx.x % kRowLanes;
   int64_t base[SPT], pbase[SPT];   // first element of each of the thread's systems (X, R) and positions (Y, P)
-  float al[SPT];
 #pragma unroll
   for (int u = 0; u < SPT; ++u) {
     const int s = slot * SPT + u;
     base[u] = sys[s] < 0 ? -1 : (int64_t)sys[s] * dp + abase;
     pbase[u] = (g0 + s) * dp + abase;
-    al[u] = als[s];
   }
   float acc[SPT][32 * NV32];
 #pragma unroll
@@ -295,7 +284,19 @@ __global__ void __launch_bounds__(kUpdThreads) k_tpcg_update(const ProblemDev* d
       }
     }
   };
-  load(cur, 4 * r0);
+  load(cur, 4 * r0);   // in flight while alpha is formed
+  if (update == 2) {
+    for (int s = warp; s < kSys; s += kUpdThreads / 32) {
+      const int j = sys[s];
+      if (j < 0) continue;
+      const double al = warp_alpha(pr, j, g0 + s, it, blockIdx.x == 0, lane);
+      if (lane == 0) als[s] = (float)al;
+    }
+    __syncthreads();
+  }
+  float al[SPT];
+#pragma unroll
+  for (int u = 0; u < SPT; ++u) al[u] = als[slot * SPT + u];
   if (k > 0 && !mbar_wait(&bar, 0)) {
     atomicOr(&pr.status[0], kStatTimeout);
     return;
