@@ -31,6 +31,17 @@ __device__ __forceinline__ Coord3 flat_to_coord(const GridDev& g, int64_t idx) {
   return c;
 }
 
+// The same for grids of less than 2^31 points, without 64-bit divisions.
+__device__ __forceinline__ Coord3 flat_to_coord32(const GridDev& g, uint32_t idx) {
+  const uint32_t nx = (uint32_t)g.ext[0], ny = (uint32_t)g.ext[1];
+  const uint32_t t = idx / nx, z = t / ny;
+  Coord3 c;
+  c.x = idx - t * nx;
+  c.y = t - z * ny;
+  c.z = z;
+  return c;
+}
+
 __device__ __forceinline__ double axis_distance(const GridDev& g, int ax, int64_t a, int64_t b) {
   int64_t delta = a > b ? a - b : b - a;
   const int64_t e = g.ext[ax];
@@ -104,11 +115,27 @@ __device__ __forceinline__ int64_t lower_bound_i64(const int64_t* a, int64_t lo,
   return lo;
 }
 
+// The same by a whole warp (all lanes call it with the same arguments): 32
+// probes a step, so 1024 entries take two dependent reads instead of ten.
+__device__ __forceinline__ int64_t lower_bound_warp(const int64_t* a, int64_t lo, int64_t hi, int64_t key) {
+  const int lane = threadIdx.x & 31;
+  while (lo < hi) {
+    const int64_t step = (hi - lo + 32) / 33;
+    const int64_t at = lo + step * (lane + 1) - 1;
+    const int below = __popc(__ballot_sync(0xffffffffu, at < hi && a[at] < key));
+    const int64_t next = lo + step * (below + 1) - 1;   // probe `below`: not below the key, if it is in range
+    lo += step * below;
+    if (below < 32 && next < hi) hi = next;
+  }
+  return lo;
+}
+
 // Visits the obs-index ranges [b0, b1) whose grid points can lie inside the
 // Gaspari-Cohn support of point p: one box row (z, y) at a time, with the x
 // window split at the periodic seam.  Candidates are supersets; callers test
 // r < 2 exactly.  f(b0, b1) is called with increasing flat index within a row.
-template <typename F>
+// WARP: called by whole warps with the same point on every lane.
+template <bool WARP = false, typename F>
 __device__ __forceinline__ void for_each_candidate_range(const GridDev& g, const int64_t* obs, int64_t d,
                                                          const Coord3& p, F&& f) {
   const int64_t nx = g.ext[0], ny = g.ext[1], nz = g.ext[2];
@@ -147,8 +174,14 @@ __device__ __forceinline__ void for_each_candidate_range(const GridDev& g, const
         }
       }
       for (int k = 0; k < nint; ++k) {
-        const int64_t b0 = lower_bound_i64(obs, 0, d, base + lo[k]);
-        const int64_t b1 = lower_bound_i64(obs, b0, d, base + hi[k] + 1);
+        int64_t b0, b1;
+        if constexpr (WARP) {
+          b0 = lower_bound_warp(obs, 0, d, base + lo[k]);
+          b1 = lower_bound_warp(obs, b0, d, base + hi[k] + 1);
+        } else {
+          b0 = lower_bound_i64(obs, 0, d, base + lo[k]);
+          b1 = lower_bound_i64(obs, b0, d, base + hi[k] + 1);
+        }
         if (b1 > b0) f(b0, b1);
       }
     }
