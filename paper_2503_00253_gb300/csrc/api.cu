@@ -538,23 +538,23 @@ int run_batch(const info_esrf_problem* probs, int32_t count, const info_esrf_opt
     launch_finish(tab, dtab, st);
   } else if (o.solver == INFO_ESRF_SOLVER_MULTISHIFT) {
     launch_band_obs(tab, dtab, st);
-    // no Ritz stage and no learned coefficients: the quadrature and the
-    // state-obs band run on the side stream while nothing else waits
+    // no Ritz stage and no learned coefficients.  The state-obs band is for the
+    // finish only: it runs on the side stream under the solver, whose clusters
+    // leave part of the chip idle, and is enqueued after it, so that they don't wait
+    // for its CTAs to drain.
     AuxStream* aux = aux_stream();
+    launch_quadrature(tab, dtab, st);
+    if (aux) cudaEventRecord(aux->mid, st);
+    mark(1);
+    mark(2);
+    const int solved = launch_mscg(tab, dtab, tab.ms, sms, st);
+    if (solved != 0) return INFO_ESRF_ERR_CUDA;
     if (aux) {
-      cudaEventRecord(aux->mid, st);
       cudaStreamWaitEvent(aux->s, aux->mid, 0);
       launch_band_state(tab, dtab, aux->s);
       cudaEventRecord(aux->jb, aux->s);
     } else {
       launch_band_state(tab, dtab, st);
-    }
-    launch_quadrature(tab, dtab, st);
-    mark(1);
-    mark(2);
-    if (launch_mscg(tab, dtab, tab.ms, sms, st) != 0) {
-      if (aux) cudaStreamWaitEvent(st, aux->jb, 0);
-      return INFO_ESRF_ERR_CUDA;
     }
     mark(3);
     if (aux) cudaStreamWaitEvent(st, aux->jb, 0);
