@@ -246,7 +246,8 @@ __global__ void __launch_bounds__(32 * kHWarps) k_observe_H(const ProblemDev* ta
 // row, one warp per observation with its lanes over the row's entries; rows
 // that miss the supports cost no arithmetic.  (Each (x, b) formed its own
 // products z_x . z_j, so every pair (x, j) was formed once per observation
-// that sees j: 656 to 865 us at n = 2000, d = 100, rows of 137 entries.)
+// that sees j: 656 to 865 us at n = 2000, d = 100, rows of 137 entries; 155 us with
+// the squared distance of every pair in FP64, 115 us with the support's box checked in integers.)
 constexpr int kXB = 4;
 constexpr size_t kSxhSmem = 200 * 1024;
 template <typename T>
@@ -262,13 +263,26 @@ __global__ void __launch_bounds__(256) k_sxh_H(const ProblemDev* tab) {
   const T* Zt = tp<const T>(pr.Zt);
   Coord3 px[kXB];
 #pragma unroll
-  for (int u = 0; u < kXB; ++u) px[u] = flat_to_coord(g, x0 + u < n ? x0 + u : x0);
+  for (int u = 0; u < kXB; ++u) px[u] = flat_to_coord32(g, (uint32_t)(x0 + u < n ? x0 + u : x0));
+  // in integers: beyond the support's box on some axis
+  auto outside = [&](const Coord3& a, const Coord3& b) {
+    const int64_t ca[3] = {a.x, a.y, a.z}, cb[3] = {b.x, b.y, b.z};
+    bool out = false;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      if (g.whole[ax]) continue;
+      int64_t delta = ca[ax] > cb[ax] ? ca[ax] - cb[ax] : cb[ax] - ca[ax];
+      if (g.periodic[ax] && g.ext[ax] - delta < delta) delta = g.ext[ax] - delta;
+      out |= delta > g.reach[ax];
+    }
+    return out;
+  };
   for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-    const Coord3 pj = flat_to_coord(g, j);
+    const Coord3 pj = flat_to_coord32(g, (uint32_t)j);
     const T* zj = Zt + j * N;
     for (int u = 0; u < kXB; ++u) {
       double v = 0.0;
-      if (x0 + u < n) {
+      if (x0 + u < n && !outside(px[u], pj)) {
         const double r2 = scaled_r2_tab(g, pr.d2tab, px[u], pj);
         if (r2 < 4.0) {
           DotAcc<T> dot;
@@ -966,11 +980,17 @@ __global__ void k_ritz_orth(const ProblemDev* tab, int src) {
 // at 1024.)  A non-positive pivot
 // zeroes that column (rank loss) and flags kStatEigFail.
 constexpr int kOrthThreads = kMaxRitz * kMaxRitz;   // one thread per entry of G and W
-constexpr int kOrthEntries = kOrthThreads;          // entries of X_dst per block
-__global__ void __launch_bounds__(kOrthThreads) k_ritz_orth64(const ProblemDev* tab, int src) {
+// Entries of X_dst per block (a multiple of 128): few enough that all SMs share
+// the dot products, whose FP64 instructions hold an SM's pipe for 16 clocks a warp
+// (1024 entries: 20 us a launch at 60 to 100 rows, 14 us now); every block repeats
+// the factorization.
+static int orth_entries(int64_t total) {
+  return (int)std::min<int64_t>(std::max<int64_t>((total / 152 + 127) / 128 * 128, 128), kOrthThreads);
+}
+__global__ void __launch_bounds__(kOrthThreads) k_ritz_orth64(const ProblemDev* tab, int src, int entries) {
   const ProblemDev& pr = tab[blockIdx.y];
   const int l = pr.l;
-  const int64_t e0 = (int64_t)blockIdx.x * kOrthEntries, total = pr.d * l;
+  const int64_t e0 = (int64_t)blockIdx.x * entries, total = pr.d * l;
   if (l <= 0 || e0 >= total) return;
   __shared__ FF G[kMaxRitz][kMaxRitz + 1];   // upper triangle
   __shared__ FF W[kMaxRitz][kMaxRitz + 1];   // lower triangle: R^-T
@@ -1014,7 +1034,7 @@ __global__ void __launch_bounds__(kOrthThreads) k_ritz_orth64(const ProblemDev* 
   const double* X = ritz_buf<double>(pr, src);
   double* Y = ritz_buf<double>(pr, 1 - src);
   const int64_t e = e0 + t;
-  if (e < total) {
+  if (t < entries && e < total) {
     const int64_t a = e / l;
     const int j = (int)(e - a * l);
     double s0 = 0.0, s1 = 0.0;   // two chains
@@ -1440,7 +1460,8 @@ static void launch_ritz_t(const ProblemTable& tab, const ProblemDev* dtab, cudaS
   if (lmax <= 0 || kmax <= 0) return;
   const dim3 gdl((unsigned)((dl + 255) / 256), tab.count);
   const dim3 gd((unsigned)((dmax + 255) / 256), tab.count);
-  const dim3 go((unsigned)((dl + kOrthEntries - 1) / kOrthEntries), tab.count);
+  const int oe = orth_entries(dl * tab.count);
+  const dim3 go((unsigned)((dl + oe - 1) / oe), tab.count);
   const dim3 gv((unsigned)((dmax * kmax + kVecEntries - 1) / kVecEntries), tab.count);
   const dim3 gdw((unsigned)((dmax * 32 + 255) / 256), tab.count);   // one warp per row
   const dim3 gll((unsigned)(lmax * lmax), tab.count);
@@ -1454,7 +1475,7 @@ static void launch_ritz_t(const ProblemTable& tab, const ProblemDev* dtab, cudaS
     note_launches(1);
   };
   auto orth = [&](int x) {
-    if constexpr (sizeof(T) == 8) k_ritz_orth64<<<go, kOrthThreads, 0, st>>>(dtab, x);
+    if constexpr (sizeof(T) == 8) k_ritz_orth64<<<go, kOrthThreads, 0, st>>>(dtab, x, oe);
     else k_ritz_orth<T><<<gd, 256, 0, st>>>(dtab, x);
   };
   auto orth2 = [&](int x) {   // orthonormalize buf[x] in place (scratch: the other buffer)
