@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(128, 1)
       const __nv_bfloat16* src = args.P + (int64_t)(c0 + i * kTileUnit) * args.d_pad + a;
 #pragma unroll
       for (int c = 0; c < kTileUnit; ++c)
-        p[c] = c0 + i * kTileUnit + c < T ? __bfloat162float(__ldg(src + (int64_t)c * args.d_pad)) : 0.f;
+        p[c] = c0 + i * kTileUnit + c < T ? __bfloat162float(src[(int64_t)c * args.d_pad]) : 0.f;
     };
     float p[kTileUnit];
     load_p(p, 0);

@@ -154,10 +154,21 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 // Start of a kernel that launch_overlapped may start early: waits until the
 // kernels before it in the stream have finished and their results are visible,
 // then lets the next one be scheduled.  No memory that they write, or read, is
-// touched before it.
+// touched before it.  What the kernel right before wrote is read with ordinary
+// loads (or TMA), never through the non-coherent path (__ldg): that path asks
+// for data that nobody writes while the reader is resident, and the reader is
+// resident while its predecessor still runs.
 __device__ __forceinline__ void grid_dependency_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Non-coherent load in such a kernel, of settled data: written before the
+// kernel right before it was allowed to let this one start, that is by kernels at
+// least two launches back (each waits for all before it first) or before the loop.
+template <typename T>
+__device__ __forceinline__ T ld_settled(const T* p) {
+  return __ldg(p);
 }
 
 // Launches a kernel that begins with grid_dependency_wait so that its CTAs may

@@ -569,10 +569,10 @@ __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev
     if (in) {
       const float* src = reinterpret_cast<const float*>(pr.phiT) + (int64_t)mm * dp + a;
       if constexpr (RPL == 4) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(src));
+        const float4 t = ld_settled(reinterpret_cast<const float4*>(src));
         c[m][0] = t.x; c[m][1] = t.y; c[m][2] = t.z; c[m][3] = t.w;
       } else {
-        const float2 t = __ldg(reinterpret_cast<const float2*>(src));
+        const float2 t = ld_settled(reinterpret_cast<const float2*>(src));
         c[m][0] = t.x; c[m][1] = t.y;
       }
     }
@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev
           const float* u = pr.learn_u + (int64_t)j * dp;
           float su = 0.f;
 #pragma unroll
-          for (int n = 0; n < kLatPts; ++n) su = fmaf(ltap[s][lat_bin(n)], __ldg(u + nb[n]), su);
+          for (int n = 0; n < kLatPts; ++n) su = fmaf(ltap[s][lat_bin(n)], ld_settled(u + nb[n]), su);
           z[b][i] = fmaf(la, z[b][i], su);
         }
         const uint32_t w = pw[b][i / 2];
