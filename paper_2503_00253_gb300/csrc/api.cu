@@ -28,21 +28,26 @@ AuxStream* aux_stream() {
   }
   AuxStream& a = aux[dev];
   if (!a.s) {
-    cudaStream_t s = nullptr;
-    cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
-    bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
-    for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&e[i], cudaEventDisableTiming) == cudaSuccess;
+    cudaStream_t s[2] = {nullptr, nullptr};
+    cudaEvent_t e[5] = {};
+    bool ok = true;
+    for (int i = 0; i < 2 && ok; ++i) ok = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking) == cudaSuccess;
+    for (int i = 0; i < 5 && ok; ++i) ok = cudaEventCreateWithFlags(&e[i], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();
-      for (int i = 0; i < 3; ++i)
-        if (e[i]) cudaEventDestroy(e[i]);
-      if (s) cudaStreamDestroy(s);
+      for (cudaEvent_t x : e)
+        if (x) cudaEventDestroy(x);
+      for (cudaStream_t x : s)
+        if (x) cudaStreamDestroy(x);
       return nullptr;
     }
-    a.s = s;
+    a.s = s[0];
+    a.count = s[1];
     a.mid = e[0];
     a.jq = e[1];
     a.jb = e[2];
+    a.counted[0] = e[3];
+    a.counted[1] = e[4];
   }
   return &a;
 }

@@ -311,14 +311,16 @@ void launch_obs_matvec(const ProblemDev& pr, const ProblemDev* dpr, int32_t nvec
 void launch_lmp_apply(const ProblemDev& pr, const ProblemDev* dpr, int32_t nvec, const double* Rv,
                       const double* sigma, double* Z, cudaStream_t st);
 
-// Side stream and events, per host thread and device, for the work that
-// overlaps the main sequence (the quadrature and the state-obs band under the
-// Ritz stage; the BF16 path's read of the running count).  Created on first
-// use and kept for the life of the thread (like a library handle); NULL when
-// that fails.
+// Side streams and events, per host thread and device, for the work that
+// overlaps the main sequence: s for device work (the quadrature and the
+// state-obs band under the Ritz stage), count for the BF16 path's reads of
+// the running count, which the host waits for and which therefore share no stream
+// with work of other calls.  Created on first use and kept for the life of the
+// thread (like a library handle); NULL when that fails.
 struct AuxStream {
-  cudaStream_t s = nullptr;
+  cudaStream_t s = nullptr, count = nullptr;
   cudaEvent_t mid = nullptr, jq = nullptr, jb = nullptr;
+  cudaEvent_t counted[2] = {nullptr, nullptr};   // the scalars of BF16 iterations in turn are done
 };
 AuxStream* aux_stream();
 

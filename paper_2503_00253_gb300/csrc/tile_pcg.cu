@@ -662,9 +662,7 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
                          const TileCapture* cap) {
   const int64_t J = p.nsys;
   if (J < 1) return 0;
-  AuxStream* aux = aux_stream();
-  if (!aux) return INFO_ESRF_ERR_CUDA;
-  const cudaEvent_t counted[2] = {aux->mid, aux->jq};   // the scalars of iterations in turn are done
+  AuxStream* aux = aux_stream();   // NULL: the counts are read on st, behind the iteration in flight
   cudaEvent_t ev[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // matvec begin and end, iterations in turn
   struct Destroy {
     cudaEvent_t (*e)[2];
@@ -739,17 +737,19 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
     update(0, nullptr, J, 0);
     if (learned) launch_tile_learn_u(p, dp, nullptr, J, nsub, 0, st);
     k_tpcg_scalars<<<(unsigned)J, kScalThreads, 0, st>>>(dp, nsub, maxit <= 0 ? 1 : 0, nullptr, lists[1], srcs, 0);
-    cudaEventRecord(counted[0], st);
+    if (aux) cudaEventRecord(aux->counted[0], st);
     direction(lists[1], J, 0);
     note_launches(3);
   };
-  // counts[it + 1] (and the status word) after iteration it, read on the side
-  // stream so that the main stream keeps running
+  // counts[it + 1] (and the status word) after iteration it, read on a stream of
+  // its own so that the main stream keeps running and the host waits for nothing
+  // else.  (Iteration it + 1 leaves the slot alone: on st the value is the same.)
   int32_t host[4] = {0, 0, 0, 0};
   auto read_counts = [&](int it) -> int {
-    if (cudaStreamWaitEvent(aux->s, counted[it & 1], 0) != cudaSuccess ||
-        cudaMemcpyAsync(host, p.nactive, sizeof(host), cudaMemcpyDeviceToHost, aux->s) != cudaSuccess ||
-        cudaStreamSynchronize(aux->s) != cudaSuccess)
+    const cudaStream_t rs = aux ? aux->count : st;
+    if ((aux && cudaStreamWaitEvent(rs, aux->counted[it & 1], 0) != cudaSuccess) ||
+        cudaMemcpyAsync(host, p.nactive, sizeof(host), cudaMemcpyDeviceToHost, rs) != cudaSuccess ||
+        cudaStreamSynchronize(rs) != cudaSuccess)
       return INFO_ESRF_ERR_CUDA;
     return 0;
   };
@@ -793,7 +793,7 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
       if (learned) launch_tile_learn_u(p, dp, list, bound, nsub, it, st);
       launch_overlapped(k_tpcg_scalars, dim3((unsigned)bound), kScalThreads, 0, st, dp, nsub, it == maxit ? 1 : 0, list,
                         next, srcs, it);
-      cudaEventRecord(counted[it & 1], st);
+      if (aux) cudaEventRecord(aux->counted[it & 1], st);
       direction(next, bound, it);
       note_launches(3);
     }
