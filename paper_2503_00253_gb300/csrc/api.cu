@@ -333,9 +333,10 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
 constexpr size_t kNoallocBytes = size_t(32) << 20;
 
 // Builds the host table for a batch; with ws == nullptr only sizes it.
+// *bytes_out is the size with the optional parts, *least_out the size that a call needs.
 int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_options& o, void* ws,
                 size_t ws_bytes, ProblemTable& tab, size_t* bytes_out, ProblemDev** dtab_out, int32_t** counter_out,
-                void** scratch_out, size_t* scratch_bytes_out, int num_sms) {
+                void** scratch_out, size_t* scratch_bytes_out, int num_sms, size_t* least_out = nullptr) {
   if (count < 1) return INFO_ESRF_ERR_INVALID_ARG;
   if (count > kMaxProblems) return INFO_ESRF_ERR_UNSUPPORTED;
   memset(&tab, 0, sizeof(tab));
@@ -439,6 +440,7 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
   }
   // the quads of C, last
   const size_t base = cv.off;
+  if (least_out) *least_out = base;
   size_t quads = 0;
   int64_t qcap[kMaxProblems];
   for (int i = 0; i < count; ++i) {
@@ -826,7 +828,12 @@ int info_esrf_autotune(const info_esrf_problem* probs, int32_t count, info_esrf_
         o.power_iters = pi_list[b];
         o.oversample = os_list[c];
         if (o.ritz_rank + o.oversample > kMaxRitz) continue;
-        if (info_esrf_batched_workspace_size(probs, count, &o) > ws_bytes) continue;
+        static thread_local ProblemTable tab;
+        size_t size = 0, least = 0;   // a call runs in `least` bytes, without the optional parts
+        if (build_table(probs, count, o, nullptr, 0, tab, &size, nullptr, nullptr, nullptr, nullptr, num_sms_current(),
+                        &least) == 0 &&
+            least > ws_bytes)
+          continue;
         int r = run_batch(probs, count, &o, workspace, ws_bytes, stream, stats.data());
         if (r < 0) {
           if (!first_rc) first_rc = r;
