@@ -1187,9 +1187,12 @@ __global__ void k_ritz_jacobi_pairs(const ProblemDev* tab) {
 // R = I - X^T X, S = X^T B X and lambda_i = S_ii / (1 - R_ii),
 //   X <- X + X E,  E_ij = (S_ij + lambda_j R_ij) / (lambda_j - lambda_i),
 // R_ij / 2 where the eigenvalues are too close to separate: 1e-6 -> 1e-12 ->
-// rounding.  FP64 Jacobi sweeps on (X^T B X, X), one thread per entry and l / 2
-// disjoint rotations per round, finish what is left, if anything
-// (unseparated eigenvalues).
+// rounding where they are separated.  Elsewhere E up to 1e-4 leaves X orthogonal
+// to |E|^2 only, so X <- X + X (I - X^T X) / 2 then makes it orthonormal to
+// rounding (once or twice): without it the matrix X^T B X that is left has other
+// eigenvalues than B (eigenvalues 1 + 1e-5 i, l = 32: wrong in the ninth digit).
+// FP64 Jacobi sweeps on (X^T B X, X), one thread per entry and l / 2 disjoint
+// rotations per round, finish what is left, if anything (unseparated eigenvalues).
 constexpr int kEigThreads = kMaxRitz * kMaxRitz;
 __device__ __forceinline__ void jacobi_rotation(double app, double aqq, double apq, double& c, double& s) {
   c = 1.0;
@@ -1309,6 +1312,19 @@ __global__ void __launch_bounds__(kEigThreads) k_ritz_jacobi(const ProblemDev* t
     if (mine) V[0][i][j] += V[1][i][j];
     __syncthreads();
   }
+  // X orthonormal to rounding: a step squares the error (3/4 R^2), so from 1e-9 one is enough
+  for (int step = 0; usable && step < 3; ++step) {
+    eig_product<true>(V[0], V[0], A[1], l);             // X^T X
+    __syncthreads();
+    const double r = mine ? (i == j ? 1.0 : 0.0) - A[1][i][j] : 0.0;
+    if (mine) A[0][i][j] = 0.5 * r;
+    if (!__syncthreads_or(fabs(r) > 1e-15)) break;
+    eig_product<false>(V[0], A[0], V[1], l);
+    const int again = __syncthreads_or(fabs(r) > 1e-9);
+    if (mine) V[0][i][j] += V[1][i][j];
+    __syncthreads();
+    if (!again) break;
+  }
   if (usable) {
     eig_product<false>(sc.r.B, V[0], A[1], l);
     __syncthreads();
@@ -1319,9 +1335,9 @@ __global__ void __launch_bounds__(kEigThreads) k_ritz_jacobi(const ProblemDev* t
   }
   int cur = 0;
   __syncthreads();
-  // off-diagonal norm within 1e-14 of the whole: done, usually before the first sweep
+  // off-diagonal norm within 1e-15 of the whole: done, usually before the first sweep
   const int max_sweeps = 30;
-  const double eps = 1e-28;
+  const double eps = 1e-30;
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     {
       // off-diagonal and total squared norms: warp i holds row i
