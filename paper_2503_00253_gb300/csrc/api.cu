@@ -223,6 +223,20 @@ int64_t next_pow2(int64_t v) {
   return p;
 }
 
+// Where the transposed Ritz vectors and the BF16 path's second direction
+// buffer lie (carve_problem): in Om and Yb, else in st_W; after them in st_W, else in
+// the optional part of the workspace (build_table).
+size_t phit_bytes(const ProblemDev& pr) {
+  return (size_t)2 * pr.kR * (pr.precision == 2 ? pr.d_pad : pr.d) * (pr.precision == 0 ? 8 : 4);
+}
+bool phit_in_basis(const ProblemDev& pr) {
+  return phit_bytes(pr) <= 2 * align_up((size_t)pr.d * pr.l * (pr.precision == 0 ? 8 : 4));
+}
+size_t phit_in_st(const ProblemDev& pr) { return phit_in_basis(pr) ? 0 : align_up(phit_bytes(pr)); }
+bool pdir1_in_st(const ProblemDev& pr) {
+  return phit_in_st(pr) + (size_t)pr.nsys * pr.d_pad * 2 <= (size_t)3 * pr.d_pad * kStK * 2;
+}
+
 void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
   const size_t esz = o.precision == 0 ? 8 : 4;
   const int64_t n = pr.n, N = pr.N, d = pr.d;
@@ -233,8 +247,9 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
   pr.W = cv.take<void>(d * N * esz);
   pr.rinv = cv.take<double>(d * 8);
   pr.bmean = cv.take<double>(d * 8);
-  pr.scal = cv.take<double>(8 * 8);
-  pr.status = cv.take<int32_t>(4 * 4);
+  char* words = cv.take<char>(8 * 8 + 4 * 4);
+  pr.scal = reinterpret_cast<double*>(words);
+  pr.status = words ? reinterpret_cast<int32_t*>(words + 8 * 8) : nullptr;
   pr.s = cv.take<double>((size_t)std::max(pr.Q, 1) * 8);
   pr.p = cv.take<double>((size_t)std::max(pr.Q, 1) * 8);
   pr.oo_val = cv.take<void>((size_t)pr.max_oo * d * esz);
@@ -247,8 +262,7 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
   char* om = cv.take<char>(2 * basis);
   pr.Om = om;
   pr.Yb = om ? om + basis : nullptr;
-  const size_t phit = (size_t)2 * k * (o.precision == 2 ? pr.d_pad : d) * esz;
-  pr.phiT = phit <= 2 * basis ? om : cv.take<void>(phit);
+  pr.phiT = phit_in_basis(pr) ? om : nullptr;
   pr.Gm = cv.take<double>((size_t)l * l * 8);
   pr.Rm = cv.take<double>((size_t)l * l * 8);
   pr.ev = cv.take<double>((size_t)l * 8);
@@ -311,8 +325,12 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
     pr.alist = cv.take<int32_t>((size_t)3 * J * 4);
     // operand planes of the tensor-core state update (tile_state.cu)
     pr.st_NV = (int32_t)((N + 15) / 16 * 16);
-    pr.st_W = cv.take<__nv_bfloat16>((size_t)3 * dp * kStK * 2);
-    pr.Pdir1 = J <= 3 * kStK ? pr.st_W : cv.take<__nv_bfloat16>((size_t)J * dp * 2);   // the finish fills st_W anew
+    // st_W is filled for the set-up and again for the finish: between them it
+    // holds what only the PCG needs, where that fits
+    char* w = cv.take<char>((size_t)3 * dp * kStK * 2);
+    pr.st_W = reinterpret_cast<__nv_bfloat16*>(w);
+    if (!phit_in_basis(pr)) pr.phiT = w;
+    pr.Pdir1 = w && pdir1_in_st(pr) ? reinterpret_cast<__nv_bfloat16*>(w + phit_in_st(pr)) : nullptr;
     pr.st_V = cv.take<__nv_bfloat16>((size_t)2 * pr.st_NV * dp * 2);
     pr.st_vm = cv.take<float>((size_t)dp * 4);
     pr.st_xyz = cv.take<int4>((size_t)dp * 16);
@@ -328,8 +346,8 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
 }
 
 // Workspace up to which info_esrf_analysis_noalloc serves a call.  The optional
-// quads of C are left out of a reported size that they alone would push past
-// it, and out of any workspace that they don't fit.
+// parts (build_table) are left out of a reported size that they alone would push
+// past it, and out of any workspace that they don't fit.
 constexpr size_t kNoallocBytes = size_t(32) << 20;
 
 // Builds the host table for a batch; with ws == nullptr only sizes it.
@@ -433,22 +451,35 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
   tab.total_sys = sys_base;
   tab.solver = o.solver;
   const size_t sb = o.solver == INFO_ESRF_SOLVER_PCG ? pcg_scratch_bytes(tab, num_sms) : 0;
+  const size_t sat = cv.off;
   void* scratch = cv.take<void>(sb);
+  const size_t sroom = cv.off - sat;
   if (o.solver == INFO_ESRF_SOLVER_MULTISHIFT) {
     if (mscg_plan(tab, num_sms, o.cluster_size, &tab.ms) != 0) return INFO_ESRF_ERR_UNSUPPORTED;
     tab.ms_scratch = tab.ms.scratch_bytes ? cv.take<void>(tab.ms.scratch_bytes) : nullptr;
   }
-  // the quads of C, last
+  // Optional parts, last.  FP32: the quads of C.  BF16: a second direction
+  // buffer for the problems whose st_W has no room for it.  The problems are
+  // solved one after another, so one buffer serves all; it begins with the scratch
+  // of the general PCG kernel, which this path does not run.
   const size_t base = cv.off;
   if (least_out) *least_out = base;
-  size_t quads = 0;
+  size_t extra = 0, second = 0;
   int64_t qcap[kMaxProblems];
   for (int i = 0; i < count; ++i) {
-    const int64_t nb = (tab.p[i].d + 3) / 4;
-    qcap[i] = pcg_quad_cap(tab.p[i], count, o.solver, o.cluster_size);
-    if (qcap[i]) quads += align_up(qcap[i] * nb * 16) + align_up(qcap[i] * nb * 4) + align_up(nb * 4);
+    const ProblemDev& pr = tab.p[i];
+    const int64_t nb = (pr.d + 3) / 4;
+    qcap[i] = pcg_quad_cap(pr, count, o.solver, o.cluster_size);
+    if (qcap[i]) extra += align_up(qcap[i] * nb * 16) + align_up(qcap[i] * nb * 4) + align_up(nb * 4);
+    if (o.precision == 2 && !pdir1_in_st(pr)) second = std::max(second, (size_t)pr.nsys * pr.d_pad * 2);
   }
-  if (ws ? base + quads <= ws_bytes : (base > kNoallocBytes || base + quads <= kNoallocBytes))
+  if (second > sroom) extra = align_up(second) - sroom;
+  const bool taken = ws ? base + extra <= ws_bytes : (base > kNoallocBytes || base + extra <= kNoallocBytes);
+  if (taken && o.precision == 2) {
+    if (extra) cv.take<char>(extra);
+    for (int i = 0; i < count; ++i)
+      if (ws && !tab.p[i].Pdir1) tab.p[i].Pdir1 = reinterpret_cast<__nv_bfloat16*>(scratch);
+  } else if (taken) {
     for (int i = 0; i < count; ++i) {
       ProblemDev& pr = tab.p[i];
       const int64_t nb = (pr.d + 3) / 4;
@@ -458,6 +489,7 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
       pr.qcol = cv.take<int32_t>(pr.qcap * nb * 4);
       pr.qn = cv.take<int32_t>(nb * 4);
     }
+  }
   *bytes_out = cv.off;
   if (dtab_out) *dtab_out = dtab;
   if (counter_out) *counter_out = counter;

@@ -169,7 +169,7 @@ struct ProblemDev {
   void* CPhi;           // [d][kR] T C Phi
   double* theta;        // [kR] Ritz values of C
   void* phiT;           // [2 kR][d] T Phi and C Phi transposed (BF16 path: rows of d_pad), in the memory of
-                        // Om and Yb where it fits: made after the eigensolver is done with them
+                        // Om and Yb, or of st_W: made after the eigensolver and the set-up are done with them
   double* gram;         // [3][kR][kR]: Phi^T Phi, A^T Phi, A^T A with A = C Phi
   // C by quads of rows for the general kernel's FP32 matvec, or NULL (see k_pcg_quads)
   float* qval;                  // [qcap][ceil(d / 4)][4]
@@ -217,8 +217,12 @@ struct ProblemDev {
   float* rinvp;                 // [d_pad] R^-1/2 in tile order (0 at padding)
   // BF16 PCG state: systems j = sid (mean first, then q * N + i), J = nsys
   __nv_bfloat16* Pdir;          // [J][d_pad] search directions by position (bf16, as used), even iterations
-  __nv_bfloat16* Pdir1;         // [J][d_pad] of odd iterations; in the memory of st_W where it fits
-  __host__ __device__ __nv_bfloat16* Pcur(int it) const { return (it & 1) ? Pdir1 : Pdir; }
+  __nv_bfloat16* Pdir1;         // [J][d_pad] of odd iterations, or NULL: Pdir holds all of them, and the next
+                                // directions are formed in the memory of Yv and copied
+  __host__ __device__ __nv_bfloat16* Pcur(int it) const { return (it & 1) && Pdir1 ? Pdir1 : Pdir; }
+  __host__ __device__ __nv_bfloat16* Pnext(int it) const {
+    return Pdir1 ? Pcur(it + 1) : reinterpret_cast<__nv_bfloat16*>(Yv);
+  }
   float* Yv;                    // [J][d_pad] sigma p + C p by position
   float* Xv;                    // [J][d_pad] iterates
   float* Rv;                    // [J][d_pad] residuals
@@ -347,7 +351,7 @@ int launch_mscg(const ProblemTable& tab, const ProblemDev* dtab, const MsPlan& p
 // Work counters of the PCG stage: [0] group queue of the general kernel,
 // [1 + i] system queue of the band kernel for problem i, [1 + kMaxProblems + i]
 // its fall-back flag.
-constexpr int kCounterInts = 256;
+constexpr int kCounterInts = 192;
 static_assert(1 + 2 * kMaxProblems <= kCounterInts, "PCG counter area");
 
 int64_t pcg_quad_cap(const ProblemDev& p, int count, int32_t solver, int32_t cluster_size);
