@@ -27,7 +27,13 @@
  *   - R_diag [d]: observation-error variances, > 0.
  *   - workspace: caller-allocated device memory of info_esrf_workspace_size()
  *     bytes, 256-byte aligned.  The library keeps no pointer after return
- *     and allocates nothing.
+ *     and allocates nothing.  The size includes parts that only make a call
+ *     faster: FP32 PCG on the general kernel keeps C a second time by blocks of
+ *     four rows (at most 128 MiB a problem; 64 problems up to 8 GiB), BF16 a
+ *     second direction buffer (2 bytes per system and padded observation, of
+ *     the largest problem).  They are left out of a size that they alone would
+ *     push past 32 MiB, and a call runs without them in a smaller workspace; FP32
+ *     results then differ by rounding, and by nothing in any larger one.
  *   - stream: a cudaStream_t passed as void*; NULL is the legacy stream.  All
  *     work is stream-ordered.  If stats is NULL the call returns as soon as
  *     the work is queued; otherwise it waits for the stream and fills stats,

@@ -345,11 +345,6 @@ void carve_problem(Carver& cv, ProblemDev& pr, const info_esrf_options& o) {
   }
 }
 
-// Workspace up to which info_esrf_analysis_noalloc serves a call.  The optional
-// parts (build_table) are left out of a reported size that they alone would push
-// past it, and out of any workspace that they don't fit.
-constexpr size_t kNoallocBytes = size_t(32) << 20;
-
 // Builds the host table for a batch; with ws == nullptr only sizes it.
 // *bytes_out is the size with the optional parts, *least_out the size that a call needs.
 int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_options& o, void* ws,
@@ -474,7 +469,12 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
     if (o.precision == 2 && !pdir1_in_st(pr)) second = std::max(second, (size_t)pr.nsys * pr.d_pad * 2);
   }
   if (second > sroom) extra = align_up(second) - sroom;
-  const bool taken = ws ? base + extra <= ws_bytes : (base > kNoallocBytes || base + extra <= kNoallocBytes);
+  // Left out of a size that they alone would push past what the allocation-free
+  // entry point serves, and of a workspace that they don't fit.  The quads change the
+  // order of the matvec's sums, so the first rule holds for larger workspaces too: the
+  // bits depend on the problem, except in a workspace below the reported size.
+  const bool within = base > kNoallocBytes || base + extra <= kNoallocBytes;
+  const bool taken = ws ? base + extra <= ws_bytes && (within || o.precision == 2) : within;
   if (taken && o.precision == 2) {
     if (extra) cv.take<char>(extra);
     for (int i = 0; i < count; ++i)

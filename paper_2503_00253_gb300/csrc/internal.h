@@ -328,6 +328,9 @@ struct AuxStream {
 };
 AuxStream* aux_stream();
 
+// Workspace up to which info_esrf_analysis_noalloc serves a call (the documented maximum).
+constexpr size_t kNoallocBytes = size_t(32) << 20;
+
 // Host-side count of kernel launches issued by this library.
 void note_launches(int n);
 

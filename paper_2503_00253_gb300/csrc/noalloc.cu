@@ -8,7 +8,7 @@
 // carves it from a fixed array that is part of the library image.
 //
 // The array is a file-scope __device__ variable: every GPU on which the
-// library is loaded holds kNoAllocBytes of it until the process exits.  Host
+// library is loaded holds kNoallocBytes of it until the process exits.  Host
 // code cannot use the symbol itself as a device address, so each call asks
 // the runtime for the array's device address in the calling thread's current
 // context (cudaGetSymbolAddress).  That address belongs to the context's
@@ -24,13 +24,15 @@
 
 #include "info_esrf.h"
 #include "info_esrf_stages.h"
+#include "internal.h"
+
+using infoesrf::kNoallocBytes;
 
 namespace {
 
-constexpr size_t kNoAllocBytes = (size_t)32 << 20;   // 32 MiB, the documented maximum
 constexpr int kMaxContexts = 64;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
 using CtxGetCurrentFn = CUresult (*)(CUcontext*);
 
@@ -119,10 +121,10 @@ extern "C" int info_esrf_analysis_noalloc(const info_esrf_grid* grid, int64_t N,
   // need == 0: the arguments or options are invalid or unsupported; the
   // regular entry point validates them before any kernel touches the array
   // and returns the same code it would for a caller's workspace
-  if (need > kNoAllocBytes) return INFO_ESRF_ERR_UNSUPPORTED;
+  if (need > kNoallocBytes) return INFO_ESRF_ERR_UNSUPPORTED;
   // Every scratch word the analysis reads is written earlier in the same
   // call (tables, counters and accumulators are reset by its own kernels), so
   // the previous call's leftovers need no clearing.
-  return info_esrf_analysis(grid, N, X_dev, d, obs_idx_dev, y_dev, R_diag_dev, Q, tol, opt, ws, kNoAllocBytes,
+  return info_esrf_analysis(grid, N, X_dev, d, obs_idx_dev, y_dev, R_diag_dev, Q, tol, opt, ws, kNoallocBytes,
                             stream, mu_a_dev, A_a_dev, nullptr);
 }
