@@ -29,7 +29,8 @@
  *     bytes, 256-byte aligned.  The library keeps no pointer after return
  *     and allocates nothing.  The size includes parts that only make a call
  *     faster: FP32 PCG on the general kernel keeps C a second time by blocks of
- *     four rows (at most 128 MiB a problem; 64 problems up to 8 GiB), BF16 a
+ *     four rows (at most 128 MiB a problem; 64 problems up to 8 GiB) and, above
+ *     rank 12 and 4298 observations, the vectors of one CTA in 17; BF16 a
  *     second direction buffer (2 bytes per system and padded observation, of
  *     the largest problem).  They are left out of a size that they alone would
  *     push past 32 MiB, and a call runs without them in a smaller workspace; FP32

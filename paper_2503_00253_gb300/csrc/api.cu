@@ -445,7 +445,8 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
   tab.total_groups = group_base;
   tab.total_sys = sys_base;
   tab.solver = o.solver;
-  const size_t sb = o.solver == INFO_ESRF_SOLVER_PCG ? pcg_scratch_bytes(tab, num_sms) : 0;
+  const size_t sfull = o.solver == INFO_ESRF_SOLVER_PCG ? pcg_scratch_bytes(tab, num_sms) : 0;
+  size_t sb = o.solver == INFO_ESRF_SOLVER_PCG ? pcg_scratch_least(tab, num_sms) : 0;
   const size_t sat = cv.off;
   void* scratch = cv.take<void>(sb);
   const size_t sroom = cv.off - sat;
@@ -453,7 +454,8 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
     if (mscg_plan(tab, num_sms, o.cluster_size, &tab.ms) != 0) return INFO_ESRF_ERR_UNSUPPORTED;
     tab.ms_scratch = tab.ms.scratch_bytes ? cv.take<void>(tab.ms.scratch_bytes) : nullptr;
   }
-  // Optional parts, last.  FP32: the quads of C.  BF16: a second direction
+  // Optional parts, last.  FP32: the rest of the general PCG kernel's scratch
+  // (behind it, so in one piece), and the quads of C.  BF16: a second direction
   // buffer for the problems whose st_W has no room for it.  The problems are
   // solved one after another, so one buffer serves all; it begins with the scratch
   // of the general PCG kernel, which this path does not run.
@@ -468,7 +470,9 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
     if (qcap[i]) extra += align_up(qcap[i] * nb * 16) + align_up(qcap[i] * nb * 4) + align_up(nb * 4);
     if (o.precision == 2 && !pdir1_in_st(pr)) second = std::max(second, (size_t)pr.nsys * pr.d_pad * 2);
   }
-  if (second > sroom) extra = align_up(second) - sroom;
+  const size_t rest = o.precision == 1 && sfull > sroom ? align_up(sfull) - sroom : 0;
+  if (o.precision == 2) extra = second > sroom ? align_up(second) - sroom : 0;
+  else extra += rest;
   // Left out of a size that they alone would push past what the allocation-free
   // entry point serves, and of a workspace that they don't fit.  The quads change the
   // order of the matvec's sums, so the first rule holds for larger workspaces too: the
@@ -480,6 +484,10 @@ int build_table(const info_esrf_problem* probs, int32_t count, const info_esrf_o
     for (int i = 0; i < count; ++i)
       if (ws && !tab.p[i].Pdir1) tab.p[i].Pdir1 = reinterpret_cast<__nv_bfloat16*>(scratch);
   } else if (taken) {
+    if (rest) {
+      cv.take<char>(rest);
+      sb = sfull;
+    }
     for (int i = 0; i < count; ++i) {
       ProblemDev& pr = tab.p[i];
       const int64_t nb = (pr.d + 3) / 4;

@@ -363,6 +363,7 @@ void launch_pcg_quads(const ProblemTable& tab, const ProblemDev* dtab, cudaStrea
 
 // PCG vector scratch per CTA when vectors do not fit in shared memory.
 size_t pcg_scratch_bytes(const ProblemTable& tab, int num_sms);
+size_t pcg_scratch_least(const ProblemTable& tab, int num_sms);
 int pcg_jt(int precision, int64_t systems, int num_sms);
 
 }  // namespace infoesrf

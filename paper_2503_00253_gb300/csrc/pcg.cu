@@ -799,6 +799,24 @@ size_t pcg_scratch_bytes(const ProblemTable& tab, int num_sms) {
   return slice_elems(tab) * (tab.p[0].precision == 0 ? 8 : 4) * (size_t)num_sms;   // one CTA per SM
 }
 
+// What a call must have of it.  The vectors of level 2 take 136 bytes a row in
+// FP32 (with the padding of p); a call asks for no more than 128 bytes a row and SM,
+// twice that up to rank 12, which is at least 16 CTAs of 17.  (BF16 only keeps
+// directions here, see build_table.)
+size_t pcg_scratch_least(const ProblemTable& tab, int num_sms) {
+  const size_t full = pcg_scratch_bytes(tab, num_sms);
+  const int precision = tab.p[0].precision;
+  if (precision == 0) return full;
+  int64_t dmax = 0, kmax = 0;
+  for (int i = 0; i < tab.count; ++i) {
+    dmax = std::max<int64_t>(dmax, tab.p[i].d);
+    kmax = std::max<int64_t>(kmax, tab.p[i].kR);
+  }
+  const size_t slice = slice_elems(tab) * sizeof(float);
+  const size_t room = (size_t)128 * dmax * num_sms * (precision == 1 && kmax <= 12 ? 2 : 1);
+  return full <= room ? full : room / slice * slice;
+}
+
 template <typename T, int KMAX>
 static int launch_pcg_t(const ProblemTable& tab, const ProblemDev* dtab, int32_t* counter, void* scratch,
                         size_t scratch_bytes, int num_sms, cudaStream_t st, uint64_t band_mask,

@@ -55,6 +55,12 @@ def test_calls_need_no_more_than_they_did(form, served):
     assert 0 < B.library().info_esrf_batched_workspace_size(arr, count, ctypes.byref(o)) <= served
 
 
+def test_bf16_calls_of_many_observations_need_no_more_than_they_did():
+    from paper_2503_00253_gb300 import binding as B
+    o = B.make_options(precision=2, ritz_rank=24, oversample=8)
+    assert 0 < B.workspace_size(grid_of((96, 64, 5.0)), 16, 5000, 2, o) <= 172_187_392
+
+
 def dev(a):
     return torch.tensor(np.ascontiguousarray(a), device="cuda")
 
@@ -102,3 +108,20 @@ def test_one_direction_buffer_gives_the_same_bits(shape, d, N, Q, max_iter):
     one = B.info_esrf_analysis(*args, o, ws=B.workspace(size - 256))
     assert two[2]["status"] == one[2]["status"] and two[2]["iters_max"] == one[2]["iters_max"]
     assert torch.equal(two[0], one[0]) and torch.equal(two[1], one[1])
+
+
+@pytest.mark.gpu
+def test_fp32_vectors_beyond_shared_memory_run_in_the_scratch_they_had():
+    """136 bytes a row and SM are asked for, 128 are enough (the optional last CTAs of 152 are left out); no
+    blocks of rows at this size, so the bits are the same."""
+    from paper_2503_00253_gb300 import binding as B
+    d = 33000
+    pr = workloads.gaussian_problem_1d("scratch", n=2 * d, N=3, length_scale=3.0, obs_stride=2, r2=0.5, half_width=3.0,
+                                       Q=2, tol=1e-6, seed=3)
+    args = [pr.grid, dev(pr.X), dev(pr.obs_idx), dev(pr.y), dev(pr.R), pr.Q, pr.tol]
+    o = B.make_options(precision=1, ritz_rank=24, oversample=8, cluster_size=-1)
+    size = B.workspace_size(pr.grid, pr.N, pr.d, pr.Q, o)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    full, served = (B.info_esrf_analysis(*args, o, ws=B.workspace(n)) for n in (size, size - 7 * d * sms))
+    assert full[2]["status"] == 0 and full[2]["solver_path"] == 0
+    assert torch.equal(full[0], served[0]) and torch.equal(full[1], served[1])
