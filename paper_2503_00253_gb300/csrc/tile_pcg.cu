@@ -226,7 +226,7 @@ struct VecStep {
 
 template <int NV32, int SPT>
 __global__ void __launch_bounds__(kUpdThreads) k_tpcg_update(const ProblemDev* dpr, int update, const int32_t* list,
-                                                             int it) {
+                                                             const __nv_bfloat16* P, int it) {
   grid_dependency_wait();
   constexpr int kSys = kUpdSlots * SPT;
   extern __shared__ float4 phs_dyn4[];   // [2 k][kDotRows / 4]
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_tpcg_update(const ProblemDev* d
       if (update) {
         w[u].y = *reinterpret_cast<const float4*>(pr.Yv + pbase[u] + r4);
         w[u].x = *reinterpret_cast<const float4*>(pr.Xv + base[u] + r4);
-        w[u].p = *reinterpret_cast<const uint2*>(pr.Pcur(it) + pbase[u] + r4);
+        w[u].p = *reinterpret_cast<const uint2*>(P + pbase[u] + r4);
       }
     }
   };
@@ -514,7 +514,8 @@ __global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev*
 // learned != 0: a learned system takes z = a (r - (C Phi) t + Phi c) + S u.
 template <int K, int RPL>
 __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev* dpr, const int32_t* list,
-                                                                const int32_t* src, int group, int learned, int it) {
+                                                                const int32_t* src, const __nv_bfloat16* Pold,
+                                                                __nv_bfloat16* Pnew, int group, int learned, int it) {
   constexpr int kBatch = 4;
   grid_dependency_wait();
   const ProblemDev& pr = *dpr;
@@ -555,8 +556,6 @@ __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev
     }
     tcf[e] = v;
   }
-  const __nv_bfloat16* Pold = pr.Pcur(it);
-  __nv_bfloat16* Pnew = pr.Pnext(it);
   const int64_t chunk = (int64_t)blockIdx.x * kVecWarps + warp;
   const bool mine = chunk < dp / (32 * RPL);
   const int64_t a = chunk * 32 * RPL + lane * RPL;
@@ -719,19 +718,22 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
   auto update = [&](int mode, const int32_t* list, int64_t count, int it) {
     // two systems per thread (half the reads of [Phi | C Phi]) once that still
     // gives every SM two CTAs; 64 dot values (k > 15) leave registers for one
+    const __nv_bfloat16* P = p.Pcur(it);
     const int spt = p.kR <= 15 && nsub * count >= 32 * (int64_t)sms ? 2 : 1;
     const dim3 grid((unsigned)nsub, (unsigned)((count + kUpdSlots * spt - 1) / (kUpdSlots * spt)));
-    if (p.kR > 15) launch_overlapped(k_tpcg_update<2, 1>, grid, kUpdThreads, usm, st, dp, mode, list, it);
-    else if (spt == 2) launch_overlapped(k_tpcg_update<1, 2>, grid, kUpdThreads, usm, st, dp, mode, list, it);
-    else launch_overlapped(k_tpcg_update<1, 1>, grid, kUpdThreads, usm, st, dp, mode, list, it);
+    if (p.kR > 15) launch_overlapped(k_tpcg_update<2, 1>, grid, kUpdThreads, usm, st, dp, mode, list, P, it);
+    else if (spt == 2) launch_overlapped(k_tpcg_update<1, 2>, grid, kUpdThreads, usm, st, dp, mode, list, P, it);
+    else launch_overlapped(k_tpcg_update<1, 1>, grid, kUpdThreads, usm, st, dp, mode, list, P, it);
   };
   auto direction = [&](const int32_t* list, int64_t count, int it) {
     const int group = dir_group(dchunks, count, sms);
     const dim3 grid((unsigned)((dchunks + kVecWarps - 1) / kVecWarps), (unsigned)((count + group - 1) / group));
     const int32_t* from = srcs;
+    const __nv_bfloat16* Pold = p.Pcur(it);
+    __nv_bfloat16* Pnew = p.Pnext(it);
     const int lrn = learned ? 1 : 0;
-    if (wide) launch_overlapped(k_tpcg_direction<24, 2>, grid, kVecThreads, 0, st, dp, list, from, group, lrn, it);
-    else launch_overlapped(k_tpcg_direction<12, 2>, grid, kVecThreads, 0, st, dp, list, from, group, lrn, it);
+    auto kernel = wide ? k_tpcg_direction<24, 2> : k_tpcg_direction<12, 2>;
+    launch_overlapped(kernel, grid, kVecThreads, 0, st, dp, list, from, Pold, Pnew, group, lrn, it);
     // one direction buffer: y, where they were formed, is free until the next matvec (3.34 ms
     // for 3.13 at 961 systems x 960 observations, the same bits)
     if (!p.Pdir1)
