@@ -238,8 +238,9 @@ __global__ void __launch_bounds__(kUpdThreads) k_tpcg_update(const ProblemDev* d
   const int64_t dp = pr.d_pad;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t count = list_count(pr, list, it);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) pr.nactive[(it + 2) % 3] = 0;
-  const int64_t g0 = (int64_t)blockIdx.y * kSys;
+  const int64_t group = (int64_t)blockIdx.z * gridDim.y + blockIdx.y;
+  if (blockIdx.x == 0 && group == 0 && threadIdx.x == 0) pr.nactive[(it + 2) % 3] = 0;
+  const int64_t g0 = group * kSys;
   if (g0 >= count) return;
   const int64_t abase = (int64_t)blockIdx.x * kDotRows;
   const int nrow = (int)(dp - abase < kDotRows ? dp - abase : kDotRows);   // a multiple of 128
@@ -720,7 +721,8 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
     // gives every SM two CTAs; 64 dot values (k > 15) leave registers for one
     const __nv_bfloat16* P = p.Pcur(it);
     const int spt = p.kR <= 15 && nsub * count >= 32 * (int64_t)sms ? 2 : 1;
-    const dim3 grid((unsigned)nsub, (unsigned)((count + kUpdSlots * spt - 1) / (kUpdSlots * spt)));
+    const int64_t groups = (count + kUpdSlots * spt - 1) / (kUpdSlots * spt), layers = (groups + 65534) / 65535;
+    const dim3 grid((unsigned)nsub, (unsigned)((groups + layers - 1) / layers), (unsigned)layers);
     if (p.kR > 15) launch_overlapped(k_tpcg_update<2, 1>, grid, kUpdThreads, usm, st, dp, mode, list, P, it);
     else if (spt == 2) launch_overlapped(k_tpcg_update<1, 2>, grid, kUpdThreads, usm, st, dp, mode, list, P, it);
     else launch_overlapped(k_tpcg_update<1, 1>, grid, kUpdThreads, usm, st, dp, mode, list, P, it);
