@@ -106,7 +106,7 @@ int run_tile_pcg_capture(const ProblemDev& p, const ProblemDev* dp, const TileCa
 void launch_tile_learn_u(const ProblemDev& p, const ProblemDev* dp, const int32_t* list, int64_t count, int nsub,
                          int it, cudaStream_t st);
 void launch_tile_capture_record(const ProblemDev& p, const ProblemDev* dp, const TileCapture& cap, int it,
-                                const int32_t* list, int64_t count, cudaStream_t st);
+                                const int32_t* list, cudaStream_t st);
 void launch_tile_capture_finish(const ProblemDev& p, const ProblemDev* dp, const TileCapture& cap, float* Z,
                                 float* feat, cudaStream_t st);
 

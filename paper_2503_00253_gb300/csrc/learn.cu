@@ -816,10 +816,10 @@ int info_esrf_learn_loss_grad(const float* theta_dev, int32_t nsamp, int64_t d, 
   const size_t need = (size_t)nsamp * kLearnParams * sizeof(float) + (size_t)nsamp * sizeof(double);
   if (!scratch_dev || scratch_bytes < need || (reinterpret_cast<uintptr_t>(scratch_dev) % 16) != 0)
     return INFO_ESRF_ERR_WORKSPACE;
-  const size_t dyn = (size_t)6 * d * sizeof(float);
-  if (dyn > 200 * 1024) return INFO_ESRF_ERR_UNSUPPORTED;
+  // the limit that the entry point has had (d <= 8192 documented); the kernel's rows would allow more
+  if ((size_t)6 * d * sizeof(float) > 200 * 1024) return INFO_ESRF_ERR_UNSUPPORTED;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  float* rec = reinterpret_cast<float*>(scratch_dev);
+  float* rec = reinterpret_cast<float*>(scratch_dev);   // kRec floats a sample of the kLearnParams asked for
   double* sl = reinterpret_cast<double*>(rec + (size_t)nsamp * kLearnParams);
   cudaGetLastError();
   int dev = 0, sms = 0;

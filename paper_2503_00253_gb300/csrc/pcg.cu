@@ -773,10 +773,16 @@ void launch_pcg_phit(const ProblemTable& tab, const ProblemDev* dtab, cudaStream
 // to its end, so the hardest group's iterations bound the call from below.
 // FP64, whose pipe is the bound: groups of one halve that time where groups of
 // two leave CTAs without work (100 weighted sums, 161 systems: 1.30 -> 1.12
-// ms; at 321 systems, more groups of two than CTAs, 0.57 -> 0.61).  FP32: half
-// a group's iteration costs almost what a whole one does (layered 961 systems 7.0 -> 7.3 ms).
+// ms; at 321 systems, more groups of two than CTAs, 0.57 -> 0.61).  The line is
+// where groups of two would have a CTA each.  One problem of 60 observations:
+// groups of one take 0.53 ms from 141 to 241 systems and 0.58 at 301, groups of
+// two 0.56 at 321; of 500 observations, 1.49 ms at 141 to 301 against 1.93 at 321.
+// FP32: half a group's iteration costs almost what a whole one does (layered
+// 961 systems 7.0 -> 7.3 ms).
 // The rule looks at the problem alone, and so a batched call solves it in the
-// same way as a call of its own.
+// same way, with the same bits, as a call of its own.  A batch that fills the chip
+// anyway pays for that: 64 problems of 250 observations take 35.8 ms with 301
+// systems each (groups of one) and 27.8 ms with 321.
 int pcg_jt(int precision, int64_t systems, int num_sms) {
   if (precision != 0) return kJTWide<float>;
   return (systems + 1) / 2 <= num_sms ? kJTNarrow<double> : kJTWide<double>;

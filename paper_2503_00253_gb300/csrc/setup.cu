@@ -992,7 +992,8 @@ constexpr int kOrthThreads = kMaxRitz * kMaxRitz;   // one thread per entry of G
 // (1024 entries: 20 us a launch at 60 to 100 rows, 14 us now); every block repeats
 // the factorization.
 static int orth_entries(int64_t total) {
-  return (int)std::min<int64_t>(std::max<int64_t>((total / 152 + 127) / 128 * 128, 128), kOrthThreads);
+  constexpr int kSms = 152;   // of a GB300; any other count only changes the split
+  return (int)std::min<int64_t>(std::max<int64_t>((total / kSms + 127) / 128 * 128, 128), kOrthThreads);
 }
 __global__ void __launch_bounds__(kOrthThreads) k_ritz_orth64(const ProblemDev* tab, int src, int entries) {
   const ProblemDev& pr = tab[blockIdx.y];

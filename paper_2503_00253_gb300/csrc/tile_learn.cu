@@ -366,8 +366,7 @@ void launch_tile_learn_u(const ProblemDev& p, const ProblemDev* dp, const int32_
 }
 
 void launch_tile_capture_record(const ProblemDev& p, const ProblemDev* dp, const TileCapture& cap, int it,
-                                const int32_t* list, int64_t count, cudaStream_t st) {
-  (void)count;
+                                const int32_t* list, cudaStream_t st) {
   const dim3 grid((unsigned)((p.d + 255) / 256), (unsigned)cap.nsel);
   k_tcap_record<<<grid, 256, 0, st>>>(dp, cap.sel, cap.nsel, it, cap.K, list, cap.V, cap.Y);
   note_launches(1);

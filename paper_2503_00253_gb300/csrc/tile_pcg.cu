@@ -7,7 +7,7 @@
 //      (tensor-core block-tile matvec, tile_matvec.cu);
 //   2. alpha_j = rho_j / p_j^T y_j (FP64, partials summed in a fixed order);
 //   3. x_j += alpha_j p_j, r_j -= alpha_j y_j, and partials of r^T r,
-//      f = Phi^T r, g = (C Phi)^T r (FP32 per thread, FP64 across threads);
+//      f = Phi^T r, g = (C Phi)^T r (FP32 over 512 rows, FP64 across row blocks);
 //   4. per system: convergence test ||r|| <= tol ||b||, the preconditioner
 //      coefficients t = T^-1 f, c = (beta_lmp - sigma) t - T^-1 (g + sigma f - G_q t)
 //      with G_q = (C_q Phi)^T (C_q Phi), rho' = r^T z = r^T r - g.t + f.c and
@@ -513,7 +513,8 @@ __global__ void __launch_bounds__(kScalThreads) k_tpcg_scalars(const ProblemDev*
 // shared memory, read per system: 14.4 us a launch at 4096 rows, 52 us at 65,536.)
 // K: columns of Phi held.
 // learned != 0: a learned system takes z = a (r - (C Phi) t + Phi c) + S u.
-template <int K, int RPL>
+constexpr int kDirRows = 2;   // consecutive rows per lane
+template <int K>
 __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev* dpr, const int32_t* list,
                                                                 const int32_t* src, const __nv_bfloat16* Pold,
                                                                 __nv_bfloat16* Pnew, int group, int learned, int it) {
@@ -558,48 +559,37 @@ __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev
     tcf[e] = v;
   }
   const int64_t chunk = (int64_t)blockIdx.x * kVecWarps + warp;
-  const bool mine = chunk < dp / (32 * RPL);
-  const int64_t a = chunk * 32 * RPL + lane * RPL;
-  float c[2 * K][RPL];   // loaded while the coefficients are on their way to shared memory
+  const bool mine = chunk < dp / (32 * kDirRows);
+  const int64_t a = chunk * 32 * kDirRows + lane * kDirRows;
+  float c[2 * K][kDirRows];   // loaded while the coefficients are on their way to shared memory
 #pragma unroll
   for (int m = 0; m < 2 * K; ++m) {
     const int mm = m < K ? m : k + (m - K);
     const bool in = mine && (m < K ? m < k : m - K < k);
 #pragma unroll
-    for (int i = 0; i < RPL; ++i) c[m][i] = 0.f;
+    for (int i = 0; i < kDirRows; ++i) c[m][i] = 0.f;
     if (in) {
-      const float* src = reinterpret_cast<const float*>(pr.phiT) + (int64_t)mm * dp + a;
-      if constexpr (RPL == 4) {
-        const float4 t = ld_settled(reinterpret_cast<const float4*>(src));
-        c[m][0] = t.x; c[m][1] = t.y; c[m][2] = t.z; c[m][3] = t.w;
-      } else {
-        const float2 t = ld_settled(reinterpret_cast<const float2*>(src));
-        c[m][0] = t.x; c[m][1] = t.y;
-      }
+      const float* col = reinterpret_cast<const float*>(pr.phiT) + (int64_t)mm * dp + a;
+      const float2 t = ld_settled(reinterpret_cast<const float2*>(col));
+      c[m][0] = t.x;
+      c[m][1] = t.y;
     }
   }
   __syncthreads();
   if (!mine) return;
 #pragma unroll 1
   for (int s0 = 0; s0 < group; s0 += kBatch) {
-    float z[kBatch][RPL];
-    uint32_t pw[kBatch][RPL / 2];
+    float z[kBatch][kDirRows];
+    uint32_t pw[kBatch];
 #pragma unroll
     for (int b = 0; b < kBatch; ++b) {
       const int j = sys[s0 + b];
       if (j < 0) continue;
       const int64_t e = (int64_t)j * dp + a;
-      if constexpr (RPL == 4) {
-        const float4 r = *reinterpret_cast<const float4*>(pr.Rv + e);
-        z[b][0] = r.x; z[b][1] = r.y; z[b][2] = r.z; z[b][3] = r.w;
-        const uint2 w = *reinterpret_cast<const uint2*>(Pold + from[s0 + b] * dp + a);
-        pw[b][0] = w.x;
-        pw[b][RPL / 2 - 1] = w.y;
-      } else {
-        const float2 r = *reinterpret_cast<const float2*>(pr.Rv + e);
-        z[b][0] = r.x; z[b][1] = r.y;
-        pw[b][0] = *reinterpret_cast<const uint32_t*>(Pold + from[s0 + b] * dp + a);
-      }
+      const float2 r = *reinterpret_cast<const float2*>(pr.Rv + e);
+      z[b][0] = r.x;
+      z[b][1] = r.y;
+      pw[b] = *reinterpret_cast<const uint32_t*>(Pold + from[s0 + b] * dp + a);
     }
 #pragma unroll
     for (int b = 0; b < kBatch; ++b) {
@@ -612,12 +602,11 @@ __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-          for (int i = 0; i < RPL; ++i) z[b][i] = fmaf(c[4 * q + u][i], cq[u], z[b][i]);
+          for (int i = 0; i < kDirRows; ++i) z[b][i] = fmaf(c[4 * q + u][i], cq[u], z[b][i]);
       }
       const float be = bes[s], la = las[s];
-      __nv_bfloat162 out[RPL / 2];
 #pragma unroll
-      for (int i = 0; i < RPL; ++i) {
+      for (int i = 0; i < kDirRows; ++i) {
         if (la > 0.f) {   // z = a P^-1 r + S u
           const int32_t* nb = pr.lat_nbr + (a + i) * kLatPts;
           const float* u = pr.learn_u + (int64_t)j * dp;
@@ -626,16 +615,12 @@ __global__ void __launch_bounds__(kVecThreads) k_tpcg_direction(const ProblemDev
           for (int n = 0; n < kLatPts; ++n) su = fmaf(ltap[s][lat_bin(n)], ld_settled(u + nb[n]), su);
           z[b][i] = fmaf(la, z[b][i], su);
         }
-        const uint32_t w = pw[b][i / 2];
+        const uint32_t w = pw[b];
         const float p = __uint_as_float((i & 1) ? (w & 0xffff0000u) : (w << 16));
         // beta = 0 (a first direction): the old position holds nothing of this system
         z[b][i] = a + i < pr.d ? (be != 0.f ? fmaf(be, p, z[b][i]) : z[b][i]) : 0.f;
       }
-#pragma unroll
-      for (int i = 0; i < RPL / 2; ++i) out[i] = __floats2bfloat162_rn(z[b][2 * i], z[b][2 * i + 1]);
-      __nv_bfloat16* dst = Pnew + (g0 + s) * dp + a;
-      if constexpr (RPL == 4) *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(out);
-      else *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(out);
+      *reinterpret_cast<__nv_bfloat162*>(Pnew + (g0 + s) * dp + a) = __floats2bfloat162_rn(z[b][0], z[b][1]);
     }
   }
 }
@@ -734,7 +719,7 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
     const __nv_bfloat16* Pold = p.Pcur(it);
     __nv_bfloat16* Pnew = p.Pnext(it);
     const int lrn = learned ? 1 : 0;
-    auto kernel = wide ? k_tpcg_direction<24, 2> : k_tpcg_direction<12, 2>;
+    auto kernel = wide ? k_tpcg_direction<24> : k_tpcg_direction<12>;
     launch_overlapped(kernel, grid, kVecThreads, 0, st, dp, list, from, Pold, Pnew, group, lrn, it);
     // one direction buffer: y, where they were formed, is free until the next matvec (3.34 ms
     // for 3.13 at 961 systems x 960 observations, the same bits)
@@ -793,7 +778,7 @@ static int tile_pcg_loop(const ProblemDev& p, const ProblemDev* dp, cudaStream_t
       if (mm_ms) cudaEventRecord(ev[it & 1][0], st);
       if (launch_tile_mm(ta, p.Chi, p.Clo, p.tile_cap, st) != 0) return INFO_ESRF_ERR_CUDA;
       if (mm_ms) cudaEventRecord(ev[it & 1][1], st);
-      if (cap) launch_tile_capture_record(p, dp, *cap, it, list, bound, st);
+      if (cap) launch_tile_capture_record(p, dp, *cap, it, list, st);
       if (!fused_alpha) {
         k_tpcg_alpha<<<(unsigned)((32 * bound + 255) / 256), 256, 0, st>>>(dp, it, list);
         note_launches(1);

@@ -39,7 +39,7 @@ def test_no_non_coherent_read_of_what_the_predecessor_writes(file, name, body):
     assert not re.search(r"__ldg\s*\(|\.nc\b", body), (file, name)
     # settled data only: the Ritz vectors (made before the loop) and S r (two launches back)
     for arg in re.findall(r"ld_settled\(([^;]*);", body):
-        assert "src)" in arg or arg.startswith("u + "), (name, arg)
+        assert "col)" in arg or arg.startswith("u + "), (name, arg)
 
 
 @pytest.mark.parametrize("file,name,body", OVERLAPPED, ids=[k[1] for k in OVERLAPPED])
